@@ -31,9 +31,9 @@ def listed():
              dt=1e-3, kappa=0.7, steps=333),
         # coupled Allen-Cahn / Cahn-Hilliard precipitates at the headline size
         dict(name="coupled_2048", kind="coupled", ny=2048, nx=2048, hx=1.0, hy=1.0, steps=200),
-        # parameter study: 256 uneven instances, tuned schedule, one launch per step
+        # parameter study: 256 uneven instances in the default mode, one persistent launch
         dict(name="ensemble_256", kind="ensemble", count=256, lo=128, hi=512, grid=128,
-             mode="per_step", steps=200),
+             mode="persistent", steps=200),
         # calibration: loss and gradients of a 2,000-step trajectory, a mobility per node
         dict(name="misfit_512", kind="misfit", ny=512, nx=512, steps=2000, ckpt=100),
         # small implicit run (100 x 100 domain, 64 x 64 mesh, 6 steps): host round trips count
