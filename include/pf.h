@@ -145,8 +145,13 @@ pf_status pf_step_explicit(pf_ctx* ctx, float* state, int64_t n_steps);
 /* Execution form of the 2-D explicit step (AC and CH without a mobility field;
  * no counterpart in the paper, which has one array program).  All forms
  * compute the same discretisation in FP32 on the shifted state:
- *   PF_FORM_FUSED_GRAPH   one fused kernel per step, replayed from a CUDA graph
- *                         of 64 steps (default)
+ *   PF_FORM_FUSED_GRAPH   the default: all steps in one cooperative launch with
+ *                         the state on chip where the mesh fits (up to about
+ *                         2,100^2 nodes) and the steps pay for it; otherwise one
+ *                         fused kernel per step, replayed from a CUDA graph of
+ *                         64 steps.  Bitwise the same results either way; should
+ *                         a bounded wait between blocks expire, the state is
+ *                         filled with NaN
  *   PF_FORM_FUSED_STREAM  the same kernel, one launch per step from the host
  *   PF_FORM_TWO_PASS      the plain form: node-centric quadrature with index
  *                         reflection, CH's mu written to and read back from
@@ -231,7 +236,8 @@ pf_status pf_adjoint(pf_ctx* ctx, const float* state0, const float* target, int6
 
 /* Ensemble stepping modes for pf_step_ensemble. */
 enum {
-  PF_ENS_PERSISTENT = 0, /* one persistent launch for all steps (graph-captured), grid barrier */
+  PF_ENS_PERSISTENT = 0, /* one persistent launch for all steps: the instances on chip where
+                            each fits, otherwise planes in memory and a grid barrier */
   PF_ENS_PER_STEP = 1,   /* one launch per step covering every instance */
   PF_ENS_PLAIN = 2       /* the single-mesh fused step, one launch per instance and step */
 };
@@ -285,8 +291,8 @@ pf_status pf_tune_ensemble(pf_ctx* ctx, int reps, int* ty_out, int* l2_out, doub
 
 /* Advance every instance of the packed state (device, in/out) by n_steps
  * explicit steps (Eq. 12) in the given mode.  PF_ENS_PERSISTENT synchronises
- * the stream and returns PF_ERR_TIMEOUT if a grid-barrier wait expired
- * (about one second); the other modes only enqueue. */
+ * the stream and returns PF_ERR_TIMEOUT if a wait between blocks expired
+ * (about one second and more with n_steps); the other modes only enqueue. */
 pf_status pf_step_ensemble(pf_ctx* ctx, float* packed_state, int64_t n_steps, int mode);
 
 /* Failure-detection self-test of the bounded grid barrier used by the persistent

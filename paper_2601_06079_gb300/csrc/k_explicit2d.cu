@@ -13,13 +13,12 @@
 // columns) with the f32x2 instructions of sm_100+, which halve the issue slots
 // of the FP32 work.
 //
-// Quadrature is sum-factorised: per row, two x-interpolated values per
-// segment; per element, the four Gauss values from the segment values of its
-// two rows; the weights N_a(q) are applied back the same way (y first into
-// per-segment sums, then x into the nodes).  Interpolation uses
-// g_hi = 1 - g_lo, e.g. g_hi a + g_lo b = a + g_lo (b - a).  The linear
-// gradient term is the exact assembled 9-point Q1 stencil (2x2 Gauss
-// integrates it exactly); on square cells it is a v + b (sum of the 3x3 block).
+// Quadrature is sum-factorised (sweep2d.h): per row, two x-interpolated values
+// per segment; per element, the four Gauss values from the segment values of
+// its two rows; the weights N_a(q) are applied back the same way (y first into
+// per-segment sums, then x into the nodes).  The linear gradient term is the
+// exact assembled 9-point Q1 stencil (2x2 Gauss integrates it exactly); on
+// square cells it is a v + b (sum of the 3x3 block).
 // Zero-flux boundaries are the mirror extension about the boundary nodes,
 // which equals the partial element sets divided by the partial lumped masses
 // (both double when mirrored), so every node uses the interior formula.  The
@@ -28,12 +27,19 @@
 // the same branch-free sweep with no index reflection.
 #include <string.h>
 
+#include <cmath>
+#include <type_traits>
+
 #include "pf_internal.h"
+#include "sweep2d.h"
 
 namespace pf {
 namespace {
 
-typedef unsigned long long u64;  // packed FP32 pair: low half = lower column
+using namespace sweep;
+
+template <int V>
+using Int = std::integral_constant<int, V>;
 
 constexpr int kPair = 2;                          // columns per lane
 constexpr int kOutCols = 32 * kPair - 2 * kPair;  // 60 output columns per warp
@@ -41,7 +47,6 @@ constexpr int kOutCols = 32 * kPair - 2 * kPair;  // 60 output columns per warp
 #define PF_WARPS 2
 #endif
 constexpr int kWarps = PF_WARPS;                  // warps per block, stacked in y
-constexpr unsigned kFull = 0xffffffffu;
 constexpr int kGhost = 2;  // mirror frame around the working planes
 #ifndef PF_ROWS_AHEAD
 #define PF_ROWS_AHEAD 6
@@ -60,43 +65,6 @@ constexpr int kGhost = 2;  // mirror frame around the working planes
 #endif
 constexpr int kAhead = PF_ROWS_AHEAD;  // rows loaded ahead of use (divides the unroll of 6)
 
-__device__ __forceinline__ u64 pk(float lo, float hi) {
-  u64 r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-  return r;
-}
-__device__ __forceinline__ float plo(u64 v) {
-  float l, h;
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(l), "=f"(h) : "l"(v));
-  return l;
-}
-__device__ __forceinline__ float phi(u64 v) {
-  float l, h;
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(l), "=f"(h) : "l"(v));
-  return h;
-}
-__device__ __forceinline__ u64 fma2(u64 a, u64 b, u64 c) {
-  u64 d;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-  return d;
-}
-__device__ __forceinline__ u64 add2(u64 a, u64 b) {
-  u64 d;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-__device__ __forceinline__ u64 sub2(u64 a, u64 b) {
-  u64 d;
-  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-__device__ __forceinline__ u64 mul2(u64 a, u64 b) {
-  u64 d;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-__device__ __forceinline__ u64 bc(float v) { return pk(v, v); }
-
 __device__ __forceinline__ int reflect_row(int k, int n) {
   k = k < 0 ? -k : k;
   k = k >= n ? 2 * (n - 1) - k : k;
@@ -108,117 +76,6 @@ __device__ __forceinline__ int reflect_col(int x, int n) {
   x %= p;
   if (x < 0) x += p;
   return x < n ? x : p - x;
-}
-
-// f'(shift + d) / 4 (times the stage factor) as a cubic in d
-__device__ __forceinline__ u64 cubic2(u64 d, u64 p0, u64 p1, u64 p2, u64 p3) {
-  return fma2(fma2(fma2(p3, d, p2), d, p1), d, p0);
-}
-
-// Packed constants, read straight from the kernel parameter space.
-struct Coef {
-  const unsigned long long* c;
-  __device__ __forceinline__ u64 glo() const { return c[0]; }
-  __device__ __forceinline__ u64 ghi() const { return c[1]; }
-  __device__ __forceinline__ u64 nglo() const { return c[2]; }
-  __device__ __forceinline__ u64 p(int i) const { return c[3 + i]; }
-  __device__ __forceinline__ u64 k(int stage, int i) const { return c[7 + 6 * stage + i]; }
-};
-
-// Per-row stencil helper value: iso -> v + (v_W + v_E) (3-sum of the row);
-// general -> v_W + v_E.
-template <bool kIso>
-__device__ __forceinline__ u64 row_aux(u64 v, u64 hs) {
-  return kIso ? add2(v, hs) : hs;
-}
-
-// init + K v at the centre row (own values s/c/n, row helpers aux_s/aux_c/aux_n)
-template <bool kIso>
-__device__ __forceinline__ u64 stencil2(u64 init, u64 s, u64 c, u64 n, u64 aux_s, u64 aux_c,
-                                        u64 aux_n, u64 ka, u64 kb, u64 c0, u64 cx, u64 cy,
-                                        u64 cd) {
-  if (kIso) {
-    const u64 s9 = add2(add2(aux_s, aux_c), aux_n);
-    return fma2(kb, s9, fma2(ka, c, init));
-  } else {
-    return fma2(cd, add2(aux_s, aux_n), fma2(cy, add2(s, n), fma2(cx, aux_c, fma2(c0, c, init))));
-  }
-}
-
-// Sliding-window state of one lane (rows k-1, k-2, ...).
-struct Window {
-  u64 c1 = 0, c2 = 0, x1 = 0, x2 = 0;      // own values and row helpers, rows k-1, k-2
-  u64 am1 = 0, ap1 = 0;                    // x-interpolants of row k-1
-  u64 tl1 = 0, th1 = 0;                    // element row k-2 -> node row k-1
-  u64 mua = 0, mub = 0, mxa = 0, mxb = 0;  // CH: mu and helpers, rows k-3, k-2
-};
-
-// One row of the sweep: consume row k (P), advance the window, return the
-// finished output row (k-1 for AC, k-2 for CH).
-template <bool kCH, bool kIso>
-__device__ __forceinline__ u64 sweep_row(const u64 P, Window& w, const Coef& K) {
-  const float c0 = plo(P), c1v = phi(P);
-  const float cl = __shfl_up_sync(kFull, c1v, 1);   // column x-1
-  const float cr = __shfl_down_sync(kFull, c0, 1);  // column x+2
-  // horizontal neighbour sums and segment differences, formed as scalars so
-  // that no pair has to be re-packed from halves of other pairs
-  const u64 hs = pk(cl + c1v, c0 + cr);
-  const u64 dc = pk(c1v - c0, cr - c1v);
-  const u64 xr = row_aux<kIso>(P, hs);
-
-  // x-interpolation of row k on segments x, x+1 at xi = g_lo (am) and g_hi (ap)
-  const u64 am = fma2(K.glo(), dc, P);
-  const u64 ap = fma2(K.ghi(), dc, P);
-
-  // element row k-1: four Gauss values, f', weights back in y
-  const u64 dm = sub2(am, w.am1);
-  const u64 dp = sub2(ap, w.ap1);
-  const u64 fll = cubic2(fma2(K.glo(), dm, w.am1), K.p(0), K.p(1), K.p(2), K.p(3));
-  const u64 flh = cubic2(fma2(K.ghi(), dm, w.am1), K.p(0), K.p(1), K.p(2), K.p(3));
-  const u64 fhl = cubic2(fma2(K.glo(), dp, w.ap1), K.p(0), K.p(1), K.p(2), K.p(3));
-  const u64 fhh = cubic2(fma2(K.ghi(), dp, w.ap1), K.p(0), K.p(1), K.p(2), K.p(3));
-  const u64 dl = sub2(flh, fll);
-  const u64 dh = sub2(fhh, fhl);
-  const u64 sl = add2(fma2(K.glo(), dl, fll), w.tl1);  // node row k-1, xi = g_lo
-  const u64 sh = add2(fma2(K.glo(), dh, fhl), w.th1);  // node row k-1, xi = g_hi
-  const u64 tl = fma2(K.nglo(), dl, flh);              // node row k (next row)
-  const u64 th = fma2(K.nglo(), dh, fhh);
-  // weights back in x: segment s gives A to node s and B to node s+1
-  const u64 ds = sub2(sh, sl);
-  const u64 A = fma2(K.glo(), ds, sl);
-  const u64 B = fma2(K.nglo(), ds, sh);
-  const float bl = __shfl_up_sync(kFull, phi(B), 1);
-  const u64 F = pk(plo(A) + bl, phi(A) + plo(B));
-
-  u64 o;
-  if constexpr (!kCH) {
-    // u(k-1) <- u + F + K1 u   (coefficients carry -dt L / m)
-    o = stencil2<kIso>(add2(w.c1, F), w.c2, w.c1, P, w.x2, w.x1, xr, K.k(0, 0), K.k(0, 1), K.k(0, 2),
-                       K.k(0, 3), K.k(0, 4), K.k(0, 5));
-  } else {
-    // mu(k-1) = F + K1 c ; then c(k-2) <- c + K2 mu   (K2 carries -dt M / m)
-    const u64 mu = stencil2<kIso>(F, w.c2, w.c1, P, w.x2, w.x1, xr, K.k(0, 0), K.k(0, 1), K.k(0, 2),
-                                  K.k(0, 3), K.k(0, 4), K.k(0, 5));
-    const float m0 = plo(mu), m1 = phi(mu);
-    const float ml = __shfl_up_sync(kFull, m1, 1);
-    const float mr = __shfl_down_sync(kFull, m0, 1);
-    const u64 mx = row_aux<kIso>(mu, pk(ml + m1, m0 + mr));
-    o = stencil2<kIso>(w.c2, w.mua, w.mub, mu, w.mxa, w.mxb, mx, K.k(1, 0), K.k(1, 1), K.k(1, 2), K.k(1, 3),
-                       K.k(1, 4), K.k(1, 5));
-    w.mua = w.mub;
-    w.mxa = w.mxb;
-    w.mub = mu;
-    w.mxb = mx;
-  }
-  w.c2 = w.c1;
-  w.x2 = w.x1;
-  w.c1 = P;
-  w.x1 = xr;
-  w.am1 = am;
-  w.ap1 = ap;
-  w.tl1 = tl;
-  w.th1 = th;
-  return o;
 }
 
 // Output of one finished pair: real row y, real columns x (lo) and x+1 (hi),
@@ -290,11 +147,10 @@ __device__ __forceinline__ u64 l2_policy(int l2) {
   return p;
 }
 
-template <bool kCH, bool kIso, int kTY, bool kCoherent = false, bool kHint = false>
+template <bool kCH, bool kIso, bool kOdd, int kTY, bool kCoherent = false, bool kHint = false>
 __device__ __forceinline__ void sweep_task(const Explicit2DArgs& a, const float* in, float* out,
                                            const Coef& K, int bx, int y0, u64 pol = 0) {
   constexpr int kLag = kCH ? 2 : 1;
-  constexpr int kWarm = 2 * kLag;  // rows consumed before the first finished row
   const int lane = threadIdx.x & 31;
   const int nx = a.nx, ny = a.ny;
   const int64_t pitch = a.pitch;
@@ -308,48 +164,56 @@ __device__ __forceinline__ void sweep_task(const Explicit2DArgs& a, const float*
   const float* __restrict__ in0 = in + kGhost * pitch + kGhost;
   float* __restrict__ out0 = out + kGhost * pitch + kGhost;
   const float* src = in0 + (int64_t)(y0 - kLag) * pitch + x;
-  Window w;
+  Window<1> w;
   u64 ahead[kAhead];  // rows k .. k+kAhead-1 in flight
 #pragma unroll
   for (int j = 0; j < kAhead; ++j) {
     ahead[j] = ld_row<kCoherent, kHint>(src, pol);
     src += pitch;
   }
-#pragma unroll
-  for (int it = 0; it < kWarm; ++it) {  // fill the window, nothing to store yet
+  const auto next = [&]() {
     const u64 P = ahead[0];
 #pragma unroll
     for (int j = 0; j + 1 < kAhead; ++j) ahead[j] = ahead[j + 1];
     ahead[kAhead - 1] = ld_row<kCoherent, kHint>(src, pol);
     src += pitch;
-    sweep_row<kCH, kIso>(P, w, K);
+    return P;
+  };
+  u64 o[1];
+  const auto consume = [&](auto stage) {
+    const u64 P[1] = {next()};
+    const float cl = __shfl_up_sync(kFull, phi(P[0]), 1);   // column x-1
+    const float cr = __shfl_down_sync(kFull, plo(P[0]), 1);  // column x+2
+    row<kCH, kIso, kOdd, 1, decltype(stage)::value, false>(P, cl, cr, 0.0f, w, K, o);
+  };
+  // fill the window, nothing to store yet: each row goes as far as later rows need
+  consume(Int<kInterp>{});
+  consume(Int<kElement>{});
+  if constexpr (kCH) {
+    consume(Int<kMu>{});
+    consume(Int<kMu>{});
   }
 #pragma unroll 6
   for (int it = 0; it < kTY; ++it) {
-    const u64 P = ahead[0];
-#pragma unroll
-    for (int j = 0; j + 1 < kAhead; ++j) ahead[j] = ahead[j + 1];
-    ahead[kAhead - 1] = ld_row<kCoherent, kHint>(src, pol);
-    src += pitch;
-    const u64 o = sweep_row<kCH, kIso>(P, w, K);
+    consume(Int<kOutput>{});
     const int y = y0 + it;
     if (plain)
-      st_row<kHint>(out0 + (int64_t)y * pitch + x, o, pol);
+      st_row<kHint>(out0 + (int64_t)y * pitch + x, o[0], pol);
     else if (writer && y < ny)
-      store_out(out0, pitch, y, ny, x, nx, o);
+      store_out(out0, pitch, y, ny, x, nx, o[0]);
   }
 }
 
 // One warp per block and one (column, band) task per warp: many small blocks
 // spread evenly over the SMs and keep each scheduler fed from several warps.
-template <bool kCH, bool kIso, int kTY>
+template <bool kCH, bool kIso, bool kOdd, int kTY>
 __global__ void __launch_bounds__(kWarps * 32, PF_MINB) k_explicit2d(const Explicit2DArgs a) {
 #if PF_PDL
   asm volatile("griddepcontrol.wait;" ::: "memory");  // the previous step is complete
 #endif
   const int warp = threadIdx.x >> 5;
   const int y0 = (block_row() * kWarps + warp) * kTY;
-  if (y0 < a.ny) sweep_task<kCH, kIso, kTY>(a, a.in, a.out, Coef{a.pair}, blockIdx.x, y0);
+  if (y0 < a.ny) sweep_task<kCH, kIso, kOdd, kTY>(a, a.in, a.out, Coef{a.pair}, blockIdx.x, y0);
 #if PF_PDL
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 #endif
@@ -363,7 +227,7 @@ __global__ void __launch_bounds__(kWarps * 32, PF_MINB) k_explicit2d(const Expli
 // whole ensemble.  The persistent form keeps one launch resident for all
 // steps, with a bounded grid barrier between steps.
 
-template <bool kIso, bool kCoherent>
+template <bool kIso, bool kOdd, bool kCoherent>
 __device__ __forceinline__ void ensemble_task(const EnsTask& t, const Explicit2DArgs* inst,
                                               int parity) {
   const Explicit2DArgs& a = inst[t.inst];
@@ -386,20 +250,20 @@ __device__ __forceinline__ void ensemble_task(const EnsTask& t, const Explicit2D
   float* out = parity ? const_cast<float*>(a.in) : a.out;
   const u64 pol = l2_policy(a.l2);
   switch (t.ty) {
-    case 6: sweep_task<false, kIso, 6, kCoherent, true>(a, in, out, K, t.bx, t.y0, pol); break;
-    case 12: sweep_task<false, kIso, 12, kCoherent, true>(a, in, out, K, t.bx, t.y0, pol); break;
-    default: sweep_task<false, kIso, 24, kCoherent, true>(a, in, out, K, t.bx, t.y0, pol); break;
+    case 6: sweep_task<false, kIso, kOdd, 6, kCoherent, true>(a, in, out, K, t.bx, t.y0, pol); break;
+    case 12: sweep_task<false, kIso, kOdd, 12, kCoherent, true>(a, in, out, K, t.bx, t.y0, pol); break;
+    default: sweep_task<false, kIso, kOdd, 24, kCoherent, true>(a, in, out, K, t.bx, t.y0, pol); break;
   }
 }
 
-template <bool kIso>
+template <bool kIso, bool kOdd>
 __global__ void __launch_bounds__(kEnsThreads, PF_ENS_MINB) k_ensemble_step(const EnsTask* __restrict__ tasks,
                                                               int ntasks,
                                                               const Explicit2DArgs* inst,
                                                               int parity) {
   const int warps = kEnsThreads / 32;
   for (int t = blockIdx.x * warps + (threadIdx.x >> 5); t < ntasks; t += gridDim.x * warps)
-    ensemble_task<kIso, false>(tasks[t], inst, parity);
+    ensemble_task<kIso, kOdd, false>(tasks[t], inst, parity);
 }
 
 // Grid-wide barrier for a co-resident (cooperative) grid.  bar[0] counts
@@ -435,14 +299,14 @@ __device__ bool grid_barrier(unsigned* bar, long long limit) {
   return ok != 0;
 }
 
-template <bool kIso>
+template <bool kIso, bool kOdd>
 __global__ void __launch_bounds__(kEnsThreads, PF_ENS_MINB) k_ensemble_persistent(
     const EnsTask* __restrict__ tasks, int ntasks, const Explicit2DArgs* inst, int n_steps,
     unsigned* bar, long long limit) {
   const int warps = kEnsThreads / 32;
   for (int s = 0; s < n_steps; ++s) {
     for (int t = blockIdx.x * warps + (threadIdx.x >> 5); t < ntasks; t += gridDim.x * warps)
-      ensemble_task<kIso, true>(tasks[t], inst, s & 1);
+      ensemble_task<kIso, kOdd, true>(tasks[t], inst, s & 1);
     if (!grid_barrier(bar, limit)) return;
   }
 }
@@ -550,12 +414,16 @@ __global__ void k_from_work(const float* __restrict__ work, float* __restrict__ 
 #define PF_TY_CH 6
 #endif
 #ifndef PF_TY_AC
-#define PF_TY_AC 12
+#define PF_TY_AC 6
 #endif
-constexpr int kTYAc = PF_TY_AC;  // output rows per warp band (a multiple of the unroll of 6)
+// Output rows per warp band (a multiple of the unroll of 6).  Taller bands
+// repeat fewer warm-up rows but leave fewer warps and, as a loop, hold the
+// coefficients in registers (110 against 70): Allen-Cahn at 12 rows took 59 us
+// per step at 4096^2 and 22 at 2700^2, at 6 rows 29 and 13.
+constexpr int kTYAc = PF_TY_AC;
 constexpr int kTYCh = PF_TY_CH;
 
-template <bool kCH, bool kIso, int kTY>
+template <bool kCH, bool kIso, bool kOdd, int kTY>
 cudaError_t launch(const Explicit2DArgs& a, cudaStream_t s) {
   const dim3 grid = row_grid((a.nx + kOutCols - 1) / kOutCols, (a.ny + kWarps * kTY - 1) / (kWarps * kTY));
 #if PF_PDL
@@ -568,9 +436,9 @@ cudaError_t launch(const Explicit2DArgs& a, cudaStream_t s) {
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_explicit2d<kCH, kIso, kTY>, a);
+  return cudaLaunchKernelEx(&cfg, k_explicit2d<kCH, kIso, kOdd, kTY>, a);
 #else
-  k_explicit2d<kCH, kIso, kTY><<<grid, kWarps * 32, 0, s>>>(a);
+  k_explicit2d<kCH, kIso, kOdd, kTY><<<grid, kWarps * 32, 0, s>>>(a);
   return cudaGetLastError();
 #endif
 }
@@ -580,12 +448,19 @@ bool is_iso(const Stencil2D& k) { return k.cx == k.cd && k.cy == k.cd; }
 }  // namespace
 
 cudaError_t launch_ac2d(const Explicit2DArgs& a, cudaStream_t s) {
-  return is_iso(a.k1) ? launch<false, true, kTYAc>(a, s) : launch<false, false, kTYAc>(a, s);
+  switch (sweep_variant(is_iso(a.k1), a.odd)) {
+    case 0: return launch<false, true, true, kTYAc>(a, s);
+    case 1: return launch<false, false, true, kTYAc>(a, s);
+    default: return launch<false, false, false, kTYAc>(a, s);
+  }
 }
 
 cudaError_t launch_ch2d(const Explicit2DArgs& a, cudaStream_t s) {
-  return (is_iso(a.k1) && is_iso(a.k2)) ? launch<true, true, kTYCh>(a, s)
-                                        : launch<true, false, kTYCh>(a, s);
+  switch (sweep_variant(is_iso(a.k1) && is_iso(a.k2), a.odd)) {
+    case 0: return launch<true, true, true, kTYCh>(a, s);
+    case 1: return launch<true, false, true, kTYCh>(a, s);
+    default: return launch<true, false, false, kTYCh>(a, s);
+  }
 }
 
 void pack_explicit2d(Explicit2DArgs& a) {
@@ -594,13 +469,16 @@ void pack_explicit2d(Explicit2DArgs& a) {
     memcpy(&b, &v, 4);
     return (unsigned long long)b | ((unsigned long long)b << 32);
   };
-  a.pair[0] = pk_host(kGLo);
-  a.pair[1] = pk_host(kGHi);
-  a.pair[2] = pk_host(-kGLo);
-  a.pair[3] = pk_host(a.p0);
-  a.pair[4] = pk_host(a.p1);
-  a.pair[5] = pk_host(a.p2);
-  a.pair[6] = pk_host(a.p3);
+  // interpolated values lack a factor g_hi^2 and so do the weights back, so
+  // p_i carries g_hi^(2 i + 2); the polynomial is odd about the double well's
+  // centre (p0 = p2 = 0), and its form p3 (v^2 + p1/p3) v needs p3 != 0
+  const double g2 = (double)kGHi * kGHi;
+  const double p[4] = {a.p0 * g2, a.p1 * g2 * g2, a.p2 * g2 * g2 * g2, a.p3 * g2 * g2 * g2 * g2};
+  a.odd = a.p0 == 0.0f && a.p2 == 0.0f && a.p3 != 0.0f && std::isfinite(p[1] / p[3]);
+  a.pair[0] = pk_host((float)((double)kGLo / kGHi));
+  a.pair[1] = pk_host(a.odd ? (float)(p[1] / p[3]) : 0.0f);
+  a.pair[2] = pk_host((float)p[3]);
+  for (int i = 0; i < 4; ++i) a.pair[3 + i] = pk_host((float)p[i]);
   const Stencil2D* st[2] = {&a.k1, &a.k2};
   for (int s = 0; s < 2; ++s) {
     a.pair[7 + 6 * s + 0] = pk_host(st[s]->c0 - st[s]->cd);
@@ -613,29 +491,35 @@ void pack_explicit2d(Explicit2DArgs& a) {
 }
 
 cudaError_t launch_ensemble_step(const EnsTask* tasks, int ntasks, const Explicit2DArgs* inst,
-                                 int parity, bool iso, int grid, cudaStream_t s) {
-  if (iso)
-    k_ensemble_step<true><<<grid, kEnsThreads, 0, s>>>(tasks, ntasks, inst, parity);
-  else
-    k_ensemble_step<false><<<grid, kEnsThreads, 0, s>>>(tasks, ntasks, inst, parity);
+                                 int parity, bool iso, bool odd, int grid, cudaStream_t s) {
+  const int v = sweep_variant(iso, odd);
+  auto* k = v == 0   ? k_ensemble_step<true, true>
+            : v == 1 ? k_ensemble_step<false, true>
+                     : k_ensemble_step<false, false>;
+  k<<<grid, kEnsThreads, 0, s>>>(tasks, ntasks, inst, parity);
   return cudaGetLastError();
 }
 
-int ensemble_persistent_grid(bool iso) {
-  int dev = 0, sms = 0, per = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
-  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
-  cudaError_t e = iso ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                            &per, k_ensemble_persistent<true>, kEnsThreads, 0)
-                      : cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                            &per, k_ensemble_persistent<false>, kEnsThreads, 0);
-  if (e != cudaSuccess) return 0;
-  return sms * per;
+namespace {
+auto* persistent_kernel(bool iso, bool odd) {
+  const int v = sweep_variant(iso, odd);
+  return v == 0   ? k_ensemble_persistent<true, true>
+         : v == 1 ? k_ensemble_persistent<false, true>
+                  : k_ensemble_persistent<false, false>;
+}
+}  // namespace
+
+int ensemble_persistent_grid(bool iso, bool odd) {
+  int per = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, persistent_kernel(iso, odd), kEnsThreads,
+                                                    0) != cudaSuccess)
+    return 0;
+  return device_sm_count() * per;
 }
 
 cudaError_t launch_ensemble_persistent(const EnsTask* tasks, int ntasks, const Explicit2DArgs* inst,
                                        int n_steps, unsigned* bar, long long limit, bool iso,
-                                       int grid, cudaStream_t s) {
+                                       bool odd, int grid, cudaStream_t s) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(kEnsThreads);
@@ -645,10 +529,8 @@ cudaError_t launch_ensemble_persistent(const EnsTask* tasks, int ntasks, const E
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return iso ? cudaLaunchKernelEx(&cfg, k_ensemble_persistent<true>, tasks, ntasks, inst, n_steps,
-                                  bar, limit)
-             : cudaLaunchKernelEx(&cfg, k_ensemble_persistent<false>, tasks, ntasks, inst, n_steps,
-                                  bar, limit);
+  return cudaLaunchKernelEx(&cfg, persistent_kernel(iso, odd), tasks, ntasks, inst, n_steps, bar,
+                            limit);
 }
 
 cudaError_t launch_ens_to_work(const float* packed, const int64_t* off, const Explicit2DArgs* inst,

@@ -38,6 +38,10 @@ struct pf_ctx {
   double* partials = nullptr;
   double* result = nullptr;
 
+  // explicit trajectories held on chip
+  pf::OnchipJob oc{};
+  bool oc_fits = false;
+
   // derived coefficients
   pf::Explicit2DArgs ex{};
   pf::Implicit3DArgs im{};
@@ -75,6 +79,15 @@ struct pf_ctx {
   unsigned* ens_bar = nullptr;
   int ens_ntasks = 0;
   bool ens_iso = true;
+  bool ens_odd = true;
+  // the persistent form held on chip (no jobs: an instance does not fit)
+  std::vector<pf::OnchipJob> ens_jobs;
+  std::vector<pf::OnchipItem> ens_list;
+  std::vector<int> ens_first;
+  size_t ens_xchg = 0, ens_smem = 0;
+  pf::OnchipJob* ens_djobs = nullptr;
+  pf::OnchipItem* ens_dlist = nullptr;
+  int* ens_dfirst = nullptr;
 
   std::string err;
 };
@@ -82,6 +95,15 @@ struct pf_ctx {
 namespace {
 
 constexpr int kGraphSteps = 64;  // even, so a replay returns to buf_a
+// Fewest steps taken on chip.  Loading and storing the tiles, their tables, the
+// exchange buffer's zeroing and a cooperative launch cost about 15 us at 64^2
+// and 100 us at 2048^2 (the tiles are 16 times as tall), which the steps have to
+// win back against one launch each: 8 steps take 21 against 67 us (Allen-Cahn,
+// 64^2), 47 against 67 (Cahn-Hilliard, 515 x 1031), 173 against 135 (2048^2;
+// 32 steps: 383 against 431).
+int64_t onchip_steps(int64_t nodes) { return 8 + (nodes >> 18); }
+constexpr size_t kOnchipErr = 256;  // error flag in front of the exchange buffer
+constexpr long long kWaitCycles = 2000000000LL;  // about one second
 
 size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
@@ -389,7 +411,7 @@ AdjLayout adj_layout(const pf_ctx* c, int64_t n_steps, int ckpt) {
 struct EnsLayout {
   std::vector<size_t> plane;  // offset of instance i's plane A (B follows)
   std::vector<size_t> plane_bytes;
-  size_t args, tasks, offs, bar, total;
+  size_t args, tasks, offs, bar, jobs, list, first, total;
   int max_tasks;
 };
 
@@ -417,6 +439,12 @@ EnsLayout ens_layout(const pf_ctx* c) {
   off += align_up(sizeof(int64_t) * (c->ens_count + 1), 256);
   L.bar = off;
   off += 256;
+  L.jobs = off;
+  off += align_up(sizeof(pf::OnchipJob) * c->ens_jobs.size(), 256);
+  L.list = off;
+  off += align_up(sizeof(pf::OnchipItem) * c->ens_list.size(), 256);
+  L.first = off;
+  off += align_up(sizeof(int) * c->ens_first.size(), 256);
   L.total = off;
   return L;
 }
@@ -670,6 +698,12 @@ pf_status pf_create_mesh(pf_ctx** out, int dim, const int64_t nodes[3], const do
   c->nf = n_fields;
   c->stream = (cudaStream_t)stream;
   const Layout L = layout(c);
+  if (dim == 2 && (model == PF_MODEL_AC || model == PF_MODEL_CH)) {
+    c->oc.nx = (int)nodes[0];
+    c->oc.ny = (int)nodes[1];
+    const bool ch = model == PF_MODEL_CH;
+    c->oc_fits = L.partials > kOnchipErr && pf::onchip_plan(ch, L.partials - kOnchipErr, &c->oc);
+  }
   c->ws_bytes = L.total;
   c->ws_explicit = L.explicit_total;
   *workspace_bytes = c->ws_bytes;
@@ -703,6 +737,9 @@ pf_status pf_bind_workspace(pf_ctx* c, void* dev_ptr, size_t bytes) {
     c->ens_tasks = (pf::EnsTask*)(c->ws + E.tasks);
     c->ens_doff = (int64_t*)(c->ws + E.offs);
     c->ens_bar = (unsigned*)(c->ws + E.bar);
+    c->ens_djobs = (pf::OnchipJob*)(c->ws + E.jobs);
+    c->ens_dlist = (pf::OnchipItem*)(c->ws + E.list);
+    c->ens_dfirst = (int*)(c->ws + E.first);
     destroy_graph(c);
     return PF_OK;
   }
@@ -903,6 +940,28 @@ pf_status step_plain2d(pf_ctx* c, float* state, int64_t n_steps) {
   return PF_OK;
 }
 
+// The whole trajectory in one launch, the state on chip; the working planes'
+// memory holds the exchange buffer.
+pf_status step_onchip(pf_ctx* c, float* state, int n_steps) {
+  const bool ch = c->model == PF_MODEL_CH;
+  pf::OnchipArgs a{};
+  a.state = state;
+  a.job = c->oc;
+  a.job.shift = (float)c->par.shift;
+  memcpy(a.job.pair, c->ex.pair, sizeof(a.job.pair));
+  char* buf = (char*)c->buf_a;
+  a.err = (unsigned*)buf;
+  a.xchg = buf + kOnchipErr;
+  a.limit = kWaitCycles;
+  a.n_steps = n_steps;
+  const size_t bytes = pf::onchip_exchange_bytes(ch, c->oc);
+  if (bytes) PF_CUDA(cudaMemsetAsync(buf, 0, kOnchipErr + bytes, c->stream));
+  const auto iso = [](const pf::Stencil2D& k) { return k.cx == k.cd && k.cy == k.cd; };
+  PF_CUDA(pf::launch_onchip(ch, a, iso(c->ex.k1) && (!ch || iso(c->ex.k2)),
+                            c->ex.odd != 0, c->stream));
+  return PF_OK;
+}
+
 pf_status pf_step_explicit(pf_ctx* c, float* state, int64_t n_steps) {
   if (!c) return PF_ERR_ARG;
   if (!c->ws) return fail(c, PF_ERR_STATE, "no workspace bound");
@@ -914,6 +973,9 @@ pf_status pf_step_explicit(pf_ctx* c, float* state, int64_t n_steps) {
   if (c->model == PF_MODEL_COUPLED) return step_coupled2d(c, state, n_steps);
   if (c->par.mobility_field) return step_explicit_mob(c, state, n_steps);
   if (c->form == PF_FORM_TWO_PASS) return step_plain2d(c, state, n_steps);
+  if (c->form == PF_FORM_FUSED_GRAPH && c->oc_fits && n_steps >= onchip_steps(nodes2d(c)) &&
+      n_steps <= INT32_MAX)
+    return step_onchip(c, state, (int)n_steps);
   const float shift = (float)c->par.shift;
   const int nx = (int)c->n[0], ny = (int)c->n[1];
   // working copies with the mirror frame: d = u - shift (both planes fully defined)
@@ -1087,6 +1149,20 @@ pf_status pf_create_ensemble(pf_ctx** out, int count, const int64_t* nx, const i
   }
   c->n[0] = nx[0];
   c->n[1] = ny[0];
+  for (int i = 0; i < count; ++i) {
+    pf::OnchipJob b{};
+    b.nx = (int)nx[i];
+    b.ny = (int)ny[i];
+    b.off = c->ens_off[i];
+    c->ens_jobs.push_back(b);
+  }
+  if (!pf::onchip_plan_ensemble(c->ens_jobs, &c->ens_first, &c->ens_list, &c->ens_xchg,
+                                &c->ens_smem) ||
+      c->ens_xchg > ens_layout(c).args) {
+    c->ens_jobs.clear();
+    c->ens_list.clear();
+    c->ens_first.clear();
+  }
   c->ws_bytes = ens_layout(c).total;
   *workspace_bytes = c->ws_bytes;
   if (offsets)
@@ -1100,7 +1176,7 @@ pf_status pf_set_ensemble_params(pf_ctx* c, const pf_params* p) {
   if (c->ens_count < 1) return fail(c, PF_ERR_ARG, "not an ensemble context");
   if (!c->ws) return fail(c, PF_ERR_STATE, "no workspace bound");
   if (!p) return fail(c, PF_ERR_ARG, "params is NULL");
-  c->ens_iso = true;
+  c->ens_iso = c->ens_odd = true;
   for (int i = 0; i < c->ens_count; ++i) {
     const pf_params& q = p[i];
     if (!(q.dt > 0.0) || !(q.kappa >= 0.0) || !(q.mobility > 0.0) || !(q.W >= 0.0) ||
@@ -1121,6 +1197,7 @@ pf_status pf_set_ensemble_params(pf_ctx* c, const pf_params* p) {
     a.k2 = stiffness2d(hx, hy, 0.0);
     pf::pack_explicit2d(a);
     if (!(a.k1.cx == a.k1.cd && a.k1.cy == a.k1.cd)) c->ens_iso = false;
+    if (!a.odd) c->ens_odd = false;
   }
   c->par = p[0];
   c->par_set = true;
@@ -1129,6 +1206,20 @@ pf_status pf_set_ensemble_params(pf_ctx* c, const pf_params* p) {
                           c->stream));
   PF_CUDA(cudaMemcpyAsync(c->ens_doff, c->ens_off.data(), sizeof(int64_t) * (c->ens_count + 1),
                           cudaMemcpyHostToDevice, c->stream));
+  if (!c->ens_jobs.empty()) {
+    for (int i = 0; i < c->ens_count; ++i) {
+      c->ens_jobs[i].shift = (float)p[0].shift;
+      memcpy(c->ens_jobs[i].pair, c->ens_args[i].pair, sizeof(c->ens_args[i].pair));
+    }
+    PF_CUDA(cudaMemcpyAsync(c->ens_djobs, c->ens_jobs.data(),
+                            sizeof(pf::OnchipJob) * c->ens_jobs.size(), cudaMemcpyHostToDevice,
+                            c->stream));
+    PF_CUDA(cudaMemcpyAsync(c->ens_dlist, c->ens_list.data(),
+                            sizeof(pf::OnchipItem) * c->ens_list.size(), cudaMemcpyHostToDevice,
+                            c->stream));
+    PF_CUDA(cudaMemcpyAsync(c->ens_dfirst, c->ens_first.data(), sizeof(int) * c->ens_first.size(),
+                            cudaMemcpyHostToDevice, c->stream));
+  }
   std::vector<int> all(c->ens_count);
   for (int i = 0; i < c->ens_count; ++i) all[i] = i;
   return ens_upload_tasks(c, ens_build_tasks(c, all));
@@ -1206,11 +1297,11 @@ pf_status pf_tune_ensemble(pf_ctx* c, int reps, int* ty_out, int* l2_out, double
     double best = 1e30;
     for (int round = 0; round < 3; ++round) {
       cudaError_t e = pf::launch_ensemble_step(c->ens_tasks, c->ens_ntasks, c->ens_dargs, 0,
-                                               c->ens_iso, grid, c->stream);  // warm-up
+                                               c->ens_iso, c->ens_odd, grid, c->stream);  // warm-up
       if (e == cudaSuccess) e = cudaEventRecord(e0, c->stream);
       for (int r = 0; r < reps && e == cudaSuccess; ++r)
         e = pf::launch_ensemble_step(c->ens_tasks, c->ens_ntasks, c->ens_dargs, (r + 1) & 1,
-                                     c->ens_iso, grid, c->stream);
+                                     c->ens_iso, c->ens_odd, grid, c->stream);
       if (e == cudaSuccess) e = cudaEventRecord(e1, c->stream);
       if (e == cudaSuccess) e = cudaEventSynchronize(e1);
       float ms = 0.0f;
@@ -1289,17 +1380,45 @@ pf_status pf_step_ensemble(pf_ctx* c, float* packed, int64_t n_steps, int mode) 
   if (mode < PF_ENS_PERSISTENT || mode > PF_ENS_PLAIN) return fail(c, PF_ERR_ARG, "bad mode");
   if (n_steps == 0) return PF_OK;
   const float shift = (float)c->par.shift;
+  if (mode == PF_ENS_PERSISTENT && !c->ens_jobs.empty() && n_steps >= onchip_steps(c->ens_off.back())) {
+    // one launch holds every instance on chip for all its steps; the working
+    // planes' memory is the exchange buffer
+    PF_CUDA(cudaMemsetAsync(c->ens_bar, 0, 3 * sizeof(unsigned), c->stream));
+    if (c->ens_xchg) PF_CUDA(cudaMemsetAsync(c->ws, 0, c->ens_xchg, c->stream));
+    pf::OnchipArgs a{};
+    a.state = packed;
+    a.jobs = c->ens_djobs;
+    a.list = c->ens_dlist;
+    a.list_first = c->ens_dfirst;
+    a.xchg = c->ws;
+    a.err = c->ens_bar + 2;
+    // a tile may wait for the others of its instance to finish earlier ones:
+    // far below 100,000 cycles per step of each
+    size_t longest = 0;
+    for (size_t b = 0; b + 1 < c->ens_first.size(); ++b)
+      longest = std::max(longest, (size_t)(c->ens_first[b + 1] - c->ens_first[b]));
+    a.limit = kWaitCycles + 100000LL * n_steps * (long long)longest;
+    a.n_steps = (int)n_steps;
+    PF_CUDA(pf::launch_onchip_ensemble(a, c->ens_smem, c->ens_iso, c->ens_odd,
+                                       c->stream));
+    unsigned flag = 0;
+    PF_CUDA(cudaMemcpyAsync(&flag, c->ens_bar + 2, sizeof(unsigned), cudaMemcpyDeviceToHost,
+                            c->stream));
+    PF_CUDA(cudaStreamSynchronize(c->stream));
+    if (flag) return fail(c, PF_ERR_TIMEOUT, "a tile's wait expired in the persistent ensemble");
+    return PF_OK;
+  }
   PF_CUDA(pf::launch_ens_to_work(packed, c->ens_doff, c->ens_dargs, c->ens_count, shift, c->stream));
   if (mode == PF_ENS_PERSISTENT) {
-    const int grid = pf::ensemble_persistent_grid(c->ens_iso);
+    const int grid = pf::ensemble_persistent_grid(c->ens_iso, c->ens_odd);
     if (grid < 1) return fail(c, PF_ERR_CUDA, "cannot size the persistent grid");
     PF_CUDA(cudaMemsetAsync(c->ens_bar, 0, 3 * sizeof(unsigned), c->stream));
     // one persistent launch for all steps, recorded as a one-node CUDA graph
     if (!c->cap_stream) PF_CUDA(cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking));
     PF_CUDA(cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal));
     cudaError_t le = pf::launch_ensemble_persistent(c->ens_tasks, c->ens_ntasks, c->ens_dargs,
-                                                    (int)n_steps, c->ens_bar, 2000000000LL,
-                                                    c->ens_iso, grid, c->cap_stream);
+                                                    (int)n_steps, c->ens_bar, kWaitCycles,
+                                                    c->ens_iso, c->ens_odd, grid, c->cap_stream);
     cudaGraph_t g = nullptr;
     cudaError_t ee = cudaStreamEndCapture(c->cap_stream, &g);
     if (le != cudaSuccess || ee != cudaSuccess) {
@@ -1317,11 +1436,12 @@ pf_status pf_step_ensemble(pf_ctx* c, float* packed, int64_t n_steps, int mode) 
     const int grid = ens_step_grid(c->ens_ntasks);
     for (int64_t s = 0; s < n_steps; ++s)
       PF_CUDA(pf::launch_ensemble_step(c->ens_tasks, c->ens_ntasks, c->ens_dargs, (int)(s & 1),
-                                       c->ens_iso, grid, c->stream));
+                                       c->ens_iso, c->ens_odd, grid, c->stream));
   } else {  // plain: the single-instance fused step, one launch per instance and step
     for (int64_t s = 0; s < n_steps; ++s)
       for (int i = 0; i < c->ens_count; ++i) {
         pf::Explicit2DArgs a = c->ens_args[i];
+        a.odd = c->ens_odd;  // the form of the batched kernels
         if (s & 1) {
           a.in = a.out;
           a.out = const_cast<float*>(c->ens_args[i].in);

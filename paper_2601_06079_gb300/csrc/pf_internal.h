@@ -6,6 +6,7 @@
 
 #include <atomic>
 #include <string>
+#include <vector>
 
 #include "../../include/pf.h"
 
@@ -69,6 +70,10 @@ struct Stencil2D {
   float c0, cx, cy, cd;
 };
 
+// The explicit kernels are built for square cells with the odd polynomial (0),
+// the general stencil with the odd polynomial (1), and neither (2).
+inline int sweep_variant(bool iso, bool odd) { return odd ? (iso ? 0 : 1) : 2; }
+
 // Arguments of one fused explicit step on a 2-D mesh.  The state is the
 // shifted FP32 variable d = u - shift; the mirror extension about boundary
 // nodes reproduces the zero-flux Q1 operators divided by the lumped mass, so
@@ -84,9 +89,9 @@ struct Explicit2DArgs {
   Stencil2D k1;  // AC: -dt L kappa / m * K;   CH: kappa / m * K  (mu stage)
   Stencil2D k2;  // CH: -dt M / m * K          (c stage)
   // the same constants duplicated into FP32 pairs for the packed f32x2 path
-  // (filled by pack_explicit2d): g_lo, g_hi, -g_lo, p0..p3, then per stencil
-  // a = c0 - cd, b = cd, c0, cx, cy, cd
+  // (filled by pack_explicit2d; sweep2d.h says which)
   unsigned long long pair[7 + 12];
+  int odd;  // p0 = p2 = 0: the polynomial is taken in its odd form
   // L2 eviction priority of the working planes' row loads and stores in the
   // ensemble sweep (kL2Normal, kL2Stream, kL2StreamHalf); single-mesh steps
   // ignore it
@@ -126,12 +131,12 @@ constexpr int kEnsThreads = 128;
 constexpr int kMaxEnsTY = 24;
 constexpr int kEnsOutCols = 60;
 cudaError_t launch_ensemble_step(const EnsTask* tasks, int ntasks, const Explicit2DArgs* inst,
-                                 int parity, bool iso, int grid, cudaStream_t s);
-int ensemble_persistent_grid(bool iso);
+                                 int parity, bool iso, bool odd, int grid, cudaStream_t s);
+int ensemble_persistent_grid(bool iso, bool odd);
 cudaError_t launch_barrier_selftest(unsigned* bar, long long limit, int extra, cudaStream_t s);
 cudaError_t launch_ensemble_persistent(const EnsTask* tasks, int ntasks, const Explicit2DArgs* inst,
                                        int n_steps, unsigned* bar, long long limit, bool iso,
-                                       int grid, cudaStream_t s);
+                                       bool odd, int grid, cudaStream_t s);
 cudaError_t launch_ens_to_work(const float* packed, const int64_t* off, const Explicit2DArgs* inst,
                                int count, float shift, cudaStream_t s);
 cudaError_t launch_ens_from_work(float* packed, const int64_t* off, const Explicit2DArgs* inst,
@@ -144,6 +149,41 @@ cudaError_t launch_to_work(const float* in, float* work, int nx, int ny, float s
                            cudaStream_t s);
 cudaError_t launch_from_work(const float* work, float* out, int nx, int ny, float shift,
                              cudaStream_t s);
+
+// Explicit 2-D trajectories held on chip (k_onchip2d.cu): a job is one mesh, cut
+// into gx x gy tiles of one block each.
+struct OnchipJob {
+  int64_t off;   // first value of the mesh in OnchipArgs::state
+  int nx, ny, gx, gy;
+  float shift;
+  int64_t xchg;  // first packet of the job's exchange region
+  unsigned long long pair[7 + 12];
+};
+struct OnchipItem {
+  int job, tile;
+};
+struct OnchipArgs {
+  float* state;             // in/out
+  OnchipJob job;            // a single mesh
+  const OnchipJob* jobs;    // an ensemble: jobs, and per block list[list_first[b] ..]
+  const OnchipItem* list;
+  const int* list_first;
+  void* xchg;               // zeroed exchange buffer
+  unsigned* err;            // set when a bounded wait ran out
+  long long limit;          // SM cycles of a wait
+  int n_steps;
+};
+// Tile grid for one mesh, its exchange buffer at most `bytes`; false if the
+// mesh does not fit.
+bool onchip_plan(bool ch, size_t bytes, OnchipJob* job);
+size_t onchip_exchange_bytes(bool ch, const OnchipJob& b);
+cudaError_t launch_onchip(bool ch, const OnchipArgs& a, bool iso, bool odd, cudaStream_t s);
+// Tile grids, per-block lists, exchange bytes and shared memory for Allen-Cahn
+// instances (sizes set in jobs); false if one does not fit.
+bool onchip_plan_ensemble(std::vector<OnchipJob>& jobs, std::vector<int>* first,
+                          std::vector<OnchipItem>* list, size_t* exchange, size_t* smem);
+cudaError_t launch_onchip_ensemble(const OnchipArgs& a, size_t smem, bool iso, bool odd,
+                                   cudaStream_t s);
 
 // Energy / mass diagnostics (Eq. 5-6), FP64 accumulation, deterministic.
 struct Energy2DArgs {
