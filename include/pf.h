@@ -138,8 +138,8 @@ pf_status pf_set_params(pf_ctx* ctx, const pf_params* p);
  * Euler steps with the lumped mass, Eq. 12: AC U <- U - dt L r(U)/m;
  * CH c <- c - dt K_M mu / m with m mu = r(c); COUPLED (Eq. 7) c <- c - dt M_c K mu / m
  * with m mu = dE/dc (no c gradient term) and eta <- eta - dt M_eta (dE/deta) / m, both
- * from the start of the step (one fused kernel per step, one launch per step).  2-D: one fused kernel per step
- * (see pf_set_form); 3-D: residual kernel then update.  Enqueues only. */
+ * from the start of the step (one fused kernel per step, replayed from a graph of 64
+ * steps).  2-D: see pf_set_form; 3-D: residual kernel then update.  Enqueues only. */
 pf_status pf_step_explicit(pf_ctx* ctx, float* state, int64_t n_steps);
 
 /* Execution form of the 2-D explicit step (AC and CH without a mobility field;

@@ -6,217 +6,274 @@
 //   mu  = m^-1 sum_q w N_i [f_a'(c) (1 - h) + f_b'(c) h]          (no c gradient term)
 //   c'  = c - dt M_c m^-1 K mu
 //   eta' = eta - dt M_eta m^-1 (sum_q w N_i (f_b(c) - f_a(c)) h'(eta) + kappa K eta)
-// One block per 32 x 16 node tile: c and eta are staged with a 2-node halo
-// (mirror images beyond the mesh reproduce the zero-flux operators divided by
-// the lumped mass), the per-element Gauss-point terms of both equations are
-// projected to the element corners, mu is gathered on the tile plus a 1-node
-// ring, and both updates are written in one pass: c, mu and eta never make a
-// round trip through HBM.  c is carried as the shift d = c - s (the polynomials
-// in d come expanded from the host), eta as is.
+//
+// A warp sweeps a band of rows down a strip of 64 columns (60 written, a pair
+// per lane), both fields in a sliding register window, as k_explicit2d does for
+// one field (sweep2d.h: values at Gauss points without their factor g_hi^2, in
+// packed FP32); mu never leaves the registers, and neighbouring columns come by
+// shuffles.  What binds it is the FP32 pipe: 111 packed and 16 scalar operations
+// per row of 64 columns, 84 of them the polynomials at the four points:
+//   f_a' (cubic), f_b' - f_a' (cubic), f_b - f_a (quartic) by Horner's rule in
+//   c, h = eta^3 (10 - 15 eta + 6 eta^2), h' = 30 (eta - eta^2)^2,
+// all expanded on the host in FP64 with the interpolation's factors, h' with
+// the weights and -dt M_eta.  Rows that only fill the window leave out what
+// later rows do not need (eta's terms above and below the band).
+// The working planes carry a mirror frame like k_explicit2d's.
+//
+// Measured at 2048^2 (us per step, graph replay): 49.3 with 32 x 16 node tiles
+// in shared memory, an element pass into corner arrays and gathers from them,
+// bound by index arithmetic and shared-memory addressing; 28.0 so, the FMA pipe
+// 70 % busy while SMs work (94 registers, 20 warps per SM; held to 80 or 72
+// registers the kernel spills: 31 to 34).
+#include <string.h>
+
 #include "pf_internal.h"
+#include "sweep2d.h"
 
 namespace pf {
 namespace {
 
-#ifndef PF_CPL_TY
-#define PF_CPL_TY 16
-#endif
-#ifndef PF_CPL_THREADS
-#define PF_CPL_THREADS 256
-#endif
-constexpr int TX = 32, TY = PF_CPL_TY;     // output tile
-constexpr int kThreads = PF_CPL_THREADS;
-constexpr int S2X = TX + 4, S2Y = TY + 4;  // nodes with a 2-node halo
-constexpr int EX = TX + 3, EY = TY + 3;    // elements touching the 1-halo nodes
+using namespace sweep;
 
-// Single mirror image about the end nodes, then clamped into the mesh: exact
-// for the 2-node halo of stored nodes (the coupled model needs at least 3
-// nodes per axis);
-// positions further out (the far side of a ragged last tile) only feed
-// outputs that are not stored, and the clamp keeps their loads in bounds.
-__device__ __forceinline__ int reflect(int k, int n) {
-  k = k < 0 ? -k : k;
-  k = k >= n ? 2 * (n - 1) - k : k;
-  return k < 0 ? 0 : (k >= n ? n - 1 : k);
-}
+constexpr int kWarps = 2;   // warps per block, stacked in y
+constexpr int kAhead = 3;   // rows of both planes in flight, and the loop's unrolling
 
-
-__device__ __forceinline__ float gpt(int i) { return i ? kGHi : kGLo; }
-
-struct __align__(16) Tile {  // 8-byte aligned rows of c, e and mu (36 floats)
-  float c[S2Y][S2X];      // shifted composition, 2-halo
-  float e[S2Y][S2X];      // order parameter, 2-halo
-  float mu[S2Y][S2X];     // chemical potential on the 1-halo nodes (same indexing)
-  float Ec[4][EY][EX];    // per-element corner terms of mu
-  float Ee[4][EY][EX];    // per-element corner terms of the eta residual
+struct Window {
+  u64 c1, c2, e1, e2, x1, x2;    // rows k-1, k-2; row helpers of eta
+  u64 amc, apc, ame, ape;        // x-interpolants of row k-1
+  u64 tlc, thc, tle, the;        // element row k-2: its share of node row k-1
+  u64 mua, mub, mxa, mxb;        // mu of rows k-3, k-2 and helpers
 };
 
-typedef unsigned long long u64;  // packed FP32 pair: the two x Gauss points of a row
+// Packed constants (pack_coupled2d)
+struct Coef {
+  const u64* c;
+  __device__ __forceinline__ u64 rho() const { return c[0]; }
+  __device__ __forceinline__ u64 g2() const { return c[1]; }            // -g_hi^2
+  __device__ __forceinline__ u64 p(int i) const { return c[2 + i]; }    // f_a'
+  __device__ __forceinline__ u64 q(int i) const { return c[6 + i]; }    // f_b' - f_a'
+  __device__ __forceinline__ u64 r(int i) const { return c[10 + i]; }   // f_b - f_a
+  __device__ __forceinline__ u64 h(int i) const { return c[15 + i]; }   // h / eta^3
+  __device__ __forceinline__ u64 k(int stage, int i) const { return c[18 + 6 * stage + i]; }
+};
 
-__device__ __forceinline__ u64 pk(float lo, float hi) {
-  u64 r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-  return r;
-}
-__device__ __forceinline__ float plo(u64 v) {
-  float l;
-  asm("{ .reg .f32 t; mov.b64 {%0, t}, %1; }" : "=f"(l) : "l"(v));
-  return l;
-}
-__device__ __forceinline__ float phi(u64 v) {
-  float h;
-  asm("{ .reg .f32 t; mov.b64 {t, %0}, %1; }" : "=f"(h) : "l"(v));
-  return h;
-}
-__device__ __forceinline__ u64 fma2(u64 a, u64 b, u64 c) {
-  u64 d;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-  return d;
-}
-__device__ __forceinline__ u64 add2(u64 a, u64 b) {
-  u64 d;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-__device__ __forceinline__ u64 sub2(u64 a, u64 b) {
-  u64 d;
-  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-__device__ __forceinline__ u64 mul2(u64 a, u64 b) {
-  u64 d;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-__device__ __forceinline__ u64 bc(float v) { return pk(v, v); }
+// How far a row goes: its interpolation; c's element row; node row k-1 of c
+// and eta's element row; eta's finished row k-1; c's finished row k-2; and
+// past eta's band, c alone.
+enum Stage { kStart, kElementC, kNodeC, kFirst, kBoth, kOnlyC };
 
-// Horner evaluation of sum_k a[k] x^k (N coefficients) on a packed pair
-template <int N>
-__device__ __forceinline__ u64 horner2(const float* a, u64 x) {
-  u64 s = bc(a[N - 1]);
-#pragma unroll
-  for (int k = N - 2; k >= 0; --k) s = fma2(s, x, bc(a[k]));
-  return s;
-}
-
-__global__ void __launch_bounds__(kThreads) k_coupled2d(const Coupled2DArgs a) {
-  __shared__ Tile T;
-  const int tiles_x = (a.nx + TX - 1) / TX;
-  const int x0 = (blockIdx.x % tiles_x) * TX, y0 = (blockIdx.x / tiles_x) * TY;
-  const int64_t N = (int64_t)a.nx * a.ny;
-
-  for (int i = threadIdx.x; i < S2X * S2Y; i += kThreads) {
-    const int lx = i % S2X, ly = i / S2X;
-    const int64_t g = (int64_t)reflect(y0 - 2 + ly, a.ny) * a.nx + reflect(x0 - 2 + lx, a.nx);
-    T.c[ly][lx] = a.in[g];
-    T.e[ly][lx] = a.in[N + g];
+// f_a' + (f_b' - f_a') h, and (f_b - f_a) h' up to constant factors, at one
+// Gauss point of both columns
+template <bool kEta>
+__device__ __forceinline__ void point(u64 d, u64 n, const Coef& K, u64& gc, u64& ge) {
+  const u64 n2 = mul2(n, n);
+  const u64 h = mul2(mul2(n2, n), fma2(fma2(K.h(2), n, K.h(1)), n, K.h(0)));
+  const u64 q = fma2(fma2(fma2(K.q(3), d, K.q(2)), d, K.q(1)), d, K.q(0));
+  const u64 p = fma2(fma2(fma2(K.p(3), d, K.p(2)), d, K.p(1)), d, K.p(0));
+  gc = fma2(q, h, p);
+  if constexpr (kEta) {
+    const u64 r = fma2(fma2(fma2(fma2(K.r(4), d, K.r(3)), d, K.r(2)), d, K.r(1)), d, K.r(0));
+    const u64 w = fma2(K.g2(), n2, n);  // eta (1 - eta), without one factor
+    ge = mul2(r, mul2(w, w));
   }
-  __syncthreads();
+}
 
-  // elements (ex, ey) with lower-left node (ex, ey) in 2-halo coordinates, for
-  // the elements that touch the 1-halo nodes: ex, ey in [0, EX), [0, EY).
-  // The two Gauss points of a row (xi = g_lo, g_hi) travel as one packed
-  // pair, so every interpolation and polynomial is one f32x2 instruction
-  // for two points; rows qy = 0, 1 are the pairs P[0], P[1].
-  const u64 X = pk(kGLo, kGHi);
-  for (int i = threadIdx.x; i < EX * EY; i += kThreads) {
-    const int ex = i % EX, ey = i / EX;
-    const float c0 = T.c[ey][ex], c1 = T.c[ey][ex + 1], c2 = T.c[ey + 1][ex], c3 = T.c[ey + 1][ex + 1];
-    const float e0 = T.e[ey][ex], e1 = T.e[ey][ex + 1], e2 = T.e[ey + 1][ex], e3 = T.e[ey + 1][ex + 1];
-    // bottom and top rows at the two x Gauss points, then the two y Gauss points
-    const u64 cb = fma2(X, bc(c1 - c0), bc(c0)), ct = fma2(X, bc(c3 - c2), bc(c2));
-    const u64 eb = fma2(X, bc(e1 - e0), bc(e0)), etp = fma2(X, bc(e3 - e2), bc(e2));
-    const u64 dc = sub2(ct, cb), de = sub2(etp, eb);
-    u64 gc[2], ge[2];
-#pragma unroll
-    for (int qy = 0; qy < 2; ++qy) {
-      const u64 et = bc(gpt(qy));
-      const u64 d = fma2(et, dc, cb);   // shifted c at the row's two Gauss points
-      const u64 n = fma2(et, de, eb);   // eta there
-      const u64 h = horner2<6>(a.h, n), dh = horner2<5>(a.dh, n);
-      const u64 dfa = horner2<4>(a.dfa, d), dfb = horner2<2>(a.dfb, d);
-      const u64 fa = horner2<5>(a.fa, d), fb = horner2<3>(a.fb, d);
-      gc[qy] = fma2(h, sub2(dfb, dfa), dfa);  // f_a' (1 - h) + f_b' h
-      ge[qy] = mul2(sub2(fb, fa), dh);
+// x-interpolants of a row (scalar FMAs, see sweep2d.h)
+__device__ __forceinline__ void interpolate(u64 P, float right, float rho, u64& am, u64& ap) {
+  const float v0 = plo(P), v1 = phi(P);
+  am = pk(fmaf(rho, v1, v0), fmaf(rho, right, v1));
+  ap = pk(fmaf(rho, v0, v1), fmaf(rho, v1, right));
+}
+
+// weights back in x: the share of the left neighbour comes from its lane
+__device__ __forceinline__ u64 back(u64 sl, u64 sh, const Coef& K) {
+  const u64 A = fma2(K.rho(), sh, sl), B = fma2(K.rho(), sl, sh);
+  const float bl = __shfl_up_sync(kFull, phi(B), 1);
+  return pk(plo(A) + bl, phi(A) + plo(B));
+}
+
+template <bool kIso>
+__device__ __forceinline__ u64 helper(u64 v, float r) {  // r: the column right of the lane's
+  const float l = __shfl_up_sync(kFull, phi(v), 1);
+  const u64 hs = pk(l + phi(v), plo(v) + r);
+  return kIso ? add2(v, hs) : hs;
+}
+
+// init + K v at the centre row
+template <bool kIso>
+__device__ __forceinline__ u64 apply(u64 init, u64 s, u64 c, u64 n, u64 as, u64 ac, u64 an,
+                                     const Coef& K, int st) {
+  if constexpr (kIso) return fma2(K.k(st, 1), add2(add2(as, an), ac), fma2(K.k(st, 0), c, init));
+  return fma2(K.k(st, 5), add2(as, an),
+              fma2(K.k(st, 4), add2(s, n), fma2(K.k(st, 3), ac, fma2(K.k(st, 2), c, init))));
+}
+
+// Consumes row k: c and eta in C and E.  oe: eta's finished row k-1 (from
+// kFirst on, not kOnlyC); oc: c's finished row k-2 (kBoth, kOnlyC).
+template <bool kIso, int kStage>
+__device__ __forceinline__ void row(u64 C, u64 E, Window& w, const Coef& K, u64& oc, u64& oe) {
+  constexpr bool kEta = kStage >= kNodeC && kStage <= kBoth;   // eta's element row
+  constexpr bool kEtaOut = kStage == kFirst || kStage == kBoth;
+  const float rho = plo(K.rho());
+  u64 amc, apc, ame, ape;
+  interpolate(C, __shfl_down_sync(kFull, plo(C), 1), rho, amc, apc);
+  const float er = __shfl_down_sync(kFull, plo(E), 1);
+  interpolate(E, er, rho, ame, ape);
+  u64 xe = 0;
+  if constexpr (kStage != kOnlyC) xe = helper<kIso>(E, er);
+  if constexpr (kStage >= kElementC) {
+    u64 gc[4], ge[4];  // (low x, low y), (low, high), (high, low), (high, high)
+    point<kEta>(fma2(K.rho(), amc, w.amc), fma2(K.rho(), ame, w.ame), K, gc[0], ge[0]);
+    point<kEta>(fma2(K.rho(), w.amc, amc), fma2(K.rho(), w.ame, ame), K, gc[1], ge[1]);
+    point<kEta>(fma2(K.rho(), apc, w.apc), fma2(K.rho(), ape, w.ape), K, gc[2], ge[2]);
+    point<kEta>(fma2(K.rho(), w.apc, apc), fma2(K.rho(), w.ape, ape), K, gc[3], ge[3]);
+    if constexpr (kStage >= kNodeC) {
+      const u64 sl = add2(fma2(K.rho(), gc[1], gc[0]), w.tlc);
+      const u64 sh = add2(fma2(K.rho(), gc[3], gc[2]), w.thc);
+      const u64 mu = back(sl, sh, K);
+      const u64 mx = helper<kIso>(mu, __shfl_down_sync(kFull, plo(mu), 1));
+      if constexpr (kStage >= kBoth)
+        oc = apply<kIso>(w.c2, w.mua, w.mub, mu, w.mxa, w.mxb, mx, K, 1);
+      w.mua = w.mub;
+      w.mxa = w.mxb;
+      w.mub = mu;
+      w.mxb = mx;
     }
-    // 1/4 sum_q v_q N_a(q): the Gauss weight |cell|/4 over the interior mass
-    // |cell|, folded into the packed weights N_a of the two x points per row
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      const float wlo = (c & 1) ? kGLo : 1.0f - kGLo, whi = (c & 1) ? kGHi : 1.0f - kGHi;
-      const float y0 = 0.25f * ((c >> 1) ? kGLo : 1.0f - kGLo);
-      const float y1 = 0.25f * ((c >> 1) ? kGHi : 1.0f - kGHi);
-      const u64 w0 = pk(wlo * y0, whi * y0), w1 = pk(wlo * y1, whi * y1);
-      const u64 sc = fma2(w1, gc[1], mul2(w0, gc[0]));
-      const u64 se = fma2(w1, ge[1], mul2(w0, ge[0]));
-      T.Ec[c][ey][ex] = plo(sc) + phi(sc);
-      T.Ee[c][ey][ex] = plo(se) + phi(se);
+    if constexpr (kEtaOut) {
+      const u64 sl = add2(fma2(K.rho(), ge[1], ge[0]), w.tle);
+      const u64 sh = add2(fma2(K.rho(), ge[3], ge[2]), w.the);
+      const u64 F = back(sl, sh, K);
+      oe = apply<kIso>(add2(w.e1, F), w.e2, w.e1, E, w.x2, w.x1, xe, K, 0);
     }
-  }
-  __syncthreads();
-
-  // mu on the tile and its 1-node ring: node (y, x) in 2-halo coordinates,
-  // y in [1, TY + 3), x in [1, TX + 3); its elements have lower-left corners
-  // (y - ay, x - ax), ay, ax in {0, 1}
-  for (int i = threadIdx.x; i < (TX + 2) * (TY + 2); i += kThreads) {
-    const int x = 1 + i % (TX + 2), y = 1 + i / (TX + 2);
-    T.mu[y][x] = T.Ec[0][y][x] + T.Ec[1][y][x - 1] + T.Ec[2][y - 1][x] + T.Ec[3][y - 1][x - 1];
-  }
-  __syncthreads();
-
-  // the updates, two adjacent nodes (x, x+1) per thread: one 64-bit load
-  // fetches a row's pair and two scalars its outer neighbours, and the 9-point
-  // stencils of mu and eta run on packed pairs
-  for (int i = threadIdx.x; i < TX * TY / 2; i += kThreads) {
-    const int lx = 2 * (i % (TX / 2)), ly = i / (TX / 2);
-    const int gx = x0 + lx, gy = y0 + ly;
-    if (gx >= a.nx || gy >= a.ny) continue;
-    const int x = lx + 2, y = ly + 2;  // x even: the pair is 8-byte aligned
-    // packed 9-point stencil on rows y-1 .. y+1 of a 36-wide plane; ctr_out
-    // receives the centre pair of row y
-    auto stencil_pair = [&](const float (*V)[S2X], const Stencil2D& k, u64& ctr_out) {
-      u64 ctr[3], hs[3];
-#pragma unroll
-      for (int r = 0; r < 3; ++r) {
-        const u64 P = *reinterpret_cast<const u64*>(&V[y - 1 + r][x]);
-        const float l = V[y - 1 + r][x - 1], rr = V[y - 1 + r][x + 2];
-        ctr[r] = P;
-        hs[r] = pk(l + phi(P), plo(P) + rr);  // west + east of each node
-      }
-      ctr_out = ctr[1];
-      u64 o = mul2(bc(k.c0), ctr[1]);
-      o = fma2(bc(k.cx), hs[1], o);
-      o = fma2(bc(k.cy), add2(ctr[0], ctr[2]), o);
-      return fma2(bc(k.cd), add2(hs[0], hs[2]), o);
-    };
-    u64 centre, e_c;
-    const u64 lap_mu = stencil_pair(T.mu, a.k2, centre);  // -dt M_c / m K mu
-    const u64 lap_e = stencil_pair(T.e, a.k1, e_c);       // kappa / m K eta (e_c: eta itself)
-    // element terms of the eta residual around each node (rows of 35: scalar)
-    const float re0 = T.Ee[0][y][x] + T.Ee[1][y][x - 1] + T.Ee[2][y - 1][x] + T.Ee[3][y - 1][x - 1];
-    const float re1 = T.Ee[0][y][x + 1] + T.Ee[1][y][x] + T.Ee[2][y - 1][x + 1] + T.Ee[3][y - 1][x];
-    const u64 re = add2(pk(re0, re1), lap_e);
-    const u64 cc = *reinterpret_cast<const u64*>(&T.c[y][x]);
-    const u64 oc = add2(cc, lap_mu);
-    const u64 oe = fma2(bc(a.neg_dt_meta), re, e_c);
-    const int64_t g = (int64_t)gy * a.nx + gx;
-    a.out[g] = plo(oc);
-    a.out[N + g] = plo(oe);
-    if (gx + 1 < a.nx) {
-      a.out[g + 1] = phi(oc);
-      a.out[N + g + 1] = phi(oe);
+    w.tlc = fma2(K.rho(), gc[0], gc[1]);
+    w.thc = fma2(K.rho(), gc[2], gc[3]);
+    if constexpr (kEta) {
+      w.tle = fma2(K.rho(), ge[0], ge[1]);
+      w.the = fma2(K.rho(), ge[2], ge[3]);
     }
   }
+  w.c2 = w.c1;
+  w.c1 = C;
+  w.e2 = w.e1;
+  w.e1 = E;
+  w.x2 = w.x1;
+  w.x1 = xe;
+  w.amc = amc;
+  w.apc = apc;
+  w.ame = ame;
+  w.ape = ape;
+}
+
+// kTY: output rows per band, 1 + a multiple of kAhead
+template <bool kIso, int kTY>
+__global__ void __launch_bounds__(kWarps * 32) k_coupled2d(const Coupled2DArgs a) {
+  static_assert((kTY - 1) % kAhead == 0, "the loop takes kAhead rows at a time");
+  const int lane = threadIdx.x & 31;
+  const int y0 = (block_row() * kWarps + (threadIdx.x >> 5)) * kTY;
+  const int nx = a.nx, ny = a.ny;
+  if (y0 >= ny) return;
+  const Coef K{a.pair};
+  const int64_t pitch = a.pitch, plane = a.plane;
+  const int x = blockIdx.x * kOutCols - kPair + kPair * lane;  // real column of the low half
+  const bool writer = lane >= 1 && lane <= 30 && x < nx;
+  const bool plain = writer && x > 2 && x + 1 < nx - 3 && y0 > 2 && y0 + kTY + 3 < ny;
+  const float* src = a.in + (int64_t)(y0 - 2 + kGhost) * pitch + kGhost + x;
+  float* const out0 = a.out + kGhost * pitch + kGhost;
+  u64 nc[kAhead], ne[kAhead];  // rows in flight
+  const auto load = [&](int j) {
+    nc[j] = __ldg(reinterpret_cast<const u64*>(src));
+    ne[j] = __ldg(reinterpret_cast<const u64*>(src + plane));
+    src += pitch;
+  };
+#pragma unroll
+  for (int j = 0; j < kAhead; ++j) load(j);
+  Window w;
+  u64 oc, oe;
+  const auto consume = [&](auto stage, int j) {  // j: rows consumed before, modulo kAhead
+    const u64 C = nc[j], E = ne[j];
+    load(j);  // past the band's last row: not used
+    row<kIso, decltype(stage)::value>(C, E, w, K, oc, oe);
+  };
+  const auto store = [&](float* p, int y, u64 v) {
+    if (plain)
+      *reinterpret_cast<u64*>(p + (int64_t)y * pitch + x) = v;
+    else if (writer && y < ny)
+      store_out(p, pitch, y, ny, x, nx, v);
+  };
+  consume(std::integral_constant<int, kStart>{}, 0);
+  consume(std::integral_constant<int, kElementC>{}, 1);
+  consume(std::integral_constant<int, kNodeC>{}, 2);
+  consume(std::integral_constant<int, kFirst>{}, 0);
+  store(out0 + plane, y0, oe);
+#pragma unroll 1
+  for (int i = 1; i < kTY; i += kAhead) {
+#pragma unroll
+    for (int j = 0; j < kAhead; ++j) {
+      consume(std::integral_constant<int, kBoth>{}, (1 + j) % kAhead);
+      store(out0, y0 + i + j - 1, oc);
+      store(out0 + plane, y0 + i + j, oe);
+    }
+  }
+  consume(std::integral_constant<int, kOnlyC>{}, 1);
+  store(out0, y0 + kTY - 1, oc);
 }
 
 }  // namespace
 
-cudaError_t launch_coupled2d(const Coupled2DArgs& a, cudaStream_t s) {
-  const int tiles = ((a.nx + TX - 1) / TX) * ((a.ny + TY - 1) / TY);
-  k_coupled2d<<<tiles, kThreads, 0, s>>>(a);
-  return cudaGetLastError();
+void pack_coupled2d(const CoupledPoly& f, double neg_dt_meta, Coupled2DArgs& a) {
+  auto two = [](double v) {
+    const float x = (float)v;
+    unsigned int b;
+    memcpy(&b, &x, 4);
+    return (unsigned long long)b | ((unsigned long long)b << 32);
+  };
+  // a value at a Gauss point is g2 times the one carried, and so is the weight
+  // back; the Gauss weight is |cell|/4 over the interior mass |cell|
+  const double g2 = (double)kGHi * kGHi, wt = 0.25 * g2;
+  double s = 1.0;
+  a.pair[0] = two((double)kGLo / kGHi);
+  a.pair[1] = two(-g2);
+  for (int i = 0; i < 5; ++i, s *= g2) {
+    const double dfa = i < 4 ? (i + 1) * f.fa[i + 1] : 0.0;
+    const double dfb = i < 2 ? (i + 1) * f.fb[i + 1] : 0.0;
+    const double fb = i < 3 ? f.fb[i] : 0.0;
+    if (i < 4) a.pair[2 + i] = two(wt * s * dfa);
+    if (i < 4) a.pair[6 + i] = two(wt * s * (dfb - dfa));
+    // h' = 30 (eta - eta^2)^2, eta - eta^2 carried without one factor g2
+    a.pair[10 + i] = two(neg_dt_meta * 30.0 * g2 * g2 * wt * s * (fb - f.fa[i]));
+  }
+  const double h[3] = {10.0, -15.0, 6.0};
+  s = g2 * g2 * g2;
+  for (int i = 0; i < 3; ++i, s *= g2) a.pair[15 + i] = two(h[i] * s);
+  const Stencil2D* st[2] = {&a.k1, &a.k2};
+  for (int k = 0; k < 2; ++k) {
+    const double v[6] = {(double)st[k]->c0 - st[k]->cd, st[k]->cd, st[k]->c0,
+                         st[k]->cx, st[k]->cy, st[k]->cd};
+    for (int i = 0; i < 6; ++i) a.pair[18 + 6 * k + i] = two(v[i]);
+  }
 }
 
-size_t coupled2d_smem_bytes() { return sizeof(Tile); }
+namespace {
+template <bool kIso, int kTY>
+cudaError_t launch(const Coupled2DArgs& a, cudaStream_t s) {
+  const dim3 grid = row_grid((a.nx + kOutCols - 1) / kOutCols,
+                             (a.ny + kWarps * kTY - 1) / (kWarps * kTY));
+  k_coupled2d<kIso, kTY><<<grid, kWarps * 32, 0, s>>>(a);
+  return cudaGetLastError();
+}
+}  // namespace
+
+// Bands of 4 rows while 7-row bands would not fill the SMs twice (20 warps of
+// them fit), 7 beyond: us per step at 64^2 / 515 x 1031 / 1024^2 / 2048^2 with
+// 4 rows 3.8 / 6.9 / 10.4 / 30.6, with 7 rows 5.7 / 8.3 / 11.2 / 28.0, with 13
+// rows 9.0 / 11.1 / 12.7 / 28.6.
+cudaError_t launch_coupled2d(const Coupled2DArgs& a, cudaStream_t s) {
+  const auto iso = [](const Stencil2D& k) { return k.cx == k.cd && k.cy == k.cd; };
+  const bool both = iso(a.k1) && iso(a.k2);
+  const int64_t warps = (int64_t)((a.nx + kOutCols - 1) / kOutCols) * ((a.ny + 6) / 7);
+  if (warps < 40 * (int64_t)device_sm_count())
+    return both ? launch<true, 4>(a, s) : launch<false, 4>(a, s);
+  return both ? launch<true, 7>(a, s) : launch<false, 7>(a, s);
+}
 
 }  // namespace pf

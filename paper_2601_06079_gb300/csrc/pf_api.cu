@@ -265,6 +265,12 @@ struct CallGraphs {
 };
 
 cudaError_t launch_step(pf_ctx* c, const float* in, float* out, cudaStream_t s) {
+  if (c->model == PF_MODEL_COUPLED) {
+    pf::Coupled2DArgs a = c->cp;
+    a.in = in;
+    a.out = out;
+    return pf::launch_coupled2d(a, s);
+  }
   pf::Explicit2DArgs a = c->ex;
   a.in = in;
   a.out = out;
@@ -787,45 +793,44 @@ void shift_poly(const double* a, int n, double s, double* out) {
 void set_params_coupled(pf_ctx* c, const pf_params* p) {
   static const double fa[5] = {-1.6704, -4.776, 5.1622, -2.7375, 1.3687};
   static const double fb[3] = {-1.5924, -5.9746, 5.0};
-  static const double h[6] = {0.0, 0.0, 0.0, 10.0, -15.0, 6.0};
   pf::Coupled2DArgs& a = c->cp;
   a.nx = (int)c->n[0];
   a.ny = (int)c->n[1];
-  double sa[5], sb[3];
-  shift_poly(fa, 5, p->shift, sa);
-  shift_poly(fb, 3, p->shift, sb);
-  for (int k = 0; k < 5; ++k) a.fa[k] = (float)sa[k];
-  for (int k = 0; k < 4; ++k) a.dfa[k] = (float)((k + 1) * sa[k + 1]);
-  for (int k = 0; k < 3; ++k) a.fb[k] = (float)sb[k];
-  for (int k = 0; k < 2; ++k) a.dfb[k] = (float)((k + 1) * sb[k + 1]);
-  for (int k = 0; k < 6; ++k) a.h[k] = (float)h[k];
-  for (int k = 0; k < 5; ++k) a.dh[k] = (float)((k + 1) * h[k + 1]);
-  const double hx = c->h[0], hy = c->h[1], m = hx * hy;
-  a.k1 = stiffness2d(hx, hy, p->kappa / m);
+  a.pitch = pf::work_pitch(a.nx);
+  a.plane = a.pitch * pf::work_rows(a.ny);
+  pf::CoupledPoly f;
+  shift_poly(fa, 5, p->shift, f.fa);
+  shift_poly(fb, 3, p->shift, f.fb);
+  const double hx = c->h[0], hy = c->h[1], m = hx * hy, neg = -p->dt * p->mobility2;
+  a.k1 = stiffness2d(hx, hy, neg * p->kappa / m);
   a.k2 = stiffness2d(hx, hy, -p->dt * p->mobility / m);
-  a.neg_dt_meta = (float)(-p->dt * p->mobility2);
+  pf::pack_coupled2d(f, neg, a);
 }
 
-// The coupled step: working planes [c - shift; eta] without a frame in buf_a /
-// buf_b (ping-pong), one fused launch per step.
+// The coupled step: framed working planes [c - shift; eta] in buf_a / buf_b
+// (ping-pong), one fused launch per step, replayed from graphs of kGraphSteps.
 pf_status step_coupled2d(pf_ctx* c, float* state, int64_t n_steps) {
-  const int64_t N = nodes2d(c);
+  const int64_t N = nodes2d(c), plane = c->cp.plane;
+  const int nx = (int)c->n[0], ny = (int)c->n[1];
   const float shift = (float)c->par.shift;
+  for (float* buf : {c->buf_a, c->buf_b}) {
+    PF_CUDA(pf::launch_to_work(state, buf, nx, ny, shift, c->stream));
+    PF_CUDA(pf::launch_to_work(state + N, buf + plane, nx, ny, 0.0f, c->stream));
+  }
+  int64_t left = n_steps;
+  if (left >= kGraphSteps) {
+    pf_status st = ensure_graph(c);
+    if (st != PF_OK) return st;
+    for (; left >= kGraphSteps; left -= kGraphSteps) PF_CUDA(cudaGraphLaunch(c->graph, c->stream));
+  }
   float* cur = c->buf_a;
   float* oth = c->buf_b;
-  PF_CUDA(pf::launch_add(state, cur, N, -shift, c->stream));
-  PF_CUDA(cudaMemcpyAsync(cur + N, state + N, sizeof(float) * N, cudaMemcpyDeviceToDevice,
-                          c->stream));
-  pf::Coupled2DArgs a = c->cp;
-  for (int64_t s = 0; s < n_steps; ++s) {
-    a.in = cur;
-    a.out = oth;
-    PF_CUDA(pf::launch_coupled2d(a, c->stream));
+  for (; left > 0; --left) {
+    PF_CUDA(launch_step(c, cur, oth, c->stream));
     std::swap(cur, oth);
   }
-  PF_CUDA(pf::launch_add(cur, state, N, shift, c->stream));
-  PF_CUDA(cudaMemcpyAsync(state + N, cur + N, sizeof(float) * N, cudaMemcpyDeviceToDevice,
-                          c->stream));
+  PF_CUDA(pf::launch_from_work(cur, state, nx, ny, shift, c->stream));
+  PF_CUDA(pf::launch_from_work(cur + plane, state + N, nx, ny, 0.0f, c->stream));
   return PF_OK;
 }
 

@@ -104,17 +104,22 @@ constexpr int kL2StreamHalf = 2;  // evict_first for half of the lines, the rest
 
 cudaError_t launch_ac2d(const Explicit2DArgs& a, cudaStream_t s);
 
-// Coupled Allen-Cahn / Cahn-Hilliard step (planes [c - shift; eta], no frame).
+// Coupled Allen-Cahn / Cahn-Hilliard step (framed planes [c - shift; eta] like
+// the single-field step's, `plane` floats apart).
 struct Coupled2DArgs {
   const float* in;
   float* out;
   int nx, ny;
-  float fa[5], dfa[4], fb[3], dfb[2];  // f_alpha, f_beta and derivatives in d = c - shift
-  float h[6], dh[5];                   // h(eta), h'(eta)
-  Stencil2D k1;                        // kappa_eta / m K
-  Stencil2D k2;                        // -dt M_c / m K
-  float neg_dt_meta;                   // -dt M_eta
+  int64_t pitch, plane;
+  Stencil2D k1;  // -dt M_eta kappa_eta / m K
+  Stencil2D k2;  // -dt M_c / m K
+  unsigned long long pair[30];  // packed constants (pack_coupled2d)
 };
+// f_alpha and f_beta in d = c - shift, increasing powers
+struct CoupledPoly {
+  double fa[5], fb[3];
+};
+void pack_coupled2d(const CoupledPoly& f, double neg_dt_meta, Coupled2DArgs& a);
 cudaError_t launch_coupled2d(const Coupled2DArgs& a, cudaStream_t s);
 // The plain two-pass comparison form (d, mu, out: nx x ny arrays without frame).
 cudaError_t launch_plain2d(bool ch, const Explicit2DArgs& a, const float* d, float* mu, float* out,

@@ -222,5 +222,40 @@ __device__ __forceinline__ void row(const u64 (&P)[kP], float cl, float cr, floa
   }
 }
 
+// Planes with a mirror frame (k_explicit2d.cu, k_coupled2d.cu): a warp takes 64
+// columns, a pair per lane, and writes the 60 of lanes 1..30.
+constexpr int kPair = 2;                          // columns per lane
+constexpr int kOutCols = 32 * kPair - 2 * kPair;  // 60 output columns per warp
+constexpr int kGhost = 2;                         // width of the frame
+
+// Output of one finished pair: real row y, real columns x (lo) and x+1 (hi),
+// plus every ghost cell that mirrors it (rows -1, -2 <- 1, 2 and
+// ny, ny+1 <- ny-2, ny-3; the same for columns), so the next step reads the
+// mirror extension without any index reflection.
+__device__ __forceinline__ void store_cols(float* __restrict__ row, int x, int nx, u64 v) {
+  const float lo = plo(v), hi = phi(v);
+  if (x + 1 < nx) {
+    *reinterpret_cast<u64*>(row + x) = v;
+  } else {
+    row[x] = lo;
+  }
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int xc = x + h;
+    const float val = h ? hi : lo;
+    if (xc >= nx) break;
+    if (xc == 1 || xc == 2) row[-xc] = val;
+    if (xc == nx - 2 || xc == nx - 3) row[2 * (nx - 1) - xc] = val;
+  }
+}
+
+__device__ __forceinline__ void store_out(float* __restrict__ base0, int64_t pitch, int y, int ny,
+                                          int x, int nx, u64 v) {
+  store_cols(base0 + (int64_t)y * pitch, x, nx, v);
+  if (y == 1 || y == 2) store_cols(base0 - (int64_t)y * pitch, x, nx, v);
+  if ((y == ny - 2 || y == ny - 3) && y >= 0)
+    store_cols(base0 + (int64_t)(2 * (ny - 1) - y) * pitch, x, nx, v);
+}
+
 }  // namespace sweep
 }  // namespace pf
