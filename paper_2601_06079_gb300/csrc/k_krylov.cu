@@ -1,11 +1,13 @@
 // Vector kernels of the Newton-GMRES solver (JAX-PF Eq. 13-14).  The Krylov
 // basis is FP32; every inner product and norm keeps about 48 bits per thread
 // and finishes in FP64: each thread forms FP32 sums over 8 consecutive
-// products and adds them into a compensated FP32 pair (hi + lo, Knuth's
-// two-sum), warps combine the pairs the same way and blocks add the warps'
+// products (4 in the projections) and adds them into a compensated FP32 pair
+// (hi + lo, Knuth's two-sum), warps combine the pairs the same way and blocks add the warps'
 // values in FP64, and the last block sums the per-block partials in a fixed
 // order, so results are deterministic.  No FP64 arithmetic runs per element: GB300 issues about 2
 // FP64 operations per clock per SM, 64 times fewer than FP32.
+#include <type_traits>
+
 #include "pf_internal.h"
 
 namespace pf {
@@ -34,22 +36,18 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
-// Block-wide FP64 sum; the result is valid in thread 0.
-__device__ double block_sum(double v, double* scratch) {
-  v = warp_sum(v);
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  __syncthreads();
-  if (l == 0) scratch[w] = v;
-  __syncthreads();
-  v = (threadIdx.x < kThreads / 32) ? scratch[threadIdx.x] : 0.0;
-  if (w == 0) v = warp_sum(v);
-  return v;
-}
+// The reductions' last stages.  warp_value: the warp's sum of accumulator j
+// into shared memory (no block barrier per vector); then finish_sums: the
+// block's sums into partials[j * blocks + b], and the last block to finish adds
+// all blocks' partials into out[j], a warp per vector, in a fixed order (blocks
+// in steps of 32 per lane, then a tree), so one launch gives the final,
+// repeatable values.  count: device counter, 0 before the launch and reset to
+// 0 by the last block.  (With two barriers per vector and block, and the last
+// block taking the vectors one after another, 8 products of 4,096 values took
+// 16.5 us, nearly all of it here; now 4.)
+constexpr int kWarpsPerBlock = kThreads / 32;
 
-// Block-wide sum of the threads' compensated pairs, valid in thread 0: the
-// warp tree combines pairs in FP32 (two-sum, the low parts added), only the
-// warps' values are summed in FP64 (a tree in warp 0), in a fixed order.
-__device__ double block_sum2(Acc2 a, double* scratch) {
+__device__ __forceinline__ void warp_value(Acc2 a, int j, double (*sums)[kWarpsPerBlock]) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     const float h = __shfl_down_sync(0xffffffffu, a.hi, o);
@@ -57,37 +55,35 @@ __device__ double block_sum2(Acc2 a, double* scratch) {
     a.add(h);
     a.lo += l;
   }
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  __syncthreads();
-  if (l == 0) scratch[w] = a.value();
-  __syncthreads();
-  double v = 0.0;
-  if (w == 0) {
-    v = l < kThreads / 32 ? scratch[l] : 0.0;
-#pragma unroll
-    for (int o = kThreads / 64; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-  }
-  return v;
+  if ((threadIdx.x & 31) == 0) sums[j][threadIdx.x >> 5] = a.value();
 }
 
-// The last block to finish sums all blocks' partials[b * k + j] into out[j]
-// in the fixed order of a separate single-block pass (b ascending per thread,
-// then the block sum), so one launch gives the final, repeatable values.
-// count: device counter, 0 before the launch and reset to 0 by the last block.
-__device__ void finish_sum(const double* partials, int k, double* __restrict__ out,
-                           unsigned* count, double* scratch) {
+__device__ void finish_sums(double (*sums)[kWarpsPerBlock], double* partials, int k,
+                            double* __restrict__ out, unsigned* count) {
   __shared__ bool last;
+  const int blocks = gridDim.x, w = threadIdx.x >> 5, l = threadIdx.x & 31;
+  __syncthreads();
+  for (int j = threadIdx.x; j < k; j += kThreads) {
+    double v = 0.0;
+#pragma unroll
+    for (int i = 0; i < kWarpsPerBlock; ++i) v += sums[j][i];
+    if (blocks == 1)
+      out[j] = v;
+    else
+      partials[(int64_t)j * blocks + blockIdx.x] = v;
+  }
+  if (blocks == 1) return;
   __threadfence();
   __syncthreads();
-  if (threadIdx.x == 0) last = atomicAdd(count, 1u) == gridDim.x - 1;
+  if (threadIdx.x == 0) last = atomicAdd(count, 1u) == blocks - 1;
   __syncthreads();
   if (!last) return;
   __threadfence();
-  for (int j = 0; j < k; ++j) {
-    double acc = 0.0;
-    for (int b = threadIdx.x; b < (int)gridDim.x; b += kThreads) acc += __ldcg(partials + b * k + j);
-    acc = block_sum(acc, scratch);
-    if (threadIdx.x == 0) out[j] = acc;
+  for (int j = w; j < k; j += kWarpsPerBlock) {
+    double v = 0.0;
+    for (int b = l; b < blocks; b += 32) v += __ldcg(partials + (int64_t)j * blocks + b);
+    v = warp_sum(v);
+    if (l == 0) out[j] = v;
   }
   if (threadIdx.x == 0) *count = 0;
 }
@@ -111,18 +107,25 @@ __device__ __forceinline__ void load8(const float* __restrict__ p, int64_t i0, i
   }
 }
 
-// load8 through L2 only (ld.global.cg): for values this kernel wrote itself,
-// which the non-coherent read-only path of load8 may not see
 template <bool kVec>
-__device__ __forceinline__ void load8_cg(const float* p, int64_t i0, int64_t n, float v[kChunk]) {
-  if (kVec && i0 + kChunk <= n) {
-    const float4 a = __ldcg(reinterpret_cast<const float4*>(p + i0));
-    const float4 b = __ldcg(reinterpret_cast<const float4*>(p + i0 + 4));
+__device__ __forceinline__ void load4(const float* p, int64_t i0, int64_t n, float v[4]) {
+  if (kVec && i0 + 4 <= n) {
+    const float4 a = *reinterpret_cast<const float4*>(p + i0);
     v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
-    v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
   } else {
 #pragma unroll
-    for (int t = 0; t < kChunk; ++t) v[t] = (i0 + t < n) ? __ldcg(p + i0 + t) : 0.0f;
+    for (int t = 0; t < 4; ++t) v[t] = (i0 + t < n) ? p[i0 + t] : 0.0f;
+  }
+}
+
+template <bool kVec>
+__device__ __forceinline__ void store4(float* p, int64_t i0, int64_t n, const float v[4]) {
+  if (kVec && i0 + 4 <= n) {
+    *reinterpret_cast<float4*>(p + i0) = make_float4(v[0], v[1], v[2], v[3]);
+  } else {
+#pragma unroll
+    for (int t = 0; t < 4; ++t)
+      if (i0 + t < n) p[i0 + t] = v[t];
   }
 }
 
@@ -149,98 +152,85 @@ __device__ __forceinline__ float chunk_dot(const float v[kChunk], const float u[
   return s;
 }
 
-// Block sums of the accumulators of vectors j0 .. j0 + G - 1 (those below k)
-// into partials[blockIdx.x * k + j].
-template <int G>
-__device__ __forceinline__ void group_partials(Acc2 (&acc)[G], int j0, int k, double* scratch,
-                                               double* partials) {
-#pragma unroll
-  for (int j = 0; j < G; ++j) {
-    if (j0 + j < k) {
-      const double r = block_sum2(acc[j], scratch);
-      if (threadIdx.x == 0) partials[blockIdx.x * k + j0 + j] = r;
-    }
+// out[j] = V_j . w (j < k <= KMAX), V_j = V + j * ldv; kUpdate: for
+// w <- w - sum_j coef[j] V_j first (coef: device FP64), the two halves of a CGS2
+// pass boundary in one pass over V and w.  If w == nullptr the squared norm of
+// V_0 is taken (k must be 1).
+// A thread takes C chunks of 4 values of w and of every vector at a time and
+// keeps them in registers for the update and the products, so each value is
+// read once and the loads of all vectors are in flight together.  HBM binds
+// it; 64 registers of values (128 at KMAX 32) at 2 blocks (1) per SM keep
+// enough bytes on the way.  Measured at 2^23 values, products alone / with the
+// update, us per launch: 9 to 16 vectors 76 / 98 (6.4 / 5.3 TB/s), 5 to 8 44 /
+// 50; with 8 vectors per pass, and the vectors read again from L2 for the
+// products, 99 / 144 and 54 / 78.
+template <int KMAX, bool kVec, bool kUpdate>
+__global__ void __launch_bounds__(kThreads, KMAX <= 16 ? 2 : 1)
+    k_project(const float* __restrict__ V, int64_t ldv, int k, const double* __restrict__ coef,
+              float* w, int64_t n, double* partials, double* out, unsigned* count) {
+  constexpr int C = KMAX <= 4 ? 4 : (KMAX <= 8 ? 2 : 1);
+  __shared__ double sums[KMAX][kWarpsPerBlock];
+  __shared__ float cf[KMAX];
+  if constexpr (kUpdate) {
+    for (int j = threadIdx.x; j < k; j += kThreads) cf[j] = (float)coef[j];
+    __syncthreads();
   }
-}
-
-// Inner products take the basis vectors in groups per pass over the chunks
-// (w re-read per group; kGroupDots in k_dots, which holds two chunks per
-// vector in flight, kGroup in the fused k_update_dots): each j's per-thread
-// sum still runs over the same chunks in the same order, so the results do
-// not depend on the grouping, and the accumulators (2 registers per vector)
-// stay within the 80 registers a thread may hold at 3 blocks of 256 threads
-// per SM, the residency that the fixed grid of 3 blocks per SM needs to run
-// in one wave.
-constexpr int kGroup = 16;
-constexpr int kGroupDots = 8;
-constexpr int kMinBlocks = 3;
-
-// out[j] = V_j . w (j < k <= KMAX), V_j = V + j * ldv; w is read once per
-// group of kGroupDots products (per-block partials in `partials`).  If
-// w == nullptr the squared norm of V_0 is taken (k must be 1).
-template <int KMAX, bool kVec>
-__global__ void __launch_bounds__(kThreads, kMinBlocks) k_dots(const float* __restrict__ V,
-                                                               int64_t ldv, int k,
-                                                               const float* __restrict__ w,
-                                                               int64_t n, double* partials,
-                                                               double* out, unsigned* count) {
-  constexpr int G = KMAX < kGroupDots ? KMAX : kGroupDots;
-  __shared__ double scratch[kThreads / 32];
-  const int64_t chunks = (n + kChunk - 1) / kChunk;
-  const int64_t stride = (int64_t)gridDim.x * kThreads;
+  const int64_t chunks = (n + 3) / 4, stride = (int64_t)gridDim.x * kThreads;
   const float* x = w ? w : V;
-  for (int j0 = 0; j0 < k; j0 += G) {
-    Acc2 acc[G];
-    // two of the thread's chunks per iteration (twice the loads in flight),
-    // added in chunk order
-    for (int64_t c = (int64_t)blockIdx.x * kThreads + threadIdx.x; c < chunks; c += 2 * stride) {
-      const int64_t i0 = c * kChunk, i1 = (c + stride) * kChunk;
-      const bool second = c + stride < chunks;
-      float u0[kChunk], u1[kChunk];
-      load8<kVec>(x, i0, n, u0);
-      if (second) load8<kVec>(x, i1, n, u1);
+  Acc2 acc[KMAX];
+  for (int64_t c0 = (int64_t)blockIdx.x * kThreads + threadIdx.x; c0 < chunks; c0 += C * stride) {
+    float u[C][4], v[KMAX][C][4];  // values past n are 0
 #pragma unroll
-      for (int j = 0; j < G; ++j) {
-        if (j0 + j < k) {
-          float v0[kChunk], v1[kChunk];
-          load8<kVec>(V + (j0 + j) * ldv, i0, n, v0);
-          if (second) load8<kVec>(V + (j0 + j) * ldv, i1, n, v1);
-          acc[j].add(chunk_dot(v0, u0, i0, n));
-          if (second) acc[j].add(chunk_dot(v1, u1, i1, n));
+    for (int i = 0; i < C; ++i) load4<kVec>(x, 4 * (c0 + i * stride), n, u[i]);
+#pragma unroll
+    for (int j = 0; j < KMAX; ++j) {
+      if (j < k) {
+#pragma unroll
+        for (int i = 0; i < C; ++i) load4<kVec>(V + j * ldv, 4 * (c0 + i * stride), n, v[j][i]);
+      }
+    }
+    if constexpr (kUpdate) {
+#pragma unroll
+      for (int j = 0; j < KMAX; ++j) {
+        if (j < k) {
+#pragma unroll
+          for (int i = 0; i < C; ++i)
+#pragma unroll
+            for (int t = 0; t < 4; ++t) u[i][t] = fmaf(-cf[j], v[j][i][t], u[i][t]);
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < C; ++i) store4<kVec>(w, 4 * (c0 + i * stride), n, u[i]);
+    }
+#pragma unroll
+    for (int j = 0; j < KMAX; ++j) {
+      if (j < k) {
+#pragma unroll
+        for (int i = 0; i < C; ++i) {
+          float p = 0.0f;
+#pragma unroll
+          for (int t = 0; t < 4; ++t) p = fmaf(v[j][i][t], u[i][t], p);
+          acc[j].add(p);
         }
       }
     }
-    group_partials<G>(acc, j0, k, scratch, partials);
   }
-  finish_sum(partials, k, out, count, scratch);
-}
-
-// x <- x - sum_j cf[j] V_j over one chunk, j in order for every element
-template <int KMAX, bool kVec>
-__device__ __forceinline__ void chunk_update(const float* __restrict__ V, int64_t ldv, int k,
-                                             const float* cf, int64_t i0, int64_t n,
-                                             float x[kChunk]) {
-  // up to 8 vectors fully unrolled; beyond, groups of 4 (a full unroll of 16
-  // or 32 hoists every vector's loads and takes up to 255 registers)
-#pragma unroll(KMAX <= 8 ? KMAX : 4)
-  for (int j = 0; j < k; ++j) {
-    float v[kChunk];
-    load8<kVec>(V + j * ldv, i0, n, v);
 #pragma unroll
-    for (int t = 0; t < kChunk; ++t) x[t] = fmaf(-cf[j], v[t], x[t]);
-  }
+  for (int j = 0; j < KMAX; ++j)
+    if (j < k) warp_value(acc[j], j, sums);
+  finish_sums(sums, partials, k, out, count);
 }
 
 // w <- w - sum_j coef[j] V_j (coef: device FP64);  optionally (norm_out) |w|^2
 template <int KMAX, bool kVec>
-__global__ void __launch_bounds__(kThreads, kMinBlocks) k_update(const float* __restrict__ V,
+__global__ void __launch_bounds__(kThreads, 3) k_update(const float* __restrict__ V,
                                                                  int64_t ldv, int k,
                                                                  const double* __restrict__ coef,
                                                                  float* __restrict__ w, int64_t n,
                                                                  double* partials,
                                                                  double* norm_out,
                                                                  unsigned* count) {
-  __shared__ double scratch[kThreads / 32];
+  __shared__ double sums[1][kWarpsPerBlock];
   __shared__ float cf[KMAX];
   for (int j = threadIdx.x; j < k; j += kThreads) cf[j] = (float)coef[j];
   __syncthreads();
@@ -274,68 +264,9 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) k_update(const float* __
     }
   }
   if (norm_out) {
-    const double r = block_sum2(acc, scratch);
-    if (threadIdx.x == 0) partials[blockIdx.x] = r;
-    finish_sum(partials, 1, norm_out, count, scratch);
+    warp_value(acc, 0, sums);
+    finish_sums(sums, partials, 1, norm_out, count);
   }
-}
-
-// w <- w - sum_j coef[j] V_j, and partials[b * k + j] of V_j . w for the
-// updated w: the two halves of a CGS2 pass boundary (the first pass's update
-// and the second pass's inner products) in one pass over V and w.  Each
-// element's arithmetic and each thread's chunks are those of k_update
-// followed by k_dots, so the results are identical to the two kernels.  The
-// pass takes the products of the first kGroup vectors; later groups re-read
-// the updated w (this thread's own stores, through L2) and their vectors.
-template <int KMAX, bool kVec>
-__global__ void __launch_bounds__(kThreads, kMinBlocks) k_update_dots(
-    const float* __restrict__ V, int64_t ldv, int k, const double* __restrict__ coef,
-    float* __restrict__ w, int64_t n, double* partials, double* out, unsigned* count) {
-  constexpr int G = KMAX < kGroup ? KMAX : kGroup;
-  __shared__ double scratch[kThreads / 32];
-  __shared__ float cf[KMAX];
-  for (int j = threadIdx.x; j < k; j += kThreads) cf[j] = (float)coef[j];
-  __syncthreads();
-  const int64_t chunks = (n + kChunk - 1) / kChunk;
-  {
-    Acc2 acc[G];
-    for (int64_t c = (int64_t)blockIdx.x * kThreads + threadIdx.x; c < chunks;
-         c += (int64_t)gridDim.x * kThreads) {
-      const int64_t i0 = c * kChunk;
-      float x[kChunk];
-      load8<kVec>(w, i0, n, x);
-      chunk_update<KMAX, kVec>(V, ldv, k, cf, i0, n, x);
-      store8<kVec>(w, i0, n, x);
-#pragma unroll
-      for (int j = 0; j < G; ++j) {
-        if (j < k) {
-          float v[kChunk];
-          load8<kVec>(V + j * ldv, i0, n, v);
-          acc[j].add(chunk_dot(v, x, i0, n));
-        }
-      }
-    }
-    group_partials<G>(acc, 0, k, scratch, partials);
-  }
-  for (int j0 = G; j0 < k; j0 += G) {
-    Acc2 acc[G];
-    for (int64_t c = (int64_t)blockIdx.x * kThreads + threadIdx.x; c < chunks;
-         c += (int64_t)gridDim.x * kThreads) {
-      const int64_t i0 = c * kChunk;
-      float x[kChunk];
-      load8_cg<kVec>(w, i0, n, x);
-#pragma unroll
-      for (int j = 0; j < G; ++j) {
-        if (j0 + j < k) {
-          float v[kChunk];
-          load8<kVec>(V + (j0 + j) * ldv, i0, n, v);
-          acc[j].add(chunk_dot(v, x, i0, n));
-        }
-      }
-    }
-    group_partials<G>(acc, j0, k, scratch, partials);
-  }
-  finish_sum(partials, k, out, count, scratch);
 }
 
 // y <- a * x + b * y  (host scalars), chunks of 8
@@ -352,6 +283,23 @@ __global__ void k_axpby(float a, const float* __restrict__ x, float b, float* __
 #pragma unroll
     for (int t = 0; t < kChunk; ++t) v[t] = fmaf(a, u[t], b * v[t]);
     store8<kVec>(y, i0, n, v);
+  }
+}
+
+// x <- x / sqrt(*norm2) unless it is 0: a vector is normalised by the sum its
+// reduction left on the device, before the host has read it
+template <bool kVec>
+__global__ void k_normalise(float* x, const double* __restrict__ norm2, int64_t n) {
+  const double s = *norm2;
+  if (!(s > 0.0)) return;
+  const float a = (float)(1.0 / sqrt(s));
+  for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; 4 * c < n;
+       c += (int64_t)gridDim.x * blockDim.x) {
+    float v[4];
+    load4<kVec>(x, 4 * c, n, v);
+#pragma unroll
+    for (int t = 0; t < 4; ++t) v[t] *= a;
+    store4<kVec>(x, 4 * c, n, v);
   }
 }
 
@@ -399,7 +347,7 @@ __global__ void __launch_bounds__(kThreads) k_mass_norm(const float* __restrict_
                                                         int ny, int nz, int nf, float cell,
                                                         double* partials, double* out,
                                                         unsigned* count) {
-  __shared__ double scratch[kThreads / 32];
+  __shared__ double sums[1][kWarpsPerBlock];
   const int64_t N = (int64_t)nx * ny * nz;
   const int64_t chunks = (N + 3) / 4;
   Acc2 acc;
@@ -454,9 +402,8 @@ __global__ void __launch_bounds__(kThreads) k_mass_norm(const float* __restrict_
     }
     acc.add(run);
   }
-  const double r = block_sum2(acc, scratch);
-  if (threadIdx.x == 0) partials[blockIdx.x] = r;
-  finish_sum(partials, 1, out, count, scratch);
+  warp_value(acc, 0, sums);
+  finish_sums(sums, partials, 1, out, count);
 }
 
 // out = a * m_i^(+1 or -1) * in over nf planes of nx x ny x nz nodes, m the
@@ -479,8 +426,9 @@ unsigned elementwise_blocks(int64_t n) {
 
 }  // namespace
 
-// 3 blocks per SM, fixed per device, so the reductions' order (and result)
-// never changes between calls on one device.
+// Most blocks of a reduction (the partials' size).  Each uses as many per SM
+// as its kernel is built for and no more than its values fill, a function of
+// the device and the size alone, so the order (and result) never changes.
 int krylov_partial_blocks() { return 3 * device_sm_count(); }
 
 namespace {
@@ -489,60 +437,70 @@ bool vec_ok(const void* a, const void* b, int64_t ldv) {
   return ((uintptr_t)a % 16 == 0) && ((uintptr_t)b % 16 == 0) && (ldv % 4 == 0);
 }
 
-// calls K<KMAX, kVec> for the smallest KMAX in {4, 8, 16, 32} holding k
-template <template <int, bool> class K, typename... A>
-cudaError_t dispatch_k(int k, bool vec, cudaStream_t s, A... args) {
-  const dim3 g(krylov_partial_blocks()), b(kThreads);
-#define PF_KRYLOV_CASE(M)                                            \
-  if (k <= M) {                                                      \
-    if (vec) K<M, true>::launch(g, b, s, args...);                   \
-    else K<M, false>::launch(g, b, s, args...);                      \
-    return cudaGetLastError();                                       \
-  }
-  PF_KRYLOV_CASE(4)
-  PF_KRYLOV_CASE(8)
-  PF_KRYLOV_CASE(16)
-  PF_KRYLOV_CASE(kMaxBasis)
-#undef PF_KRYLOV_CASE
-  return cudaErrorInvalidValue;
+unsigned reduction_blocks(int per_sm, int64_t chunks) {
+  const int64_t need = (chunks + kThreads - 1) / kThreads, cap = (int64_t)per_sm * device_sm_count();
+  return (unsigned)(need < 1 ? 1 : (need < cap ? need : cap));
 }
 
-template <int M, bool V>
-struct Dots {
-  template <typename... A>
-  static void launch(dim3 g, dim3 b, cudaStream_t s, A... a) { k_dots<M, V><<<g, b, 0, s>>>(a...); }
-};
-template <int M, bool V>
-struct Update {
-  template <typename... A>
-  static void launch(dim3 g, dim3 b, cudaStream_t s, A... a) { k_update<M, V><<<g, b, 0, s>>>(a...); }
-};
-template <int M, bool V>
-struct UpdateDots {
-  template <typename... A>
-  static void launch(dim3 g, dim3 b, cudaStream_t s, A... a) {
-    k_update_dots<M, V><<<g, b, 0, s>>>(a...);
-  }
-};
+// calls fn(KMAX) for the smallest KMAX in {4, 8, 16, 32} holding k
+template <class F>
+cudaError_t with_bound(int k, F&& fn) {
+  if (k <= 4) fn(std::integral_constant<int, 4>{});
+  else if (k <= 8) fn(std::integral_constant<int, 8>{});
+  else if (k <= 16) fn(std::integral_constant<int, 16>{});
+  else if (k <= kMaxBasis) fn(std::integral_constant<int, kMaxBasis>{});
+  else return cudaErrorInvalidValue;
+  return cudaGetLastError();
+}
+
+template <bool kUpdate>
+cudaError_t project(const float* V, int64_t ldv, int k, const double* coef, float* w, int64_t n,
+                    double* partials, double* out, unsigned* count, cudaStream_t s) {
+  const bool vec = vec_ok(V, w ? w : V, ldv);
+  return with_bound(k, [&](auto bound) {
+    constexpr int M = decltype(bound)::value;
+    const unsigned g = reduction_blocks(M <= 16 ? 2 : 1, (n + 3) / 4);
+    if (vec)
+      k_project<M, true, kUpdate><<<g, kThreads, 0, s>>>(V, ldv, k, coef, w, n, partials, out, count);
+    else
+      k_project<M, false, kUpdate><<<g, kThreads, 0, s>>>(V, ldv, k, coef, w, n, partials, out,
+                                                          count);
+  });
+}
 }  // namespace
 
 cudaError_t launch_dots(const float* V, int64_t ldv, int k, const float* w, int64_t n,
                         double* partials, double* out, unsigned* count, cudaStream_t s) {
-  return dispatch_k<Dots>(k, vec_ok(V, w ? w : V, ldv), s, V, ldv, k, w, n, partials, out, count);
+  // more than 16 products in two launches: w is read twice, but at 32 vectors
+  // per pass only one block fits an SM (20 products of 2^23 values: 157 us in
+  // one pass, 125 in two)
+  float* x = const_cast<float*>(w);
+  if (k > 16) {
+    const cudaError_t e = project<false>(V, ldv, 16, nullptr, x, n, partials, out, count, s);
+    if (e != cudaSuccess) return e;
+    return project<false>(V + 16 * ldv, ldv, k - 16, nullptr, x, n, partials, out + 16, count, s);
+  }
+  return project<false>(V, ldv, k, nullptr, x, n, partials, out, count, s);
 }
 
 cudaError_t launch_update(const float* V, int64_t ldv, int k, const double* coef, float* w,
                           int64_t n, double* partials, double* norm_out, unsigned* count,
                           cudaStream_t s) {
-  return dispatch_k<Update>(k, vec_ok(V, w, ldv), s, V, ldv, k, coef, w, n, partials, norm_out,
-                            count);
+  const bool vec = vec_ok(V, w, ldv);
+  const unsigned g = reduction_blocks(3, (n + kChunk - 1) / kChunk);
+  return with_bound(k, [&](auto bound) {
+    constexpr int M = decltype(bound)::value;
+    if (vec)
+      k_update<M, true><<<g, kThreads, 0, s>>>(V, ldv, k, coef, w, n, partials, norm_out, count);
+    else
+      k_update<M, false><<<g, kThreads, 0, s>>>(V, ldv, k, coef, w, n, partials, norm_out, count);
+  });
 }
 
 cudaError_t launch_update_dots(const float* V, int64_t ldv, int k, const double* coef, float* w,
                                int64_t n, double* partials, double* out, unsigned* count,
                                cudaStream_t s) {
-  return dispatch_k<UpdateDots>(k, vec_ok(V, w, ldv), s, V, ldv, k, coef, w, n, partials, out,
-                                count);
+  return project<true>(V, ldv, k, coef, w, n, partials, out, count, s);
 }
 
 cudaError_t launch_axpby(float a, const float* x, float b, float* y, int64_t n, cudaStream_t s) {
@@ -551,6 +509,15 @@ cudaError_t launch_axpby(float a, const float* x, float b, float* y, int64_t n, 
     k_axpby<true><<<g, 256, 0, s>>>(a, x, b, y, n);
   else
     k_axpby<false><<<g, 256, 0, s>>>(a, x, b, y, n);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_normalise(float* x, const double* norm2, int64_t n, cudaStream_t s) {
+  const unsigned g = elementwise_blocks((n + 3) / 4);
+  if ((uintptr_t)x % 16 == 0)
+    k_normalise<true><<<g, 256, 0, s>>>(x, norm2, n);
+  else
+    k_normalise<false><<<g, 256, 0, s>>>(x, norm2, n);
   return cudaGetLastError();
 }
 
@@ -583,12 +550,11 @@ cudaError_t launch_mass_norm(const float* g, int nx, int ny, int nz, int nf, dou
                              double* partials, double* out, unsigned* count, cudaStream_t s) {
   const int64_t N = (int64_t)nx * ny * nz;
   if (nf < 1 || nf > kMaxFields) return cudaErrorInvalidValue;
+  const unsigned b = reduction_blocks(3, (N + 3) / 4);
   if (N % 4 == 0 && (uintptr_t)g % 16 == 0)
-    k_mass_norm<true><<<krylov_partial_blocks(), kThreads, 0, s>>>(g, nx, ny, nz, nf, (float)cell,
-                                                                    partials, out, count);
+    k_mass_norm<true><<<b, kThreads, 0, s>>>(g, nx, ny, nz, nf, (float)cell, partials, out, count);
   else
-    k_mass_norm<false><<<krylov_partial_blocks(), kThreads, 0, s>>>(g, nx, ny, nz, nf, (float)cell,
-                                                                     partials, out, count);
+    k_mass_norm<false><<<b, kThreads, 0, s>>>(g, nx, ny, nz, nf, (float)cell, partials, out, count);
   return cudaGetLastError();
 }
 

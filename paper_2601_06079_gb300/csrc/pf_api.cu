@@ -55,6 +55,7 @@ struct pf_ctx {
   float* basis = nullptr;  // kMaxBasis Krylov vectors
   int64_t ldv = 0;         // floats between consecutive Krylov vectors
   double* small = nullptr; // h1[32], h2[32], scalars
+  double* host_sc = nullptr;  // pinned: reduction results on their way to the host
   unsigned* count = nullptr;  // block counter of the single-launch reductions (0 between calls)
   bool count_zeroed = false;  // set once the counter has been cleared after a bind
 
@@ -550,15 +551,23 @@ pf_status clear_count(pf_ctx* c) {
   return PF_OK;
 }
 
+// The first n doubles at p (device) on the host, through pinned memory: a copy
+// to pageable memory is staged and costs several us more per GMRES iteration.
+constexpr int kHostScalars = 2 * pf::kMaxBasis + 1;
+pf_status fetch_scalars(pf_ctx* c, const double* p, int n) {
+  if (!c->host_sc) PF_CUDA(cudaHostAlloc((void**)&c->host_sc, sizeof(double) * kHostScalars, 0));
+  PF_CUDA(cudaMemcpyAsync(c->host_sc, p, sizeof(double) * n, cudaMemcpyDeviceToHost, c->stream));
+  PF_CUDA(cudaStreamSynchronize(c->stream));
+  return PF_OK;
+}
+
 pf_status mass_norm(pf_ctx* c, const float* g, double* out) {
   if (pf_status st = clear_count(c)) return st;
   PF_CUDA(pf::launch_mass_norm(g, (int)c->n[0], (int)c->n[1], (int)c->n[2], imp_nf(c),
                                c->h[0] * c->h[1] * c->h[2], c->partials, c->result, c->count,
                                c->stream));
-  double h;
-  PF_CUDA(cudaMemcpyAsync(&h, c->result, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-  PF_CUDA(cudaStreamSynchronize(c->stream));
-  *out = std::sqrt(h);
+  if (pf_status st = fetch_scalars(c, c->result, 1)) return st;
+  *out = std::sqrt(c->host_sc[0]);
   return PF_OK;
 }
 
@@ -577,7 +586,6 @@ pf_status gmres3d(pf_ctx* c, int m, int maxit, double rtol, double atol, int* it
   double* dh2 = c->small + pf::kMaxBasis;
   double* dnrm = c->small + 2 * pf::kMaxBasis;
   std::vector<double> H((size_t)(m + 1) * m), cs(m), sn(m), gv(m + 1), y(m);
-  double host[2 * pf::kMaxBasis + 1];
   PF_CUDA(cudaMemsetAsync(c->d, 0, sizeof(float) * n, c->stream));
   int total = 0;
   double beta0 = -1.0, rel = 1.0;
@@ -590,8 +598,9 @@ pf_status gmres3d(pf_ctx* c, int m, int maxit, double rtol, double atol, int* it
       PF_CUDA(pf::launch_axpby(-1.0f, c->g, -1.0f, V, n, c->stream));
     }
     PF_CUDA(pf::launch_dots(V, ldv, 1, nullptr, n, c->partials, dnrm, c->count, c->stream));
-    PF_CUDA(cudaMemcpyAsync(host, dnrm, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-    PF_CUDA(cudaStreamSynchronize(c->stream));
+    PF_CUDA(pf::launch_normalise(V, dnrm, n, c->stream));
+    if (pf_status st = fetch_scalars(c, dnrm, 1)) return st;
+    const double* host = c->host_sc;
     const double beta = std::sqrt(host[0]);
     if (beta0 < 0) beta0 = beta;
     if (beta0 == 0.0) {
@@ -601,7 +610,6 @@ pf_status gmres3d(pf_ctx* c, int m, int maxit, double rtol, double atol, int* it
     rel = beta / beta0;
     const double target = std::max(rtol * beta0, atol);
     if (beta <= target || total >= maxit) break;
-    PF_CUDA(pf::launch_axpby((float)(1.0 / beta), V, 0.0f, V, n, c->stream));
     std::fill(gv.begin(), gv.end(), 0.0);
     gv[0] = beta;
     int k = 0;
@@ -613,15 +621,12 @@ pf_status gmres3d(pf_ctx* c, int m, int maxit, double rtol, double atol, int* it
       PF_CUDA(pf::launch_update_dots(V, ldv, k + 1, dh1, vk1, n, c->partials, dh2, c->count,
                                        c->stream));
       PF_CUDA(pf::launch_update(V, ldv, k + 1, dh2, vk1, n, c->partials, dnrm, c->count, c->stream));
-      PF_CUDA(cudaMemcpyAsync(host, c->small, sizeof(double) * (2 * pf::kMaxBasis + 1),
-                              cudaMemcpyDeviceToHost, c->stream));
-      PF_CUDA(cudaStreamSynchronize(c->stream));
+      PF_CUDA(pf::launch_normalise(vk1, dnrm, n, c->stream));
+      if (pf_status st = fetch_scalars(c, c->small, kHostScalars)) return st;
       ++total;
       for (int j = 0; j <= k; ++j) H[(size_t)j * m + k] = host[j] + host[pf::kMaxBasis + j];
       const double hk1 = std::sqrt(std::max(host[2 * pf::kMaxBasis], 0.0));
       H[(size_t)(k + 1) * m + k] = hk1;
-      if (hk1 > 0.0)
-        PF_CUDA(pf::launch_axpby((float)(1.0 / hk1), vk1, 0.0f, vk1, n, c->stream));
       for (int j = 0; j < k; ++j) {
         const double t = cs[j] * H[(size_t)j * m + k] + sn[j] * H[(size_t)(j + 1) * m + k];
         H[(size_t)(j + 1) * m + k] = -sn[j] * H[(size_t)j * m + k] + cs[j] * H[(size_t)(j + 1) * m + k];
@@ -1691,6 +1696,7 @@ void pf_destroy(pf_ctx* c) {
   if (!c) return;
   destroy_graph(c);
   if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
+  if (c->host_sc) cudaFreeHost(c->host_sc);
   delete c;
 }
 

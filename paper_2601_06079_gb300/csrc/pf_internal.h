@@ -315,10 +315,12 @@ cudaError_t launch_update(const float* V, int64_t ldv, int k, const double* coef
                           int64_t n, double* partials, double* norm_out, unsigned* count,
                           cudaStream_t s);
 // w <- w - sum_j coef[j] V_j, then out[j] = V_j . w (j < k) for the updated w,
-// in one pass (results identical to launch_update followed by launch_dots)
+// in one pass
 cudaError_t launch_update_dots(const float* V, int64_t ldv, int k, const double* coef, float* w,
                                int64_t n, double* partials, double* out, unsigned* count,
                                cudaStream_t s);
+// x <- x / sqrt(*norm2) (device scalar), unless it is 0
+cudaError_t launch_normalise(float* x, const double* norm2, int64_t n, cudaStream_t s);
 cudaError_t launch_axpby(float a, const float* x, float b, float* y, int64_t n, cudaStream_t s);
 cudaError_t launch_mass_mul(const float* in, float* out, int nx, int ny, int nz, int nf,
                             double cell, float a, int inverse, cudaStream_t s);
