@@ -168,7 +168,10 @@ Layout layout(const pf_ctx* c) {
   }
   L.partials = off;
   const size_t np = (size_t)std::max(2 * 1024, pf::krylov_partial_blocks() * pf::kMaxBasis);
-  off += align_up(sizeof(double) * np, 256);
+  size_t pb = sizeof(double) * np;
+  if (c->dim == 2 && has_implicit(c))
+    pb = std::max(pb, pf::newton2d_packet_bytes((int)c->n[0], (int)c->n[1]));
+  off += align_up(pb, 256);
   L.result = off;
   off += 256;
   L.small = off;
@@ -1042,6 +1045,63 @@ pf_status pf_energy(pf_ctx* c, const float* state, double* energy, double* mass)
   return PF_OK;
 }
 
+// Largest mesh whose implicit 2-D steps run as one launch.  Three steps of
+// dt = 0.5, us, one launch / launches per vector operation: Allen-Cahn 64^2
+// 840 / 2,870, 512^2 1,780 / 3,290, 1024^2 4,300 / 4,570, 1448^2 7,430 / 5,290;
+// Cahn-Hilliard 64^2 1,170 / 3,580, 512^2 2,590 / 4,460, 1024^2 6,380 / 6,550,
+// 1448^2 15,800 / 9,740 (a block's tiles outgrow its L1, and its 16 warps keep
+// fewer bytes on the way than the vector kernels).
+constexpr int64_t kNewton2DNodes = 1 << 20;
+
+// n_steps steps by k_newton2d, in launches of at most 64 steps.
+pf_status step_newton2d(pf_ctx* c, float* state, int64_t n_steps, const float* guess,
+                        const pf_newton_opts& o, double atol_factor, pf_newton_stats* s) {
+  pf::Newton2DArgs a{};
+  a.op = c->im2;
+  a.state = state;
+  a.u = c->u;
+  a.un = c->un;
+  a.g = c->g;
+  a.d = c->d;
+  a.V = c->basis;
+  a.ldv = c->ldv;
+  a.packets = (uint4*)c->partials;
+  const size_t packet_bytes = pf::newton2d_packet_bytes(a.op.nx, a.op.ny);
+  a.result = c->small;
+  a.limit = kWaitCycles;
+  a.max_newton = o.max_newton;
+  a.restart = o.gmres_restart;
+  a.maxit = o.gmres_max_iters;
+  a.newton_rtol = o.newton_rtol;
+  a.gmres_rtol = o.gmres_rtol;
+  a.atol_factor = atol_factor;
+  a.inv_dt = 1.0 / c->par.dt;
+  for (int64_t done = 0; done < n_steps;) {
+    a.guess = done == 0 ? guess : nullptr;
+    a.n_steps = (int)std::min<int64_t>(64, n_steps - done);
+    PF_CUDA(cudaMemsetAsync(a.packets, 0, packet_bytes, c->stream));
+    PF_CUDA(cudaMemsetAsync(a.result, 0xff, sizeof(double), c->stream));  // NaN: no result
+    PF_CUDA(pf::launch_newton2d(a, c->stream));
+    if (pf_status st = fetch_scalars(c, a.result, 7)) return st;
+    const double* r = c->host_sc;
+    if (std::isnan(r[0]))
+      return fail(c, PF_ERR_TIMEOUT, "a wait between blocks expired in the implicit solver");
+    s->newton_iters += (int)r[1];
+    s->gmres_iters += (int)r[2];
+    if (done == 0) s->initial_residual = r[3];
+    s->final_residual = r[4];
+    const pf_status st = (pf_status)(int)r[0];
+    if (st == PF_ERR_NONFINITE) return fail(c, st, "non-finite Newton residual");
+    if (st == PF_ERR_NOT_CONVERGED) {
+      s->converged = 0;
+      return fail(c, st, "Newton did not reach ||R|| <= %g (got %g) in step %lld", r[5], r[4],
+                  (long long)(done + (int64_t)r[6]));
+    }
+    done += a.n_steps;
+  }
+  return PF_OK;
+}
+
 pf_status pf_step_implicit(pf_ctx* c, float* state, int64_t n_steps, const float* guess,
                            const pf_newton_opts* opts, pf_newton_stats* stats) {
   if (!c) return PF_ERR_ARG;
@@ -1064,6 +1124,13 @@ pf_status pf_step_implicit(pf_ctx* c, float* state, int64_t n_steps, const float
   const int64_t n = vec_len(c);
   const double inv_dt = 1.0 / c->par.dt;
   const int64_t n_state = split_ch(c) ? nnodes(c) : n;  // CH: the state is c alone
+  if (c->dim == 2 && nnodes(c) <= kNewton2DNodes) {
+    st = step_newton2d(c, state, n_steps, guess, o,
+                       kNoOversolve / std::sqrt(c->h[0] * c->h[1] * c->h[2]), &s);
+    // as in the loop below, statistics are reported unless the solve broke off
+    if (stats && (st == PF_OK || st == PF_ERR_NOT_CONVERGED)) *stats = s;
+    return st;
+  }
   for (int64_t step = 0; step < n_steps; ++step) {
     PF_CUDA(cudaMemcpyAsync(c->un, state, sizeof(float) * n_state, cudaMemcpyDeviceToDevice,
                             c->stream));

@@ -268,6 +268,24 @@ cudaError_t launch_residual2d(const Implicit2DArgs& a, cudaStream_t s);
 cudaError_t launch_jvp2d(const Implicit2DArgs& a, cudaStream_t s);
 cudaError_t launch_jvp3d(const Implicit3DArgs& a, cudaStream_t s);
 
+// Newton-GMRES steps of a 2-D mesh in one cooperative launch (k_newton2d.cu).
+struct Newton2DArgs {
+  Implicit2DArgs op;    // operator constants (U, W, out unused)
+  float* state;         // in/out (Cahn-Hilliard: c)
+  const float* guess;   // first iterate of the first step, or null
+  float *u, *un, *g, *d, *V;  // vectors of nx ny values per plane, V: restart + 1 of them
+  int64_t ldv;
+  uint4* packets;       // newton2d_packet_bytes(), zeroed
+  double* result;       // status, Newton and GMRES iterations, initial and final residual,
+                        // last tolerance, steps done
+  long long limit;      // SM cycles of a wait
+  int n_steps, max_newton, restart, maxit;
+  double newton_rtol, gmres_rtol, atol_factor, inv_dt;
+};
+int newton2d_blocks(int nx, int ny);
+size_t newton2d_packet_bytes(int nx, int ny);
+cudaError_t launch_newton2d(const Newton2DArgs& a, cudaStream_t s);
+
 // Eshelby-inclusion elasticity (Eq. 3-4, III.1): K u with the element
 // stiffness ke[(a*3+i)*24 + b*3+j] of the uniform box element and its
 // assembled interior stencil ks[(o*3+i)*3+j], o = (dz+1)*9 + (dy+1)*3 + (dx+1).
