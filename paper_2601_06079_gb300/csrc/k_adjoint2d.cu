@@ -11,306 +11,438 @@
 //   dLoss/dkappa += -dt sum_i m_i w_i (m^-1 K c)_i
 //   dLoss/dW     += -dt / W sum_i m_i w_i (m^-1 F(c))_i
 //   dLoss/dm_a   += -dt M sum_e sum_q w|J| N_a(q) grad mu_q . grad y_q
-// (F', K, K_M symmetric).  Every operator is evaluated on a block tile staged
-// in shared memory with mirror images beyond the mesh, which reproduces the
+// (F', K, K_M symmetric).  Mirror images beyond the mesh reproduce the
 // zero-flux operators divided by the lumped mass; sums that need the real
 // (unmirrored) value at a boundary node take the mirrored value times the
-// node's mass fraction.  Reductions are FP64, per block and then in a fixed
-// order; per-node gradients accumulate in FP64 in place.  No atomics.
+// node's mass fraction.  No atomics.
+//
+// A warp sweeps a band of rows down a strip of 64 columns, a pair per lane, in
+// packed FP32 (sweep2d.h: values at Gauss points without their factor g_hi per
+// direction).  The planes are plain arrays; images come from reflected load
+// addresses.  The mobility's bilinear weights factorise: a flux along x at a y
+// Gauss point needs only the sum of M over the two x points, which is the sum
+// of M at the two nodes, interpolated in y, and the same the other way round:
+//   S(y) = (d u)(y) (m(x) + m(x+1))(y),  K_M u = c_x [S(x-1) - S(x)] + ...,
+// 2 products per direction and element instead of 4 points' gradients; so does
+// the mobility's gradient (products of differences, projected along one axis).
+//
+// Measured at 512^2 (us per step, graph replay): forward 5.7 with 32 x 16 node
+// tiles in shared memory (element passes into corner arrays, four barriers), 2.9
+// so; reverse 13.6, 7.1 so.  Both are latency-bound there (8 warps per SM); the
+// reverse sweep holds 164 registers.
 #include "pf_internal.h"
+#include "sweep2d.h"
 
 namespace pf {
 namespace {
 
-constexpr int TX = 32, TY = 16;       // output tile
+using namespace sweep;
+
 constexpr int kThreads = 256;
-constexpr int S2X = TX + 4, S2Y = TY + 4;  // nodes with a 2-node halo
-constexpr int S1X = TX + 2, S1Y = TY + 2;  // nodes with a 1-node halo
-constexpr int EX = TX + 3, EY = TY + 3;    // elements touching the 1-halo nodes
+constexpr int kWarps = 2;  // warps per block of the sweeps, stacked in y
+// Output rows per band, forward and reverse.  Reverse at 100 x 80 / 512^2 /
+// 1024^2, us per step: 4 rows 5.9 / 7.1 / 17.1, 2 rows 4.3 / 8.8 / 21.0, 6 rows
+// 7.5 / 9.3 / 17.2 (a lone warp's row takes 0.5 us, so short bands suit the
+// meshes this calibration runs on); 2 rows in flight 7.5 at 512^2.
+constexpr int kTYFwd = 4;
+constexpr int kTYRev = 4;
+constexpr int kAhead = 3;  // rows in flight
 
-// Mirror image of node index k on an axis of n nodes (period 2(n-1)).  Halo
-// indices lie within one period of the axis, where a reflection at each end
-// gives the image without the integer division.
-__device__ __forceinline__ int mirror(int k, int n) {
-  const int p = 2 * (n - 1);
-  if (k >= 1 - n && k <= p) return k < 0 ? -k : (k < n ? k : p - k);
-  k %= p;
-  if (k < 0) k += p;
-  return k < n ? k : p - k;
+__device__ __forceinline__ u64 bc(float v) { return pk(v, v); }
+__device__ __forceinline__ u64 sub2(u64 a, u64 b) { return fma2(b, bc(-1.0f), a); }
+__device__ __forceinline__ float from_left(float v) { return __shfl_up_sync(kFull, v, 1); }
+__device__ __forceinline__ float from_right(float v) { return __shfl_down_sync(kFull, v, 1); }
+
+// single reflection about the end nodes, then clamped: exact for the stored
+// nodes' two-node halo
+__device__ __forceinline__ int reflect(int k, int n) {
+  k = k < 0 ? -k : k;
+  k = k >= n ? 2 * (n - 1) - k : k;
+  return k < 0 ? 0 : (k >= n ? n - 1 : k);
 }
 
-__device__ __forceinline__ float gpt(int i) { return i ? kGHi : kGLo; }
+// a row of one plane in a lane: its two columns and the one right of them
+struct Row {
+  u64 v;
+  float r;
+  __device__ __forceinline__ u64 next() const { return pk(phi(v), r); }  // columns x+1, x+2
+};
+__device__ __forceinline__ Row row_of(u64 v) { return Row{v, from_right(plo(v))}; }
 
-// Gauss values of a bilinear field from corners c[ay*2+ax]; q = qy*2+qx
-__device__ __forceinline__ void qvals(const float c[4], float v[4]) {
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const float xi = gpt(q & 1), eta = gpt(q >> 1);
-    const float b = fmaf(xi, c[1] - c[0], c[0]), t = fmaf(xi, c[3] - c[2], c[2]);
-    v[q] = fmaf(eta, t - b, b);
+// interpolants along x at the two Gauss points (scalar FMAs, see sweep2d.h)
+__device__ __forceinline__ void along_x(const Row& a, float rho, u64& lo, u64& hi) {
+  const float v0 = plo(a.v), v1 = phi(a.v);
+  lo = pk(fmaf(rho, v1, v0), fmaf(rho, a.r, v1));
+  hi = pk(fmaf(rho, v0, v1), fmaf(rho, v1, a.r));
+}
+// shares of node columns from values at the two x Gauss points
+__device__ __forceinline__ u64 back_x(u64 lo, u64 hi, u64 rho) {
+  const u64 A = fma2(rho, hi, lo), B = fma2(rho, lo, hi);
+  const float bl = from_left(phi(B));
+  return pk(plo(A) + bl, phi(A) + plo(B));
+}
+// west + east neighbours
+__device__ __forceinline__ u64 beside(const Row& a) {
+  const float l = from_left(phi(a.v));
+  return pk(l + phi(a.v), plo(a.v) + a.r);
+}
+
+// 9-point stencil from three rows and their west + east sums
+struct Stencil {
+  u64 c0, cx, cy, cd;
+  __device__ __forceinline__ explicit Stencil(const Stencil2D& k)
+      : c0(bc(k.c0)), cx(bc(k.cx)), cy(bc(k.cy)), cd(bc(k.cd)) {}
+  __device__ __forceinline__ u64 operator()(u64 s, u64 c, u64 n, u64 ws, u64 wc, u64 wn) const {
+    return fma2(cd, add2(ws, wn), fma2(cy, add2(s, n), fma2(cx, wc, mul2(c0, c))));
   }
-}
-
-// 1/4 sum_q v_q N_a(q)  (Gauss weight |cell|/4 over the interior mass |cell|)
-__device__ __forceinline__ void qproject(const float v[4], float out[4]) {
-#pragma unroll
-  for (int a = 0; a < 4; ++a) {
-    float s = 0.0f;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const float xi = gpt(q & 1), eta = gpt(q >> 1);
-      const float na = ((a & 1) ? xi : 1.0f - xi) * ((a >> 1) ? eta : 1.0f - eta);
-      s = fmaf(v[q], na, s);
-    }
-    out[a] = 0.25f * s;
-  }
-}
-
-// gradient of a bilinear field at Gauss point q
-__device__ __forceinline__ void qgrad(const float c[4], int q, float ihx, float ihy, float& gx,
-                                      float& gy) {
-  const float xi = gpt(q & 1), eta = gpt(q >> 1);
-  gx = ((c[1] - c[0]) * (1.0f - eta) + (c[3] - c[2]) * eta) * ihx;
-  gy = ((c[2] - c[0]) * (1.0f - xi) + (c[3] - c[1]) * xi) * ihy;
-}
-
-// 1/4 sum_q Mq grad u_q . grad N_a(q)   (mobility-weighted stiffness, scaled)
-__device__ __forceinline__ void mob_stiff(const float u[4], const float mq[4], float ihx,
-                                          float ihy, float out[4]) {
-#pragma unroll
-  for (int a = 0; a < 4; ++a) out[a] = 0.0f;
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const float xi = gpt(q & 1), eta = gpt(q >> 1);
-    float gx, gy;
-    qgrad(u, q, ihx, ihy, gx, gy);
-    gx *= mq[q];
-    gy *= mq[q];
-#pragma unroll
-    for (int a = 0; a < 4; ++a) {
-      const float dnx = ((a & 1) ? ihx : -ihx) * ((a >> 1) ? eta : 1.0f - eta);
-      const float dny = ((a >> 1) ? ihy : -ihy) * ((a & 1) ? xi : 1.0f - xi);
-      out[a] = fmaf(gx, dnx, fmaf(gy, dny, out[a]));
-    }
-  }
-#pragma unroll
-  for (int a = 0; a < 4; ++a) out[a] *= 0.25f;
-}
-
-struct Tile {
-  float c[S2Y][S2X];   // shifted state d, 2-halo
-  float m[S2Y][S2X];   // mobility multiplier, 2-halo
-  float y[S2Y][S2X];   // adjoint (reverse step only), 2-halo
-  float mu[S1Y][S1X];  // chemical potential, 1-halo
-  float w[S1Y][S1X];   // m^-1 K_M y, 1-halo
-  float F[S1Y][S1X];   // m^-1 F(c)
-  float Kc[S1Y][S1X];  // m^-1 K c (without kappa)
-  float E[4][EY][EX];  // per-element corner contributions
-  float G[4][EY][EX];  // mobility-gradient corner contributions
 };
 
-__device__ __forceinline__ void corners(const float (*a)[S2X], int y, int x, float c[4]) {
-  c[0] = a[y][x];
-  c[1] = a[y][x + 1];
-  c[2] = a[y + 1][x];
-  c[3] = a[y + 1][x + 1];
-}
-
-__device__ __forceinline__ float gather4(const float (*E)[EY][EX], int y, int x) {
-  // node at 2-halo coordinates (y, x): element with corner a has lower-left (y - ay, x - ax)
-  return E[0][y][x] + E[1][y][x - 1] + E[2][y - 1][x] + E[3][y - 1][x - 1];
-}
-
-__device__ __forceinline__ float stencil9(const float* p, int ld, const Stencil2D& k) {
-  return k.c0 * p[0] + k.cx * (p[-1] + p[1]) + k.cy * (p[-ld] + p[ld]) +
-         k.cd * (p[-ld - 1] + p[-ld + 1] + p[ld - 1] + p[ld + 1]);
-}
-
-// Stage arrays, then F and mu on the 1-halo nodes (shared by both kernels).
-__device__ void stage_and_mu(Tile& T, const ChMobArgs& a, const float* yin, int x0, int y0) {
-  for (int i = threadIdx.x; i < S2X * S2Y; i += kThreads) {
-    const int lx = i % S2X, ly = i / S2X;
-    const int64_t g = (int64_t)mirror(y0 - 2 + ly, a.ny) * a.nx + mirror(x0 - 2 + lx, a.nx);
-    T.c[ly][lx] = a.d[g];
-    T.m[ly][lx] = a.mfield[g];
-    if (yin) T.y[ly][lx] = yin[g];
+// m^-1 F(c) and m^-1 K c, row by row
+struct Potential {
+  u64 c1, c2, w1, w2, am, ap, tl, th;  // rows k-1, k-2 of c; their west + east sums
+  u64 g[4];                            // Gauss values of the last element row
+  __device__ __forceinline__ void start(const Row& c, float rho) {
+    c2 = c1;
+    w2 = w1;
+    c1 = c.v;
+    w1 = beside(c);
+    along_x(c, rho, am, ap);
   }
-  __syncthreads();
-  for (int i = threadIdx.x; i < EX * EY; i += kThreads) {
-    const int ex = i % EX, ey = i / EX;
-    float c[4], q[4], f[4], o[4];
-    corners(T.c, ey, ex, c);
-    qvals(c, q);
+  // row k; kNode: F and K c of row k-1
+  template <bool kNode>
+  __device__ __forceinline__ void take(const Row& c, const ChMobArgs& a, u64 rho, u64& F, u64& Kc) {
+    u64 bm, bp;
+    along_x(c, plo(rho), bm, bp);
+    const u64 wc = beside(c);
+    g[0] = fma2(rho, bm, am);
+    g[1] = fma2(rho, am, bm);
+    g[2] = fma2(rho, bp, ap);
+    g[3] = fma2(rho, ap, bp);
+    const u64 p0 = bc(a.q[0]), p1 = bc(a.q[1]), p2 = bc(a.q[2]), p3 = bc(a.q[3]);
+    u64 f[4];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) f[k] = fmaf(fmaf(fmaf(a.p3, q[k], a.p2), q[k], a.p1), q[k], a.p0);
-    qproject(f, o);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) T.E[k][ey][ex] = o[k];
+    for (int i = 0; i < 4; ++i) f[i] = fma2(fma2(fma2(p3, g[i], p2), g[i], p1), g[i], p0);
+    if constexpr (kNode) {
+      F = back_x(add2(fma2(rho, f[1], f[0]), tl), add2(fma2(rho, f[3], f[2]), th), rho);
+      Kc = Stencil(a.k)(c2, c1, c.v, w2, w1, wc);
+    }
+    tl = fma2(rho, f[0], f[1]);
+    th = fma2(rho, f[2], f[3]);
+    am = bm;
+    ap = bp;
+    c2 = c1;
+    w2 = w1;
+    c1 = c.v;
+    w1 = wc;
   }
-  __syncthreads();
-  for (int i = threadIdx.x; i < S1X * S1Y; i += kThreads) {
-    const int x = 1 + i % S1X, y = 1 + i / S1X;  // 2-halo coordinates
-    const float F = gather4(T.E, y, x);
-    const float Kc = stencil9(&T.c[y][x], S2X, a.k);
-    T.F[y - 1][x - 1] = F;
-    T.Kc[y - 1][x - 1] = Kc;
-    T.mu[y - 1][x - 1] = fmaf(a.kappa, Kc, F);
-  }
-  __syncthreads();
-}
+};
 
-__device__ __forceinline__ void mob_at(const Tile& T, int ey, int ex, float M, float mq[4]) {
-  float mc[4];
-  corners(T.m, ey, ex, mc);
-  qvals(mc, mq);
-#pragma unroll
-  for (int k = 0; k < 4; ++k) mq[k] *= M;
-}
-
-__global__ void __launch_bounds__(kThreads) k_ch_mob_step(const ChMobArgs a, float* out) {
-  __shared__ Tile T;
-  const int x0 = blockIdx.x * TX, y0 = block_row() * TY;
-  if (y0 >= a.ny) return;
-  stage_and_mu(T, a, nullptr, x0, y0);
-  // K_M mu on the elements touching the tile nodes (lower-left 1 .. T+1 in 2-halo coords)
-  for (int i = threadIdx.x; i < (TX + 1) * (TY + 1); i += kThreads) {
-    const int ex = 1 + i % (TX + 1), ey = 1 + i / (TX + 1);
-    float u[4], mq[4], o[4];
-    u[0] = T.mu[ey - 1][ex - 1];
-    u[1] = T.mu[ey - 1][ex];
-    u[2] = T.mu[ey][ex - 1];
-    u[3] = T.mu[ey][ex];
-    mob_at(T, ey, ex, a.M, mq);
-    mob_stiff(u, mq, a.ihx, a.ihy, o);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) T.E[k][ey][ex] = o[k];
+// Differences of u along x (per row) and y (per element row) at the Gauss
+// points of the other direction
+struct Diff {
+  Row u;   // row k-1
+  u64 dx;  // its differences along x
+  __device__ __forceinline__ void start(const Row& r) {
+    u = r;
+    dx = sub2(r.next(), r.v);
   }
-  __syncthreads();
-  for (int i = threadIdx.x; i < TX * TY; i += kThreads) {
-    const int x = 2 + i % TX, y = 2 + i / TX;
-    const int gx = x0 + x - 2, gy = y0 + y - 2;
-    if (gx >= a.nx || gy >= a.ny) continue;
-    out[(int64_t)gy * a.nx + gx] = fmaf(-a.dt, gather4(T.E, y, x), T.c[y][x]);
+  // row k: x-differences at the element row's two y points, y-differences at
+  // its two x points
+  __device__ __forceinline__ void take(const Row& r, u64 rho, u64 (&x)[2], u64 (&y)[2]) {
+    const u64 d = sub2(r.next(), r.v);
+    x[0] = fma2(rho, d, dx);
+    x[1] = fma2(rho, dx, d);
+    along_x(Row{sub2(r.v, u.v), r.r - u.r}, plo(rho), y[0], y[1]);
+    u = r;
+    dx = d;
   }
-}
+};
 
-__global__ void __launch_bounds__(kThreads) k_ch_adj_step(const ChMobArgs a, const float* yin,
-                                                          float* yout, float* grad_hi,
-                                                          float* grad_lo, double* acc) {
-  __shared__ Tile T;
-  __shared__ double red[3][kThreads / 32];
-  const int x0 = blockIdx.x * TX, y0 = block_row() * TY;
-  if (y0 >= a.ny) return;
-  stage_and_mu(T, a, yin, x0, y0);
-  // K_M y on elements touching the 1-halo nodes; mobility gradient on those
-  // touching the tile nodes (mu is known on the 1-halo nodes only)
-  for (int i = threadIdx.x; i < EX * EY; i += kThreads) {
-    const int ex = i % EX, ey = i / EX;
-    float u[4], mq[4], o[4];
-    corners(T.y, ey, ex, u);
-    mob_at(T, ey, ex, a.M, mq);
-    mob_stiff(u, mq, a.ihx, a.ihy, o);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) T.E[k][ey][ex] = o[k];
-    if (ex >= 1 && ex <= TX + 1 && ey >= 1 && ey <= TY + 1) {
-      float mu[4], g[4];
-      mu[0] = T.mu[ey - 1][ex - 1];
-      mu[1] = T.mu[ey - 1][ex];
-      mu[2] = T.mu[ey][ex - 1];
-      mu[3] = T.mu[ey][ex];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        float mx, my, yx, yy;
-        qgrad(mu, q, a.ihx, a.ihy, mx, my);
-        qgrad(u, q, a.ihx, a.ihy, yx, yy);
-        g[q] = fmaf(mx, yx, my * yy);
-      }
-      qproject(g, o);
-#pragma unroll
-      for (int k = 0; k < 4; ++k) T.G[k][ey][ex] = o[k];
+// The element row's mobility factors: x sums at the two y points, y sums at the
+// two x points
+struct Mobility {
+  Row m;
+  u64 sx;
+  __device__ __forceinline__ void start(const Row& r) {
+    m = r;
+    sx = add2(r.v, r.next());
+  }
+  __device__ __forceinline__ void take(const Row& r, u64 rho, u64 (&x)[2], u64 (&y)[2]) {
+    const u64 s = add2(r.v, r.next());
+    x[0] = fma2(rho, s, sx);
+    x[1] = fma2(rho, sx, s);
+    along_x(Row{add2(r.v, m.v), r.r + m.r}, plo(rho), y[0], y[1]);
+    m = r;
+    sx = s;
+  }
+};
+
+// m^-1 K_M u: the shares of node row k-1 from the element rows above and below
+struct Flux {
+  u64 X, Y;  // carried from the element row above
+  template <bool kNode>
+  __device__ __forceinline__ void take(const u64 (&dx)[2], const u64 (&dy)[2], const u64 (&mx)[2],
+                                       const u64 (&my)[2], u64 rho, u64 cX, u64 cY, u64& out) {
+    const u64 f0 = mul2(dx[0], mx[0]), f1 = mul2(dx[1], mx[1]);
+    const u64 T = back_x(mul2(dy[0], my[0]), mul2(dy[1], my[1]), rho);
+    if constexpr (kNode) {
+      const u64 S = add2(fma2(rho, f1, f0), X);
+      const u64 W = pk(from_left(phi(S)), plo(S));  // the element left of each column
+      out = fma2(cY, sub2(Y, T), mul2(cX, sub2(W, S)));
+    }
+    X = fma2(rho, f0, f1);
+    Y = T;
+  }
+};
+
+struct Lane {
+  int x, xa, xb;  // first column, load columns of the pair
+  bool writer;
+  __device__ __forceinline__ explicit Lane(int nx) {
+    const int lane = threadIdx.x & 31;
+    x = blockIdx.x * kOutCols - kPair + kPair * lane;
+    xa = reflect(x, nx);
+    xb = reflect(x + 1, nx);
+    writer = lane >= 1 && lane <= 30 && x < nx;
+  }
+  __device__ __forceinline__ u64 load(const float* __restrict__ plane, int64_t row) const {
+    return pk(__ldg(plane + row + xa), __ldg(plane + row + xb));
+  }
+  // 64-bit where the pair is whole and aligned
+  __device__ __forceinline__ void store(float* row, int nx, u64 v) const {
+    if (x + 1 < nx && (reinterpret_cast<uintptr_t>(row + x) & 7) == 0) {
+      *reinterpret_cast<u64*>(row + x) = v;
+    } else {
+      row[x] = plo(v);
+      if (x + 1 < nx) row[x + 1] = phi(v);
     }
   }
-  __syncthreads();
-  // per-node products in FP32 (GB300's FP64 rate is a small fraction of its
-  // FP32 rate); each thread's two or three nodes sum in FP32, the block sums
-  // in FP64.  The running mobility gradient, summed over all steps, is a
-  // compensated FP32 pair per node (Knuth's two-sum: the rounding error of
-  // each addition is exact in FP32 and collects in lo).  The lumped mass m_i
-  // is cell * frac, with cell applied once per thread.
-  float dM = 0.0f;
-  const float ngm = a.ngm;  // -dt M cell
-  for (int i = threadIdx.x; i < S1X * S1Y; i += kThreads) {
-    const int x = 1 + i % S1X, y = 1 + i / S1X;
-    const float w = gather4(T.E, y, x);
-    T.w[y - 1][x - 1] = w;
-    const int gx = x0 + x - 2, gy = y0 + y - 2;
-    const bool tile_node = x >= 2 && x < TX + 2 && y >= 2 && y < TY + 2;
-    if (tile_node && gx < a.nx && gy < a.ny) {
-      const float frac = ((gx == 0 || gx == a.nx - 1) ? 0.5f : 1.0f) *
-                         ((gy == 0 || gy == a.ny - 1) ? 0.5f : 1.0f);
-      dM = fmaf(frac * w, T.mu[y - 1][x - 1], dM);
-      if (grad_hi) {
-        const int64_t gi = (int64_t)gy * a.nx + gx;
-        const float v = ngm * frac * gather4(T.G, y, x);
-        const float hi = grad_hi[gi], t = hi + v, bp = t - hi;
-        grad_lo[gi] += (hi - (t - bp)) + (v - bp);
-        grad_hi[gi] = t;
-      }
+};
+
+__global__ void __launch_bounds__(kWarps * 32) k_ch_mob_step(const ChMobArgs a, float* out) {
+  const int nx = a.nx, ny = a.ny;
+  const int y0 = (block_row() * kWarps + (threadIdx.x >> 5)) * kTYFwd;
+  if (y0 >= ny) return;
+  const Lane L(nx);
+  const u64 rho = bc(kGLo / kGHi), kappa = bc(a.kappa);
+  const u64 cX = bc(-a.dt * a.cX), cY = bc(-a.dt * a.cY);
+  u64 nc[kAhead], nm[kAhead];
+  const auto load = [&](int j, int k) {  // row y0 - 2 + k into slot j
+    const int64_t row = (int64_t)reflect(y0 - 2 + k, ny) * nx;
+    nc[j] = L.load(a.d, row);
+    nm[j] = L.load(a.mfield, row);
+  };
+#pragma unroll
+  for (int j = 0; j < kAhead; ++j) load(j, j);
+  Potential pot;
+  Mobility mob;
+  Diff dif;
+  Flux flux;
+  Row c, m = {0, 0.0f}, m1 = {0, 0.0f};  // rows k; m also of row k-1
+  u64 F, Kc, cc[3];
+  // the potential and the mobility run one element row apart: mu of row k-1 is
+  // known at row k, so its differences and the mobility's rows are k-2 and k-1
+  const auto next = [&](int k) {
+    m1 = m;
+    c = row_of(nc[k % kAhead]);
+    m = row_of(nm[k % kAhead]);
+    load(k % kAhead, k + kAhead);
+    cc[k % 3] = c.v;
+  };
+  u64 dx[2], dy[2], mx[2], my[2], kw;
+  next(0);
+  pot.start(c, plo(rho));
+  next(1);
+  pot.take<false>(c, a, rho, F, Kc);
+  next(2);
+  pot.take<true>(c, a, rho, F, Kc);  // mu of row y0 - 1
+  dif.start(row_of(fma2(kappa, Kc, F)));
+  mob.start(m1);
+#pragma unroll
+  for (int k = 3; k < kTYFwd + 4; ++k) {
+    next(k);
+    pot.take<true>(c, a, rho, F, Kc);  // mu of row y0 - 3 + k
+    dif.take(row_of(fma2(kappa, Kc, F)), rho, dx, dy);
+    mob.take(m1, rho, mx, my);
+    if (k == 3) {
+      flux.take<false>(dx, dy, mx, my, rho, cX, cY, kw);
+    } else {
+      flux.take<true>(dx, dy, mx, my, rho, cX, cY, kw);
+      const int y = y0 + k - 4;
+      if (L.writer && y < ny) L.store(out + (int64_t)y * nx, nx, add2(cc[(k - 2) % 3], kw));
     }
   }
-  __syncthreads();
-  // (F'(c) + kappa K) w on the tile nodes
-  for (int i = threadIdx.x; i < (TX + 1) * (TY + 1); i += kThreads) {
-    const int ex = 1 + i % (TX + 1), ey = 1 + i / (TX + 1);
-    float c[4], cq[4], u[4], uq[4], h[4], o[4];
-    corners(T.c, ey, ex, c);
-    qvals(c, cq);
-    u[0] = T.w[ey - 1][ex - 1];
-    u[1] = T.w[ey - 1][ex];
-    u[2] = T.w[ey][ex - 1];
-    u[3] = T.w[ey][ex];
-    qvals(u, uq);
+}
+
+// The reverse step.  acc: per warp three compensated FP32 pairs (hi, lo) of the
+// sums for kappa, W and M over all steps, the factors left to the end.
+__global__ void __launch_bounds__(kWarps * 32)
+    k_ch_adj_step(const ChMobArgs a, const float* yin, float* yout, float* grad_hi, float* grad_lo,
+                  float2* acc) {
+  const int nx = a.nx, ny = a.ny;
+  const int band = block_row() * kWarps + (threadIdx.x >> 5);
+  const int y0 = band * kTYRev;
+  if (y0 >= ny) return;
+  const Lane L(nx);
+  const u64 rho = bc(kGLo / kGHi), kappa = bc(a.kappa), ndt = bc(-a.dt);
+  const u64 cX = bc(a.cX), cY = bc(a.cY), gX = bc(a.gX), gY = bc(a.gY);
+  const u64 s0 = bc(a.h[0]), s1 = bc(a.h[1]), s2 = bc(a.h[2]);
+  const Stencil K(a.k);
+  u64 nc[kAhead], nm[kAhead], nyv[kAhead];
+  const auto load = [&](int j, int k) {
+    const int64_t row = (int64_t)reflect(y0 - 2 + k, ny) * nx;
+    nc[j] = L.load(a.d, row);
+    nm[j] = L.load(a.mfield, row);
+    nyv[j] = L.load(yin, row);
+  };
 #pragma unroll
-    for (int k = 0; k < 4; ++k) h[k] = fmaf(fmaf(a.s2, cq[k], a.s1), cq[k], a.s0) * uq[k];
-    qproject(h, o);
+  for (int j = 0; j < kAhead; ++j) load(j, j);
+  // mass fractions of this lane's columns; 0 in columns that it does not own
+  const auto fx = [&](int x) { return x == 0 || x == nx - 1 ? 0.5f : 1.0f; };
+  const float f0 = L.writer ? fx(L.x) : 0.0f;
+  const float f1 = L.writer && L.x + 1 < nx ? fx(L.x + 1) : 0.0f;
+  const u64 fxp = pk(f0, f1);
+
+  Potential pot;
+  Mobility mob;
+  Diff dy_, dmu;  // differences of y (rows k-1, k) and mu (rows k-2, k-1)
+  Flux flux;
+  u64 w1 = 0, w2 = 0, v1 = 0, v2 = 0;  // w of rows k-2, k-3; west + east sums
+  u64 wa = 0, wb = 0, hl = 0, hh = 0;  // x-interpolants of w; F' w's carry
+  u64 gx = 0, gy = 0;                  // carries of the mobility gradient
+  u64 px[2], py[2];                    // y's differences in element row (k-2, k-1)
+  u64 dK = 0, dW = 0, dM = 0;
+  Row c, m, y;
+  u64 yy[3], F, Kc, gq[4];
+  const auto next = [&](int k) {
+    c = row_of(nc[k % kAhead]);
+    m = row_of(nm[k % kAhead]);
+    y = row_of(nyv[k % kAhead]);
+    load(k % kAhead, k + kAhead);
+    yy[k % 3] = y.v;
+  };
+  u64 ex[2], ey[2], mx[2], my[2], w;
+  next(0);
+  pot.start(c, plo(rho));
+  dy_.start(y);
+  mob.start(m);
+  next(1);
+  pot.take<false>(c, a, rho, F, Kc);
+  dy_.take(y, rho, ex, ey);
+  mob.take(m, rho, mx, my);
+  flux.take<false>(ex, ey, mx, my, rho, cX, cY, w);
 #pragma unroll
-    for (int k = 0; k < 4; ++k) T.E[k][ey][ex] = o[k];
+  for (int k = 2; k < kTYRev + 4; ++k) {
+    // row k is y0 - 2 + k: mu and w of the row before it
+    next(k);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) gq[i] = pot.g[i];  // c in element row (k-2, k-1)
+    px[0] = ex[0];
+    px[1] = ex[1];
+    py[0] = ey[0];
+    py[1] = ey[1];
+    pot.take<true>(c, a, rho, F, Kc);
+    dy_.take(y, rho, ex, ey);
+    mob.take(m, rho, mx, my);
+    flux.take<true>(ex, ey, mx, my, rho, cX, cY, w);
+    const Row wr = row_of(w);
+    const u64 mu = fma2(kappa, Kc, F), vw = beside(wr);
+    const int yr = y0 - 3 + k;  // the row of mu and w
+    if (k >= 3 && k < kTYRev + 3 && yr < ny) {
+      const u64 fw = mul2(mul2(fxp, bc(yr == 0 || yr == ny - 1 ? 0.5f : 1.0f)), w);
+      dK = fma2(fw, Kc, dK);
+      dW = fma2(fw, F, dW);
+      dM = fma2(fw, mu, dM);
+    }
+    u64 na, nb;
+    along_x(wr, plo(rho), na, nb);
+    if (k == 2) {
+      dmu.start(row_of(mu));
+    } else {
+      // element row (k-2, k-1): F' w, and grad mu . grad y
+      u64 ux[2], uy[2], h[4];
+      dmu.take(row_of(mu), rho, ux, uy);
+      h[0] = mul2(fma2(fma2(s2, gq[0], s1), gq[0], s0), fma2(rho, na, wa));
+      h[1] = mul2(fma2(fma2(s2, gq[1], s1), gq[1], s0), fma2(rho, wa, na));
+      h[2] = mul2(fma2(fma2(s2, gq[2], s1), gq[2], s0), fma2(rho, nb, wb));
+      h[3] = mul2(fma2(fma2(s2, gq[3], s1), gq[3], s0), fma2(rho, wb, nb));
+      const u64 q0 = mul2(ux[0], px[0]), q1 = mul2(ux[1], px[1]);
+      const u64 T = back_x(mul2(uy[0], py[0]), mul2(uy[1], py[1]), rho);
+      if (k >= 4) {
+        const int yo = y0 + k - 4;  // the finished row
+        const u64 H = back_x(add2(fma2(rho, h[1], h[0]), hl), add2(fma2(rho, h[3], h[2]), hh), rho);
+        const u64 Hw = fma2(kappa, K(w2, w1, w, v2, v1, vw), H);
+        const u64 S = add2(fma2(rho, q1, q0), gx);
+        const u64 both = add2(S, pk(from_left(phi(S)), plo(S)));  // elements right and left
+        const u64 G = fma2(gY, add2(gy, T), mul2(gX, both));
+        if (L.writer && yo < ny) {
+          const int64_t row = (int64_t)yo * nx;
+          L.store(yout + row, nx, fma2(ndt, Hw, yy[(k - 2) % 3]));
+          if (grad_hi) {
+            const u64 v = mul2(mul2(fxp, bc(yo == 0 || yo == ny - 1 ? 0.5f : 1.0f)), G);
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+              if (L.x + i < nx) {
+                float* hp = grad_hi + row + L.x + i;
+                const float s = i ? phi(v) : plo(v), hi = *hp, t = hi + s, bp = t - hi;
+                grad_lo[row + L.x + i] += (hi - (t - bp)) + (s - bp);
+                *hp = t;
+              }
+            }
+          }
+        }
+      }
+      hl = fma2(rho, h[0], h[1]);
+      hh = fma2(rho, h[2], h[3]);
+      gx = fma2(rho, q0, q1);
+      gy = T;
+    }
+    w2 = w1;
+    v2 = v1;
+    w1 = w;
+    v1 = vw;
+    wa = na;
+    wb = nb;
   }
-  __syncthreads();
-  float dK = 0.0f, dW = 0.0f;
-  for (int i = threadIdx.x; i < TX * TY; i += kThreads) {
-    const int x = 2 + i % TX, y = 2 + i / TX;
-    const int gx = x0 + x - 2, gy = y0 + y - 2;
-    if (gx >= a.nx || gy >= a.ny) continue;
-    const float w = T.w[y - 1][x - 1];
-    const float Hw = gather4(T.E, y, x) + a.kappa * stencil9(&T.w[y - 1][x - 1], S1X, a.k);
-    yout[(int64_t)gy * a.nx + gx] = fmaf(-a.dt, Hw, T.y[y][x]);
-    const float frac = ((gx == 0 || gx == a.nx - 1) ? 0.5f : 1.0f) *
-                       ((gy == 0 || gy == a.ny - 1) ? 0.5f : 1.0f);
-    const float mw = frac * w;
-    dK = fmaf(mw, T.Kc[y - 1][x - 1], dK);
-    dW = fmaf(mw, T.F[y - 1][x - 1], dW);
-  }
-  // block sums (fixed order), accumulated across steps in this block's slot:
-  // warp sums in FP32 (a shuffle tree per step in FP64 would cost about 20
-  // FP64 operations per thread, and GB300 issues 2 per clock per SM), the
-  // warps and the steps in FP64
-  float v[3] = {dK, dW, dM};
+  // the warp's sums, into its pairs (Knuth's two-sum; FP64 only at the end: an
+  // FP64 instruction takes an SM 16 cycles per warp)
+  float v[3] = {plo(dK) + phi(dK), plo(dW) + phi(dW), plo(dM) + phi(dM)};
 #pragma unroll
   for (int j = 0; j < 3; ++j) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v[j] += __shfl_down_sync(0xffffffffu, v[j], o);
-    if ((threadIdx.x & 31) == 0) red[j][threadIdx.x >> 5] = a.cell * (double)v[j];
+    for (int o = 16; o > 0; o >>= 1) v[j] += __shfl_down_sync(kFull, v[j], o);
+  }
+  if ((threadIdx.x & 31) == 0) {
+    float2* p = acc + 3 * ((int64_t)band * gridDim.x + blockIdx.x);
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      const float2 q = p[j];
+      const float t = q.x + v[j], bp = t - q.x;
+      p[j] = make_float2(t, q.y + ((q.x - (t - bp)) + (v[j] - bp)));
+    }
+  }
+}
+
+// out[j] = scale[j] times the sum of the warps' pairs acc[3 i + j], one block
+__global__ void k_scalar_sums(const float2* __restrict__ acc, int n, double s0, double s1,
+                              double s2, double* __restrict__ out) {
+  __shared__ double red[3][kThreads / 32];
+  double v[3] = {0.0, 0.0, 0.0};
+  for (int i = threadIdx.x; i < n; i += kThreads)
+    for (int j = 0; j < 3; ++j) v[j] += (double)acc[3 * (int64_t)i + j].x + (double)acc[3 * (int64_t)i + j].y;
+  for (int j = 0; j < 3; ++j) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v[j] += __shfl_down_sync(kFull, v[j], o);
+    if ((threadIdx.x & 31) == 0) red[j][threadIdx.x >> 5] = v[j];
   }
   __syncthreads();
   if (threadIdx.x == 0) {
-    const int b = block_row() * gridDim.x + blockIdx.x;
-    double s[3] = {0, 0, 0};
-    for (int w = 0; w < kThreads / 32; ++w)
-      for (int j = 0; j < 3; ++j) s[j] += red[j][w];
-    acc[3 * b + 0] += -(double)a.dt * s[0];
-    acc[3 * b + 1] += -(double)a.dt * s[1] / a.W;
-    acc[3 * b + 2] += -(double)a.dt * s[2] / a.M;
+    const double sc[3] = {s0, s1, s2};
+    for (int j = 0; j < 3; ++j) {
+      double s = 0.0;
+      for (int w = 0; w < kThreads / 32; ++w) s += red[j][w];
+      out[j] = sc[j] * s;
+    }
   }
 }
 
@@ -390,19 +522,44 @@ cudaError_t launch_add(const float* in, float* out, int64_t n, float add, cudaSt
   return cudaGetLastError();
 }
 
-int ch_mob_blocks(int nx, int ny) { return ((nx + TX - 1) / TX) * ((ny + TY - 1) / TY); }
+namespace {
+int strips(int nx) { return (nx + kOutCols - 1) / kOutCols; }
+dim3 sweep_grid(const ChMobArgs& a, int ty) {
+  return row_grid(strips(a.nx), (a.ny + kWarps * ty - 1) / (kWarps * ty));
+}
+}  // namespace
+
+int ch_mob_warps(int nx, int ny) { return strips(nx) * ((ny + kTYRev - 1) / kTYRev); }
+
+void pack_ch_mob(ChMobArgs& a) {
+  const double g = kGHi, g2 = g * g, wt = 0.25 * g2;
+  const double p[4] = {a.p0, a.p1, a.p2, a.p3}, h[3] = {a.s0, a.s1, a.s2};
+  double s = 1.0;
+  for (int i = 0; i < 4; ++i, s *= g2) a.q[i] = (float)(wt * s * p[i]);
+  s = 1.0;
+  for (int i = 0; i < 3; ++i, s *= g2) a.h[i] = (float)(wt * g2 * s * h[i]);
+  const double ix = a.ihx, iy = a.ihy, g3 = g * g2;
+  a.cX = (float)(0.25 * a.M * ix * ix * g3);
+  a.cY = (float)(0.25 * a.M * iy * iy * g3);
+  a.gX = (float)(0.25 * a.ngm * ix * ix * g3);
+  a.gY = (float)(0.25 * a.ngm * iy * iy * g3);
+}
 
 cudaError_t launch_ch_mob_step(const ChMobArgs& a, float* out, cudaStream_t s) {
-  const dim3 grid = row_grid((a.nx + TX - 1) / TX, (a.ny + TY - 1) / TY);
-  k_ch_mob_step<<<grid, kThreads, 0, s>>>(a, out);
+  k_ch_mob_step<<<sweep_grid(a, kTYFwd), kWarps * 32, 0, s>>>(a, out);
   return cudaGetLastError();
 }
 
 cudaError_t launch_ch_adj_step(const ChMobArgs& a, const float* yin, float* yout,
-                               float* grad_hi, float* grad_lo, double* acc, cudaStream_t s) {
+                               float* grad_hi, float* grad_lo, float2* acc, cudaStream_t s) {
   if ((grad_hi == nullptr) != (grad_lo == nullptr)) return cudaErrorInvalidValue;
-  const dim3 grid = row_grid((a.nx + TX - 1) / TX, (a.ny + TY - 1) / TY);
-  k_ch_adj_step<<<grid, kThreads, 0, s>>>(a, yin, yout, grad_hi, grad_lo, acc);
+  k_ch_adj_step<<<sweep_grid(a, kTYRev), kWarps * 32, 0, s>>>(a, yin, yout, grad_hi, grad_lo, acc);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_scalar_sums(const float2* acc, int n, const double scale[3], double* out,
+                               cudaStream_t s) {
+  k_scalar_sums<<<1, kThreads, 0, s>>>(acc, n, scale[0], scale[1], scale[2], out);
   return cudaGetLastError();
 }
 
@@ -419,12 +576,6 @@ cudaError_t launch_loss(const float* d, float shift, const float* target, int nx
                         cudaStream_t s) {
   k_loss<<<kLossBlocks, kThreads, 0, s>>>(d, shift, target, nx, ny, cell, nodal, y, partials);
   k_colsum<<<1, 32, 0, s>>>(partials, kLossBlocks, 1, 1, out);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_colsum(const double* in, int nb, int stride, int k, double* out,
-                          cudaStream_t s) {
-  k_colsum<<<1, 32, 0, s>>>(in, nb, stride, k, out);
   return cudaGetLastError();
 }
 

@@ -409,7 +409,7 @@ AdjLayout adj_layout(const pf_ctx* c, int64_t n_steps, int ckpt) {
   L.glo = off;
   off += field;
   L.acc = off;
-  off += align_up(sizeof(double) * 3 * pf::ch_mob_blocks((int)c->n[0], (int)c->n[1]), 256);
+  off += align_up(sizeof(float2) * 3 * (size_t)pf::ch_mob_warps((int)c->n[0], (int)c->n[1]), 256);
   L.small = off;
   off += align_up(sizeof(double) * 512, 256);
   L.total = off;
@@ -930,6 +930,7 @@ pf_status pf_set_params(pf_ctx* c, const pf_params* p) {
     b.ihx = (float)(1.0 / hx);
     b.ihy = (float)(1.0 / hy);
     b.cell = m;
+    pf::pack_ch_mob(b);
   }
   pf::pack_explicit2d(a);
   destroy_graph(c);
@@ -1623,11 +1624,11 @@ pf_status pf_adjoint(pf_ctx* c, const float* state0, const float* target, int64_
   float* y0 = (float*)(ws + L.y0);
   float* y1 = (float*)(ws + L.y1);
   float* ones = (float*)(ws + L.ones);
-  double* acc = (double*)(ws + L.acc);
+  float2* acc = (float2*)(ws + L.acc);
   double* small = (double*)(ws + L.small);
   float* ghi = grad_mobility ? (float*)(ws + L.ghi) : nullptr;
   float* glo = grad_mobility ? (float*)(ws + L.glo) : nullptr;
-  const int nb = pf::ch_mob_blocks(nx, ny);
+  const int nw = pf::ch_mob_warps(nx, ny);
   const float shift = (float)c->par.shift;
   const double cell = c->h[0] * c->h[1];
   const float* saved_field = c->mob.mfield;
@@ -1638,79 +1639,97 @@ pf_status pf_adjoint(pf_ctx* c, const float* state0, const float* target, int64_
   }
   pf::ChMobArgs a = c->mob;
   a.ngm = (float)(-(double)a.dt * a.M * a.cell);
-  // forward with checkpoints: ck(j) = d^{j * ckpt_every}, ck(last) = d^N
+  pf::pack_ch_mob(a);
+  // whole segments replay graphs captured here (while earlier work runs):
+  // g[0] recomputes seg(1 .. ckpt-1) from seg(0), g[1 + p] reverses a segment
+  // starting from y0 (p = 0) or y1 (p = 1); a shorter last segment launches
+  // its steps one by one
+  CallGraphs cg;
+  const bool graphs = ckpt_every >= 8;
+  auto recompute = [&](cudaStream_t s, int64_t len) {
+    pf::ChMobArgs r = a;
+    cudaError_t e = cudaSuccess;
+    for (int64_t t = 1; t < len && e == cudaSuccess; ++t) {
+      r.d = seg(t - 1);
+      e = pf::launch_ch_mob_step(r, seg(t), s);
+    }
+    return e;
+  };
+  auto reverse = [&](cudaStream_t s, int64_t len, float* yi, float* yo) {
+    pf::ChMobArgs r = a;
+    cudaError_t e = cudaSuccess;
+    for (int64_t t = len - 1; t >= 0 && e == cudaSuccess; --t) {
+      r.d = seg(t);
+      e = pf::launch_ch_adj_step(r, yi, yo, ghi, glo, acc, s);
+      std::swap(yi, yo);
+    }
+    return e;
+  };
+  // d^{start} .. d^{start+len-1} of segment j into the segment buffer
+  auto fill_segment = [&](int64_t j, int64_t len) -> pf_status {
+    PF_CUDA(cudaMemcpyAsync(seg(0), ck(j), sizeof(float) * N, cudaMemcpyDeviceToDevice, c->stream));
+    if (!graphs || len != ckpt_every) {
+      PF_CUDA(recompute(c->stream, len));
+      return PF_OK;
+    }
+    if (!cg.g[0]) {
+      const pf_status rs = capture_graph(
+          c, [&](cudaStream_t s) { return recompute(s, ckpt_every); }, &cg.g[0],
+          "capture the recompute");
+      if (rs != PF_OK) return rs;
+    }
+    PF_CUDA(cudaGraphLaunch(cg.g[0], c->stream));
+    return PF_OK;
+  };
+  // forward with checkpoints: ck(j) = d^{j * ckpt_every}, ck(last) = d^N; the
+  // last segment's states stay in the segment buffer for the reverse sweep
   const int64_t last = (n_steps + ckpt_every - 1) / ckpt_every;
   PF_CUDA(pf::launch_add(state0, ck(0), N, -shift, c->stream));
-  for (int64_t j = 0; j < last && st == PF_OK; ++j) {
-    const int64_t len = std::min<int64_t>(ckpt_every, n_steps - j * ckpt_every);
-    st = mob_steps(c, ck(j), ck(j + 1), len);
+  for (int64_t j = 0; j < last - 1 && st == PF_OK; ++j) st = mob_steps(c, ck(j), ck(j + 1), ckpt_every);
+  if (st == PF_OK) {
+    const int64_t len = n_steps - (last - 1) * ckpt_every;
+    st = fill_segment(last - 1, len);
+    if (st == PF_OK) {
+      pf::ChMobArgs r = a;
+      r.d = seg(len - 1);
+      const cudaError_t e = pf::launch_ch_mob_step(r, ck(last), c->stream);
+      if (e != cudaSuccess) st = cuda_fail(c, e, "adjoint forward step");
+    }
   }
   if (st == PF_OK) {
     PF_CUDA(pf::launch_loss(ck(last), shift, target, nx, ny, cell, nodal_loss, y0, small + 8,
                             small, c->stream));
-    PF_CUDA(cudaMemsetAsync(acc, 0, sizeof(double) * 3 * nb, c->stream));
+    PF_CUDA(cudaMemsetAsync(acc, 0, sizeof(float2) * 3 * (size_t)nw, c->stream));
     if (grad_mobility) {
       PF_CUDA(cudaMemsetAsync(ghi, 0, sizeof(float) * N, c->stream));
       PF_CUDA(cudaMemsetAsync(glo, 0, sizeof(float) * N, c->stream));
     }
     float* yin = y0;
     float* yout = y1;
-    // whole segments replay graphs captured here (while the forward pass runs):
-    // g[0] recomputes seg(1 .. ckpt-1) from seg(0), g[1 + p] reverses a segment
-    // starting from y0 (p = 0) or y1 (p = 1); a shorter last segment launches
-    // its steps one by one
-    CallGraphs cg;
-    const bool graphs = ckpt_every >= 8;
-    auto recompute = [&](cudaStream_t s, int64_t len) {
-      pf::ChMobArgs r = a;
-      cudaError_t e = cudaSuccess;
-      for (int64_t t = 1; t < len && e == cudaSuccess; ++t) {
-        r.d = seg(t - 1);
-        e = pf::launch_ch_mob_step(r, seg(t), s);
-      }
-      return e;
-    };
-    auto reverse = [&](cudaStream_t s, int64_t len, float* yi, float* yo) {
-      pf::ChMobArgs r = a;
-      cudaError_t e = cudaSuccess;
-      for (int64_t t = len - 1; t >= 0 && e == cudaSuccess; --t) {
-        r.d = seg(t);
-        e = pf::launch_ch_adj_step(r, yi, yo, ghi, glo, acc, s);
-        std::swap(yi, yo);
-      }
-      return e;
-    };
     for (int64_t j = last - 1; j >= 0 && st == PF_OK; --j) {
-      const int64_t start = j * ckpt_every;
-      const int64_t len = std::min<int64_t>(ckpt_every, n_steps - start);
-      const bool whole = graphs && len == ckpt_every;
-      // recompute d^{start} .. d^{start+len-1} into the segment buffer
-      PF_CUDA(cudaMemcpyAsync(seg(0), ck(j), sizeof(float) * N, cudaMemcpyDeviceToDevice,
-                              c->stream));
+      const int64_t len = std::min<int64_t>(ckpt_every, n_steps - j * ckpt_every);
+      if (j < last - 1) st = fill_segment(j, len);
       cudaError_t e = cudaSuccess;
-      if (whole) {
-        if (!cg.g[0])
-          st = capture_graph(c, [&](cudaStream_t s) { return recompute(s, ckpt_every); }, &cg.g[0],
-                             "capture the recompute");
-        if (st == PF_OK) e = cudaGraphLaunch(cg.g[0], c->stream);
+      if (st == PF_OK && graphs && len == ckpt_every) {
         const int p = yin == y0 ? 0 : 1;
-        if (st == PF_OK && e == cudaSuccess && !cg.g[1 + p])
+        if (!cg.g[1 + p])
           st = capture_graph(c, [&](cudaStream_t s) { return reverse(s, ckpt_every, yin, yout); },
                              &cg.g[1 + p], "capture the reverse sweep");
-        if (st == PF_OK && e == cudaSuccess) e = cudaGraphLaunch(cg.g[1 + p], c->stream);
-        if (ckpt_every % 2) std::swap(yin, yout);
-      } else {
-        e = recompute(c->stream, len);
-        if (e == cudaSuccess) e = reverse(c->stream, len, yin, yout);
-        if (len % 2) std::swap(yin, yout);
+        if (st == PF_OK) e = cudaGraphLaunch(cg.g[1 + p], c->stream);
+      } else if (st == PF_OK) {
+        e = reverse(c->stream, len, yin, yout);
       }
+      if (len % 2) std::swap(yin, yout);
       if (st == PF_OK && e != cudaSuccess) {
         c->mob.mfield = saved_field;
         return cuda_fail(c, e, "adjoint step");
       }
     }
     if (st == PF_OK) {
-      cudaError_t e = pf::launch_colsum(acc, nb, 3, 3, small + 1, c->stream);
+      // -dt cell sums of w with m^-1 K c, m^-1 F and mu; F = W times its own
+      // polynomial, mu's mobility factor M
+      const double f = -(double)a.dt * a.cell, scale[3] = {f, f / a.W, f / a.M};
+      cudaError_t e = pf::launch_scalar_sums(acc, nw, scale, small + 1, c->stream);
       if (e == cudaSuccess && grad_mobility)
         e = pf::launch_grad_to_double(ghi, glo, grad_mobility, N, c->stream);
       if (e == cudaSuccess && grad_state0)

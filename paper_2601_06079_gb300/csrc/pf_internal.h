@@ -215,20 +215,25 @@ struct ChMobArgs {
   float kappa, M, W, dt, ihx, ihy;
   double cell;
   float ngm;  // -dt M cell, the factor of the mobility gradient (reverse step)
+  // filled by pack_ch_mob: the polynomials and the factors of the fluxes and of
+  // the mobility gradient, with the quadrature's weights
+  float q[4], h[3], cX, cY, gX, gY;
 };
-int ch_mob_blocks(int nx, int ny);
+void pack_ch_mob(ChMobArgs& a);
+int ch_mob_warps(int nx, int ny);  // triples of pairs in the reverse step's acc
 cudaError_t launch_ch_mob_step(const ChMobArgs& a, float* out, cudaStream_t s);
 // grad_hi / grad_lo: the running mobility gradient as a compensated FP32 pair
 // per node (both null: not accumulated); grad_to_double writes hi + lo in FP64.
 cudaError_t launch_ch_adj_step(const ChMobArgs& a, const float* yin, float* yout,
-                               float* grad_hi, float* grad_lo, double* acc, cudaStream_t s);
+                               float* grad_hi, float* grad_lo, float2* acc, cudaStream_t s);
+// out[j] = scale[j] * (sum over i < n of the pair acc[3 i + j]), j < 3
+cudaError_t launch_scalar_sums(const float2* acc, int n, const double scale[3], double* out,
+                               cudaStream_t s);
 cudaError_t launch_grad_to_double(const float* hi, const float* lo, double* out, int64_t n,
                                   cudaStream_t s);
 cudaError_t launch_loss(const float* d, float shift, const float* target, int nx, int ny,
                         double cell, int nodal, float* y, double* partials, double* out,
                         cudaStream_t s);
-cudaError_t launch_colsum(const double* in, int nb, int stride, int k, double* out,
-                          cudaStream_t s);
 cudaError_t launch_mass_scale(const float* y, int nx, int ny, double cell, float* out,
                               cudaStream_t s);
 cudaError_t launch_add(const float* in, float* out, int64_t n, float add, cudaStream_t s);
