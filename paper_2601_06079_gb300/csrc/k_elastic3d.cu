@@ -44,20 +44,28 @@ __device__ double block_sum(float v) {
   return s;
 }
 
-// the same for FP64 inputs (the single-block sum of the block partials)
-__device__ double block_sum_f64(double v) {
-  __shared__ double part[32];
-  const int t = threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z);
-  const int nt = blockDim.x * blockDim.y * blockDim.z;
+// Sum of part[0 .. nb) for thread 0 of a block of kCgThreads, in a fixed order:
+// the second stage of a grid-wide sum, made by every block of the kernel that
+// needs it.  256 threads do it, because FP64 additions of more warps would only
+// queue for the SM's FP64 unit.
+constexpr int kCgThreads = 1024;
+__device__ __forceinline__ double sum_partials(const double* __restrict__ part, int nb) {
+  __shared__ double warp[8];
+  const int t = threadIdx.x;
+  if (t < 256) {
+    double v = 0.0;
+    for (int b = t; b < nb; b += 256) v += part[b];
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-  __syncthreads();
-  if ((t & 31) == 0) part[t >> 5] = v;
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    if ((t & 31) == 0) warp[t >> 5] = v;
+  }
   __syncthreads();
   double s = 0.0;
-  if (t == 0)
-    for (int w = 0; w < (nt + 31) / 32; ++w) s += part[w];
-  return s;
+  if (t == 0) {
+#pragma unroll
+    for (int w = 0; w < 8; ++w) s += warp[w];
+  }
+  return s;  // in thread 0
 }
 
 __device__ __forceinline__ int clampi(int v, int lo, int hi) { return v < lo ? lo : (v > hi ? hi : v); }
@@ -332,37 +340,61 @@ __global__ void __launch_bounds__(kThreads) k_elastic_load(ElasticLoadArgs a, fl
 }
 
 // CG, with the scalars on the device: sc[0], sc[1] = r.r (ping-pong by
-// iteration parity `slot`), sc[2] = p.Ap.
-//   x += alpha p, r -= alpha Ap   with alpha = sc[slot] / sc[2]
-//   and part[block] = the block's FP64 partial of the new r . r
-//   (float4 over the first 4 n4 entries -- n4 = 0 unless every vector is
-//   16-byte aligned -- and scalars over the rest)
-__global__ void k_cg_xr(float* __restrict__ x, float* __restrict__ r, const float* __restrict__ p,
-                        const float* __restrict__ Ap, int64_t n, int64_t n4,
-                        const double* __restrict__ sc, int slot, double* __restrict__ part) {
-  const float alpha = (float)(sc[slot] / sc[2]);
-  float rr = 0.0f;  // at most a few dozen squares per thread; blocks sum in FP64
-  const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, nth = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t i = tid; i < n4; i += nth) {
-    float4 xv = reinterpret_cast<float4*>(x)[i], rv = reinterpret_cast<float4*>(r)[i];
-    const float4 pv = reinterpret_cast<const float4*>(p)[i], av = reinterpret_cast<const float4*>(Ap)[i];
-    xv.x = fmaf(alpha, pv.x, xv.x);
-    xv.y = fmaf(alpha, pv.y, xv.y);
-    xv.z = fmaf(alpha, pv.z, xv.z);
-    xv.w = fmaf(alpha, pv.w, xv.w);
-    rv.x = fmaf(-alpha, av.x, rv.x);
-    rv.y = fmaf(-alpha, av.y, rv.y);
-    rv.z = fmaf(-alpha, av.z, rv.z);
-    rv.w = fmaf(-alpha, av.w, rv.w);
-    reinterpret_cast<float4*>(x)[i] = xv;
-    reinterpret_cast<float4*>(r)[i] = rv;
-    rr = fmaf(rv.x, rv.x, rr);
-    rr = fmaf(rv.y, rv.y, rr);
-    rr = fmaf(rv.z, rv.z, rr);
-    rr = fmaf(rv.w, rv.w, rr);
+// iteration parity `slot`), sc[2] = p.Ap.  Both kernels are bound by memory
+// (float4 over the first 4 n4 entries -- n4 = 0 unless every vector is
+// 16-byte aligned -- and scalars over the rest).
+//   k_cg_r:  r -= alpha Ap, partials of the new r.r;  alpha = sc[slot] / p.Ap
+//   k_cg_xp: x += alpha p, p = r + beta p;            beta = r.r / sc[slot]
+// x is moved along where p is read anyway, so an iteration passes over eight
+// vectors instead of nine.  Each block adds the partials of the launch before
+// it for itself, and block 0 leaves the sum in sc: as launches of their own
+// the two sums took 6 us each of a 90 us iteration on a 129^3 mesh, and
+// finished by the last block of the launch that makes them they cost its
+// blocks a fence each, as much again.  One block of 1024 threads per SM keeps
+// the sum to one per SM.  A solve on 129^3 nodes: 51.5 ms with two more launches
+// and x beside r, 50.0 with the last block's sum, 44.4 so; on a mesh whose
+// vectors all stay in L2 15.0 and 10.8 ms.
+__global__ void __launch_bounds__(kCgThreads) k_cg_r(float* __restrict__ r,
+                                                     const float* __restrict__ Ap, int64_t n,
+                                                     int64_t n4, double* __restrict__ sc, int slot,
+                                                     const double* __restrict__ pap, int npap,
+                                                     double* __restrict__ part) {
+  __shared__ float sh;
+  const double d = sum_partials(pap, npap);
+  if (threadIdx.x == 0) {
+    sh = (float)(sc[slot] / d);
+    if (blockIdx.x == 0) sc[2] = d;
   }
+  __syncthreads();
+  const float alpha = sh;
+  // four runs of at most a few dozen squares per thread; blocks sum in FP64
+  float4 q = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+  const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, nth = (int64_t)gridDim.x * blockDim.x;
+  constexpr int kU = 4;
+  for (int64_t i = tid; i < n4; i += kU * nth) {
+    float4 rv[kU], av[kU];
+#pragma unroll
+    for (int u = 0; u < kU; ++u)
+      if (i + u * nth < n4) {
+        rv[u] = reinterpret_cast<float4*>(r)[i + u * nth];
+        av[u] = reinterpret_cast<const float4*>(Ap)[i + u * nth];
+      }
+#pragma unroll
+    for (int u = 0; u < kU; ++u)
+      if (i + u * nth < n4) {
+        rv[u].x = fmaf(-alpha, av[u].x, rv[u].x);
+        rv[u].y = fmaf(-alpha, av[u].y, rv[u].y);
+        rv[u].z = fmaf(-alpha, av[u].z, rv[u].z);
+        rv[u].w = fmaf(-alpha, av[u].w, rv[u].w);
+        reinterpret_cast<float4*>(r)[i + u * nth] = rv[u];
+        q.x = fmaf(rv[u].x, rv[u].x, q.x);
+        q.y = fmaf(rv[u].y, rv[u].y, q.y);
+        q.z = fmaf(rv[u].z, rv[u].z, q.z);
+        q.w = fmaf(rv[u].w, rv[u].w, q.w);
+      }
+  }
+  float rr = (q.x + q.y) + (q.z + q.w);
   for (int64_t i = 4 * n4 + tid; i < n; i += nth) {
-    x[i] = fmaf(alpha, p[i], x[i]);
     const float ri = fmaf(-alpha, Ap[i], r[i]);
     r[i] = ri;
     rr = fmaf(ri, ri, rr);
@@ -371,29 +403,51 @@ __global__ void k_cg_xr(float* __restrict__ x, float* __restrict__ r, const floa
   if (threadIdx.x == 0) part[blockIdx.x] = s;
 }
 
-// out = sum of part[0 .. nb) in a fixed order (one block)
-__global__ void k_sum_part(const double* __restrict__ part, int nb, double* __restrict__ out) {
-  double v = 0.0;
-  for (int b = threadIdx.x; b < nb; b += blockDim.x) v += part[b];
-  const double s = block_sum_f64(v);
-  if (threadIdx.x == 0) *out = s;
-}
-
-//   p = r + beta p   with beta = sc[1 - slot] / sc[slot]
-__global__ void k_cg_p(const float* __restrict__ r, float* __restrict__ p, int64_t n, int64_t n4,
-                       const double* __restrict__ sc, int slot) {
-  const float beta = (float)(sc[1 - slot] / sc[slot]);
-  const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, nth = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t i = tid; i < n4; i += nth) {
-    float4 pv = reinterpret_cast<float4*>(p)[i];
-    const float4 rv = reinterpret_cast<const float4*>(r)[i];
-    pv.x = fmaf(beta, pv.x, rv.x);
-    pv.y = fmaf(beta, pv.y, rv.y);
-    pv.z = fmaf(beta, pv.z, rv.z);
-    pv.w = fmaf(beta, pv.w, rv.w);
-    reinterpret_cast<float4*>(p)[i] = pv;
+__global__ void __launch_bounds__(kCgThreads) k_cg_xp(float* __restrict__ x,
+                                                      const float* __restrict__ r,
+                                                      float* __restrict__ p, int64_t n, int64_t n4,
+                                                      double* __restrict__ sc, int slot,
+                                                      const double* __restrict__ part, int nb) {
+  __shared__ float sh[2];
+  const double rr = sum_partials(part, nb);
+  if (threadIdx.x == 0) {
+    sh[1] = (float)(rr / sc[slot]);
+    if (blockIdx.x == 0) sc[1 - slot] = rr;
   }
-  for (int64_t i = 4 * n4 + tid; i < n; i += nth) p[i] = fmaf(beta, p[i], r[i]);
+  if (threadIdx.x == kCgThreads - 1) sh[0] = (float)(sc[slot] / sc[2]);
+  __syncthreads();
+  const float alpha = sh[0], beta = sh[1];
+  const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, nth = (int64_t)gridDim.x * blockDim.x;
+  constexpr int kU = 3;
+  for (int64_t i = tid; i < n4; i += kU * nth) {
+    float4 pv[kU], xv[kU], rv[kU];
+#pragma unroll
+    for (int u = 0; u < kU; ++u)
+      if (i + u * nth < n4) {
+        pv[u] = reinterpret_cast<float4*>(p)[i + u * nth];
+        rv[u] = reinterpret_cast<const float4*>(r)[i + u * nth];
+        xv[u] = reinterpret_cast<float4*>(x)[i + u * nth];
+      }
+#pragma unroll
+    for (int u = 0; u < kU; ++u)
+      if (i + u * nth < n4) {
+        xv[u].x = fmaf(alpha, pv[u].x, xv[u].x);
+        xv[u].y = fmaf(alpha, pv[u].y, xv[u].y);
+        xv[u].z = fmaf(alpha, pv[u].z, xv[u].z);
+        xv[u].w = fmaf(alpha, pv[u].w, xv[u].w);
+        pv[u].x = fmaf(beta, pv[u].x, rv[u].x);
+        pv[u].y = fmaf(beta, pv[u].y, rv[u].y);
+        pv[u].z = fmaf(beta, pv[u].z, rv[u].z);
+        pv[u].w = fmaf(beta, pv[u].w, rv[u].w);
+        reinterpret_cast<float4*>(x)[i + u * nth] = xv[u];
+        reinterpret_cast<float4*>(p)[i + u * nth] = pv[u];
+      }
+  }
+  for (int64_t i = 4 * n4 + tid; i < n; i += nth) {
+    const float pi = p[i];
+    x[i] = fmaf(alpha, pi, x[i]);
+    p[i] = fmaf(beta, pi, r[i]);
+  }
 }
 
 // zero the constrained entries (symmetry planes) of a displacement vector
@@ -429,8 +483,8 @@ int elastic_apply_blocks(int nx, int ny, int nz) {
   return (int)(g.x * g.y * g.z) + boundary_blocks(nx, ny, nz);
 }
 
-// 8 blocks per SM, fixed per device (the r.r partials are summed in a fixed order)
-int cg_blocks() { return 8 * device_sm_count(); }
+// fixed per device (the r.r partials are summed in a fixed order)
+int cg_blocks() { return device_sm_count(); }
 
 cudaError_t launch_elastic_apply(const Elastic3DArgs& a, cudaStream_t s) {
   const dim3 gi = interior_grid(a.nx, a.ny, a.nz);
@@ -439,11 +493,6 @@ cudaError_t launch_elastic_apply(const Elastic3DArgs& a, cudaStream_t s) {
     k_elastic_apply<true><<<ni + nb, kThreads, 0, s>>>(a, (int)gi.x, (int)gi.y, ni);
   else
     k_elastic_apply<false><<<ni + nb, kThreads, 0, s>>>(a, (int)gi.x, (int)gi.y, ni);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_sum_part(const double* part, int nb, double* out, cudaStream_t s) {
-  k_sum_part<<<1, 256, 0, s>>>(part, nb, out);
   return cudaGetLastError();
 }
 
@@ -458,17 +507,18 @@ cudaError_t launch_elastic_constrain(float* v, int nx, int ny, int nz, cudaStrea
   return cudaGetLastError();
 }
 
-cudaError_t launch_cg_xr(float* x, float* r, const float* p, const float* Ap, int64_t n,
-                         const double* sc, int slot, double* part, cudaStream_t s) {
-  const bool al = (((uintptr_t)x | (uintptr_t)r | (uintptr_t)p | (uintptr_t)Ap) & 15) == 0;
-  k_cg_xr<<<cg_blocks(), 256, 0, s>>>(x, r, p, Ap, n, al ? n / 4 : 0, sc, slot, part);
+cudaError_t launch_cg_r(float* r, const float* Ap, int64_t n, double* sc, int slot,
+                        const double* pap, int npap, double* part, cudaStream_t s) {
+  const bool al = (((uintptr_t)r | (uintptr_t)Ap) & 15) == 0;
+  k_cg_r<<<cg_blocks(), kCgThreads, 0, s>>>(r, Ap, n, al ? n / 4 : 0, sc, slot, pap, npap, part);
   return cudaGetLastError();
 }
 
-cudaError_t launch_cg_p(const float* r, float* p, int64_t n, const double* sc, int slot,
-                        cudaStream_t s) {
-  const bool al = (((uintptr_t)r | (uintptr_t)p) & 15) == 0;
-  k_cg_p<<<blocks_for(n), 256, 0, s>>>(r, p, n, al ? n / 4 : 0, sc, slot);
+cudaError_t launch_cg_xp(float* x, const float* r, float* p, int64_t n, double* sc, int slot,
+                         const double* part, cudaStream_t s) {
+  const bool al = (((uintptr_t)x | (uintptr_t)r | (uintptr_t)p) & 15) == 0;
+  k_cg_xp<<<device_sm_count(), kCgThreads, 0, s>>>(x, r, p, n, al ? n / 4 : 0, sc, slot, part,
+                                                   cg_blocks());
   return cudaGetLastError();
 }
 

@@ -136,10 +136,10 @@ Layout layout(const pf_elastic* e) {
   Layout L;
   L.vec = ((size_t)(3 * nodes(e)) * sizeof(float) + 255) / 256 * 256;
   L.off_part = 7 * L.vec;
-  // FP64 partials, shared in turn by the apply, the update and launch_dots
+  // FP64 partials: launch_dots' or, of a CG iteration, the apply's and the update's
   size_t np = (size_t)pf::krylov_partial_blocks();
-  np = std::max(np, (size_t)pf::cg_blocks());
-  np = std::max(np, (size_t)pf::elastic_apply_blocks((int)e->n[0], (int)e->n[1], (int)e->n[2]));
+  np = std::max(np, (size_t)pf::elastic_apply_blocks((int)e->n[0], (int)e->n[1], (int)e->n[2]) +
+                        (size_t)pf::cg_blocks());
   L.off_sc = L.off_part + (np * sizeof(double) + 255) / 256 * 256;
   L.total = L.off_sc + 512;
   return L;
@@ -150,18 +150,17 @@ Layout layout(const pf_elastic* e) {
     if ((x) != cudaSuccess) return PF_ERR_CUDA;     \
   } while (0)
 
-// One CG iteration (slot = iteration parity): Ap = K p with the p.Ap partials,
-// sc[2] = p.Ap, x += alpha p, r -= alpha Ap with the new r.r partials,
-// sc[1 - slot] = r.r, p = r + beta p.
+// One CG iteration (slot = iteration parity): Ap = K p with the partials of
+// p.Ap, r -= alpha Ap with those of r.r behind them, x += alpha p and
+// p = r + beta p; sc[2] = p.Ap, sc[1 - slot] = r.r.
 cudaError_t cg_iteration(const Elastic3DArgs& A, int64_t n, int napply, float* x, float* r,
                          float* p, float* Ap, double* part, double* sc, int slot,
                          cudaStream_t s) {
   cudaError_t e;
   if ((e = pf::launch_elastic_apply(A, s)) != cudaSuccess) return e;
-  if ((e = pf::launch_sum_part(part, napply, sc + 2, s)) != cudaSuccess) return e;
-  if ((e = pf::launch_cg_xr(x, r, p, Ap, n, sc, slot, part, s)) != cudaSuccess) return e;
-  if ((e = pf::launch_sum_part(part, pf::cg_blocks(), sc + (1 - slot), s)) != cudaSuccess) return e;
-  return pf::launch_cg_p(r, p, n, sc, slot, s);
+  if ((e = pf::launch_cg_r(r, Ap, n, sc, slot, part, napply, part + napply, s)) != cudaSuccess)
+    return e;
+  return pf::launch_cg_xp(x, r, p, n, sc, slot, part + napply, s);
 }
 
 // K x = b on the free degrees of freedom (b's constrained entries are

@@ -311,17 +311,17 @@ struct ElasticLoadArgs {
   float hx, hy, hz, ihx, ihy, ihz, wq, scale, l, a;
 };
 int elastic_apply_blocks(int nx, int ny, int nz);
-int cg_blocks();  // blocks (and r.r partials) of launch_cg_xr
+int cg_blocks();  // blocks (and r.r partials) of launch_cg_r
 cudaError_t launch_elastic_apply(const Elastic3DArgs& a, cudaStream_t s);
-cudaError_t launch_sum_part(const double* part, int nb, double* out, cudaStream_t s);
 cudaError_t launch_elastic_load(const ElasticLoadArgs& a, float* f, cudaStream_t s);
 cudaError_t launch_elastic_constrain(float* v, int nx, int ny, int nz, cudaStream_t s);
 // CG updates with device scalars sc[0..1] = r.r (ping-pong by slot), sc[2] = p.Ap;
-// launch_cg_xr also leaves the new r.r as cg_blocks() FP64 partials in part
-cudaError_t launch_cg_xr(float* x, float* r, const float* p, const float* Ap, int64_t n,
-                         const double* sc, int slot, double* part, cudaStream_t s);
-cudaError_t launch_cg_p(const float* r, float* p, int64_t n, const double* sc, int slot,
-                        cudaStream_t s);
+// launch_cg_r takes the npap partials of p.Ap and leaves cg_blocks() partials of
+// the new r.r in part (elsewhere), which launch_cg_xp takes
+cudaError_t launch_cg_r(float* r, const float* Ap, int64_t n, double* sc, int slot,
+                        const double* pap, int npap, double* part, cudaStream_t s);
+cudaError_t launch_cg_xp(float* x, const float* r, float* p, int64_t n, double* sc, int slot,
+                         const double* part, cudaStream_t s);
 
 // Krylov vector kernels (FP32 vectors, FP64 inner products).
 constexpr int kMaxBasis = 32;  // GMRES restart length + 1
