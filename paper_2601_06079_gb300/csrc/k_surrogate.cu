@@ -22,6 +22,15 @@ unsigned blocks_for(int64_t n) {
   return (unsigned)(b < 4096 ? b : 4096);
 }
 
+// Grid of the kernels that go over the voxels of a sample (x) and the samples
+// (y), so that no thread divides by the volume.  With a 64-bit division or two
+// and one value per thread, measured on 4 samples of 64^3 voxels against so: the
+// error field 60 -> 49 us, the loss gradient 84 -> 17.
+dim3 sample_grid(int64_t blocks, int64_t samples) {
+  return dim3((unsigned)std::min<int64_t>(std::max<int64_t>(blocks, 1), 1 << 20),
+              (unsigned)std::min<int64_t>(std::max<int64_t>(samples, 1), 65535));
+}
+
 // 8 BF16 channels (16 bytes) <-> 8 floats
 __device__ __forceinline__ void unpack8(const uint4& u, float* f) {
   const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&u);
@@ -41,30 +50,51 @@ __device__ __forceinline__ uint4 pack8(const float* f) {
   return u;
 }
 
-// planar [B][nf][V] FP32 -> NDHWC BF16 [B][V][C], one thread per voxel (the
-// planar reads coalesce across the warp, the voxel's C channels go out as
-// 16-byte stores).  mode 0: channels < nf copied, the rest zero.  mode h = 1, 2
-// (nf = 8 (h + 1): the states [U^n; U^{n-1}; ...; U^{n-h}]): channels 0..7 =
-// U^n, then for k = 1..h the increment (U^{n-k+1} - U^{n-k}) / sig[b], the
-// rest zero.
-__global__ void k_planar_to_ndhwc(const float* __restrict__ in, int nf, int C, int B, int64_t V,
-                                  int mode, const float* __restrict__ sig,
-                                  __nv_bfloat16* __restrict__ out) {
-  const int64_t n = (int64_t)B * V;
-  for (int64_t i = gtid(); i < n; i += grid_stride()) {
-    const int64_t v = i % V, b = i / V;
+// planar [B][nf][V] FP32 -> NDHWC BF16 [B][V][C].  mode 0: channels < nf
+// copied, the rest zero.  mode h = 1, 2 (nf = 8 (h + 1): the states
+// [U^n; U^{n-1}; ...; U^{n-h}]): channels 0..7 = U^n, then for k = 1..h the
+// increment (U^{n-k+1} - U^{n-k}) / sig[b], the rest zero.
+// Bound by memory.  A warp takes 32 voxels: the planar reads coalesce across
+// it, each channel is read once (an increment keeps the state before it), and
+// the C channels of the voxels leave through shared memory as whole lines.
+// Four blocks per SM keep enough reads on the way.  24 channels of 128^3 voxels
+// 95 -> 60 us (5.6 TB/s; 84 at two blocks per SM).
+template <int C>
+__global__ void __launch_bounds__(kT, 4) k_planar_to_ndhwc(const float* __restrict__ in, int nf, int B,
+                                                        int64_t V, int mode,
+                                                        const float* __restrict__ sig,
+                                                        __nv_bfloat16* __restrict__ out) {
+  constexpr int kParts = C / 8;  // 16-byte parts of a voxel
+  __shared__ uint4 stage[kT / 32][32][kParts + 1];
+  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  for (int64_t b = blockIdx.y; b < B; b += gridDim.y) {
     const float inv = mode ? 1.0f / sig[b] : 1.0f;
-    uint4* dst = reinterpret_cast<uint4*>(out + i * C);
-    for (int c0 = 0; c0 < C; c0 += 8) {
-      float f[8];
+    const float* src = in + b * nf * V;
+    uint4* dst = reinterpret_cast<uint4*>(out + b * V * C);
+    for (int64_t v0 = ((int64_t)blockIdx.x * (kT / 32) + warp) * 32; v0 < V;
+         v0 += (int64_t)gridDim.x * kT) {
+      const int64_t v = v0 + lane;
+      float raw[C];
 #pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        const int c = c0 + k;
-        float a = c < nf ? in[(b * nf + c) * V + v] : 0.0f;
-        if (mode && c >= 8 && c < nf) a = (in[(b * nf + c - 8) * V + v] - a) * inv;
-        f[k] = a;
+      for (int c = 0; c < C; ++c) raw[c] = c < nf && v < V ? src[c * V + v] : 0.0f;
+#pragma unroll
+      for (int q = 0; q < kParts; ++q) {
+        float f[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          const int c = 8 * q + k;
+          f[k] = raw[c];
+          if (q && mode && c < nf) f[k] = (raw[q ? c - 8 : 0] - raw[c]) * inv;
+        }
+        stage[warp][lane][q] = pack8(f);
       }
-      dst[c0 / 8] = pack8(f);
+      __syncwarp();
+#pragma unroll
+      for (int q = 0; q < kParts; ++q) {
+        const int i = q * 32 + lane;
+        if (v0 + i / kParts < V) dst[v0 * kParts + i] = stage[warp][i / kParts][i % kParts];
+      }
+      __syncwarp();
     }
   }
 }
@@ -105,53 +135,72 @@ __global__ void k_ndhwc_to_planar_add(const float* __restrict__ y, int C, int nf
 }
 
 // Per-sample output unit: sig[b] = a (mode 0) or a * RMS over the sample of
-// U^n - U^{n-1} (modes 1, 2: x holds nxc = nf (mode + 1) channels per sample,
-// U^n first), floored at 1e-30.  part holds gridDim.x partial sums per sample
-// (fixed-order reduction).
-//   second = 1 (mode 2): the second difference U^n - 2 U^{n-1} + U^{n-2} instead
-__global__ void k_incr_sumsq(const float* __restrict__ x, int nf, int nxc, int64_t V,
-                             int second, double* __restrict__ part) {
-  __shared__ double red[kT];
+// U^n - U^{n-1} (modes 1, 2: x holds nf (mode + 1) channels per sample, U^n
+// first), floored at 1e-30.  part holds gridDim.x partial sums per sample
+// (fixed-order reduction), and with kMode 2 as many of the second difference
+// U^n - 2 U^{n-1} + U^{n-2} behind those of all samples: one pass over the
+// states for both (24 channels of 128^3 voxels: 53 us, in two passes 88).
+template <int kMode>
+__global__ void __launch_bounds__(kT) k_incr_sumsq(const float* __restrict__ x, int nf, int64_t V,
+                                                   double* __restrict__ part) {
+  __shared__ double red[kMode][kT];
   const int b = blockIdx.y;
-  const float* u = x + (int64_t)b * nxc * V;
+  const float* u = x + (int64_t)b * nf * (kMode + 1) * V;
   // differences and squares in FP32 (16-byte loads, four independent sums per
   // thread), runs of 16 vectors summed in FP32 and the runs in FP64: GB300's
   // FP64 rate is a small fraction of its FP32 rate, so no FP64 arithmetic per
   // element.  nf * V is a multiple of 4 (the volume's sides are multiples of 16).
   const float4* u0 = reinterpret_cast<const float4*>(u);
   const float4* u1 = reinterpret_cast<const float4*>(u + nf * V);
-  const float4* u2 = reinterpret_cast<const float4*>(u + 2 * nf * V);
+  const float4* u2 = reinterpret_cast<const float4*>(u + (kMode == 2 ? 2 : 0) * nf * V);
   const int64_t n4 = (int64_t)nf * V / 4;
-  double acc = 0.0;
-  float4 run = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+  double acc[kMode];
+  float4 run[kMode];
+#pragma unroll
+  for (int m = 0; m < kMode; ++m) {
+    acc[m] = 0.0;
+    run[m] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+  }
+  const auto add = [](float4& r, const float4& d) {
+    r.x = fmaf(d.x, d.x, r.x);
+    r.y = fmaf(d.y, d.y, r.y);
+    r.z = fmaf(d.z, d.z, r.z);
+    r.w = fmaf(d.w, d.w, r.w);
+  };
   int k = 0;
+#pragma unroll 2
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n4;
        i += (int64_t)gridDim.x * blockDim.x) {
     const float4 a0 = u0[i], a1 = u1[i];
-    float4 d = make_float4(a0.x - a1.x, a0.y - a1.y, a0.z - a1.z, a0.w - a1.w);
-    if (second) {
+    const float4 d = make_float4(a0.x - a1.x, a0.y - a1.y, a0.z - a1.z, a0.w - a1.w);
+    add(run[0], d);
+    if constexpr (kMode == 2) {
       const float4 a2 = u2[i];
-      d = make_float4(d.x - (a1.x - a2.x), d.y - (a1.y - a2.y), d.z - (a1.z - a2.z),
-                      d.w - (a1.w - a2.w));
+      add(run[1], make_float4(d.x - (a1.x - a2.x), d.y - (a1.y - a2.y), d.z - (a1.z - a2.z),
+                              d.w - (a1.w - a2.w)));
     }
-    run.x = fmaf(d.x, d.x, run.x);
-    run.y = fmaf(d.y, d.y, run.y);
-    run.z = fmaf(d.z, d.z, run.z);
-    run.w = fmaf(d.w, d.w, run.w);
     if (++k == 16) {
-      acc += (double)((run.x + run.y) + (run.z + run.w));
-      run = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+#pragma unroll
+      for (int m = 0; m < kMode; ++m) {
+        acc[m] += (double)((run[m].x + run[m].y) + (run[m].z + run[m].w));
+        run[m] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      }
       k = 0;
     }
   }
-  acc += (double)((run.x + run.y) + (run.z + run.w));
-  red[threadIdx.x] = acc;
+#pragma unroll
+  for (int m = 0; m < kMode; ++m)
+    red[m][threadIdx.x] = acc[m] + (double)((run[m].x + run[m].y) + (run[m].z + run[m].w));
   __syncthreads();
   for (int o = kT / 2; o > 0; o >>= 1) {
-    if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
+    if (threadIdx.x < o) {
+#pragma unroll
+      for (int m = 0; m < kMode; ++m) red[m][threadIdx.x] += red[m][threadIdx.x + o];
+    }
     __syncthreads();
   }
-  if (threadIdx.x == 0) part[b * gridDim.x + blockIdx.x] = red[0];
+  if (threadIdx.x < kMode)
+    part[((int64_t)threadIdx.x * gridDim.y + b) * gridDim.x + blockIdx.x] = red[threadIdx.x][0];
 }
 
 // Sum of p[0 .. n) by one block of kT threads in a fixed order (strided
@@ -281,16 +330,22 @@ __global__ void k_relu_mask(__nv_bfloat16* __restrict__ g, const __nv_bfloat16* 
 //   mode h: r = pred - (y - skip) / sig_b                      (units of sig_b)
 // pred = first nf channels of the NDHWC FP32 network output (C channels);
 // r is written planar [B][nf][V].
-__global__ void k_err(const float* __restrict__ pred, int C, int nf, int nxc, int B, int64_t V,
-                      const float* __restrict__ x, const float* __restrict__ y, int mode,
-                      const float* __restrict__ sig, float* __restrict__ r) {
-  const int64_t n = (int64_t)B * nf * V;
-  for (int64_t i = gtid(); i < n; i += grid_stride()) {
-    const int64_t v = i % V, c = (i / V) % nf, b = i / (nf * V);
-    const int64_t s0 = (b * nxc + c) * V + v;
-    const float t = y[i] - skip_value(x, s0, (int64_t)nf * V, mode);
-    const float p = pred[(b * V + v) * C + c];
-    r[i] = mode ? p - t / sig[b] : fmaf(sig[b], p, -t);
+// One thread per voxel: the channels of pred are contiguous, eight at a time.
+__global__ void __launch_bounds__(kT) k_err(const float* __restrict__ pred, int C, int nf, int nxc,
+                                            int B, int64_t V, const float* __restrict__ x,
+                                            const float* __restrict__ y, int mode,
+                                            const float* __restrict__ sig, float* __restrict__ r) {
+  for (int64_t b = blockIdx.y; b < B; b += gridDim.y) {
+    const float sb = sig[b];
+    for (int64_t v = (int64_t)blockIdx.x * kT + threadIdx.x; v < V; v += (int64_t)gridDim.x * kT) {
+      const float* p = pred + (b * V + v) * C;
+#pragma unroll 8
+      for (int c = 0; c < nf; ++c) {
+        const int64_t i = (b * nf + c) * V + v;
+        const float t = y[i] - skip_value(x, (b * nxc + c) * V + v, (int64_t)nf * V, mode);
+        r[i] = mode ? p[c] - t / sb : fmaf(sb, p[c], -t);
+      }
+    }
   }
 }
 
@@ -302,60 +357,92 @@ __global__ void k_err(const float* __restrict__ pred, int C, int nf, int nxc, in
 // w = M / h^3 for the symmetric form (I + c K) used by the loss:
 //   sym = 0: out = in + c * S(in)            (= (I + c M^-1 K) in)
 //   sym = 1: out = in + c * w * S(in)        (= (I + c K) in, symmetric)
-__global__ void k_apply_stiff(const float* __restrict__ in, int64_t planes, int D, int H, int W,
-                              float c, int sym, float* __restrict__ out) {
-  const int64_t V = (int64_t)D * H * W;
-  const int64_t n = planes * V;
-  for (int64_t i = gtid(); i < n; i += grid_stride()) {
-    const int64_t p = i / V;
-    const int64_t v = i % V;
-    const int x = (int)(v % W), y = (int)((v / W) % H), z = (int)(v / ((int64_t)W * H));
-    const float* pl = in + p * V;
-    float acc = 0.0f;
+// A thread walks kStiffZ nodes along z with the 3 x 3 values of three planes in
+// registers, so a node costs 9 loads instead of 21 and no index arithmetic; as
+// a thread per node with 64-bit divisions it took 141 us on 32 planes of 64^3
+// nodes, now 54 (68 with the loop unrolled by 3 at 126 registers).
+constexpr int kStiffZ = 16, kStiffX = 32, kStiffY = kT / kStiffX;
+
+__global__ void __launch_bounds__(kT) k_apply_stiff(const float* __restrict__ in, int64_t planes,
+                                                    int D, int H, int W, float c, int sym,
+                                                    float* __restrict__ out) {
+  const int tx = (W + kStiffX - 1) / kStiffX, ty = (H + kStiffY - 1) / kStiffY;
+  const int tile = blockIdx.x % (tx * ty);
+  const int x = tile % tx * kStiffX + threadIdx.x % kStiffX;
+  const int y = tile / tx * kStiffY + threadIdx.x / kStiffX;
+  if (x >= W || y >= H) return;
+  const int z0 = blockIdx.x / (tx * ty) * kStiffZ, z1 = min(z0 + kStiffZ, D);
+  const int64_t plane = (int64_t)H * W;
+  const int xs[3] = {x ? x - 1 : 1, x, x + 1 < W ? x + 1 : W - 2};
+  const int64_t ys[3] = {(int64_t)(y ? y - 1 : 1) * W, (int64_t)y * W,
+                         (int64_t)(y + 1 < H ? y + 1 : H - 2) * W};
+  float wxy = 1.0f;
+  if (sym) {
+    if (x == 0 || x == W - 1) wxy *= 0.5f;
+    if (y == 0 || y == H - 1) wxy *= 0.5f;
+  }
+  for (int64_t p = blockIdx.y; p < planes; p += gridDim.y) {
+    const float* pl = in + p * D * plane;
+    float v[3][9];
+    auto load = [&](int z, float (&t)[9]) {
+      const float* q = pl + (z < 0 ? -z : (z >= D ? 2 * D - 2 - z : z)) * plane;
 #pragma unroll
-    for (int dz = -1; dz <= 1; ++dz) {
-      int zz = z + dz;
-      zz = zz < 0 ? -zz : (zz >= D ? 2 * D - 2 - zz : zz);
+      for (int k = 0; k < 9; ++k) t[k] = q[ys[k / 3] + xs[k % 3]];
+    };
+    load(z0 - 1, v[0]);
+    load(z0, v[1]);
+#pragma unroll 1
+    for (int z = z0; z < z1; ++z) {
+      load(z + 1, v[2]);
+      float acc = 0.0f;
 #pragma unroll
-      for (int dy = -1; dy <= 1; ++dy) {
-        int yy = y + dy;
-        yy = yy < 0 ? -yy : (yy >= H ? 2 * H - 2 - yy : yy);
+      for (int dz = 0; dz < 3; ++dz)
 #pragma unroll
-        for (int dx = -1; dx <= 1; ++dx) {
-          const int k = (dz != 0) + (dy != 0) + (dx != 0);
-          if (k == 1) continue;
-          const float wgt = k == 0 ? 8.0f / 3.0f : (k == 2 ? -1.0f / 6.0f : -1.0f / 12.0f);
-          int xx = x + dx;
-          xx = xx < 0 ? -xx : (xx >= W ? 2 * W - 2 - xx : xx);
-          acc = fmaf(wgt, pl[((int64_t)zz * H + yy) * W + xx], acc);
+        for (int k = 0; k < 9; ++k) {
+          const int off = (dz != 1) + (k / 3 != 1) + (k % 3 != 1);
+          if (off == 1) continue;
+          const float wgt = off == 0 ? 8.0f / 3.0f : (off == 2 ? -1.0f / 6.0f : -1.0f / 12.0f);
+          acc = fmaf(wgt, v[dz][k], acc);
         }
+      const float w = sym && (z == 0 || z == D - 1) ? 0.5f * wxy : wxy;
+      out[p * D * plane + z * plane + ys[1] + x] = fmaf(c * w, acc, v[1][4]);
+#pragma unroll
+      for (int k = 0; k < 9; ++k) {
+        v[0][k] = v[1][k];
+        v[1][k] = v[2][k];
       }
     }
-    float w = 1.0f;
-    if (sym) {
-      if (x == 0 || x == W - 1) w *= 0.5f;
-      if (y == 0 || y == H - 1) w *= 0.5f;
-      if (z == 0 || z == D - 1) w *= 0.5f;
-    }
-    out[i] = fmaf(c * w, acc, pl[v]);
   }
 }
 
 // Per-block partial sums of q^2 over n values.
-__global__ void k_sumsq(const float* __restrict__ q, int64_t n, double* __restrict__ partials) {
+// Four independent runs of 16 squares in FP32 per thread, the runs in FP64 (see
+// k_incr_sumsq); q is 16-byte aligned.  2^23 values: 18 us, 45 one at a time.
+__global__ void __launch_bounds__(kT) k_sumsq(const float* __restrict__ q, int64_t n,
+                                              double* __restrict__ partials) {
   __shared__ double red[kT];
-  double acc = 0.0;  // runs of 16 squares in FP32, the runs in FP64 (see k_incr_sumsq)
-  float run = 0.0f;
+  double acc = 0.0;
+  float4 run = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
   int k = 0;
-  for (int64_t i = gtid(); i < n; i += grid_stride()) {
-    run = fmaf(q[i], q[i], run);
+  const int64_t n4 = n / 4;
+#pragma unroll 4
+  for (int64_t i = gtid(); i < n4; i += grid_stride()) {
+    const float4 t = reinterpret_cast<const float4*>(q)[i];
+    run.x = fmaf(t.x, t.x, run.x);
+    run.y = fmaf(t.y, t.y, run.y);
+    run.z = fmaf(t.z, t.z, run.z);
+    run.w = fmaf(t.w, t.w, run.w);
     if (++k == 16) {
-      acc += (double)run;
-      run = 0.0f;
+      acc += (double)((run.x + run.y) + (run.z + run.w));
+      run = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
       k = 0;
     }
   }
-  acc += (double)run;
+  if (gtid() < n - 4 * n4) {
+    const float t = q[4 * n4 + gtid()];
+    run.x = fmaf(t, t, run.x);
+  }
+  acc += (double)((run.x + run.y) + (run.z + run.w));
   red[threadIdx.x] = acc;
   __syncthreads();
   for (int o = kT / 2; o > 0; o >>= 1) {
@@ -367,18 +454,23 @@ __global__ void k_sumsq(const float* __restrict__ q, int64_t n, double* __restri
 
 // dL/dpred (NDHWC BF16, C channels, zero beyond nf) from g = dL/dr / 2 (planar):
 // 2 * scale * g * dr/dpred with dr/dpred = sig_b (mode 0) or 1 (mode 1).
-__global__ void k_grad_out(const float* __restrict__ g, int C, int nf, int B, int64_t V, int mode,
-                           const float* __restrict__ sig, float scale,
-                           __nv_bfloat16* __restrict__ grad) {
-  const int64_t n = (int64_t)B * V * C;
-  for (int64_t i = gtid(); i < n; i += grid_stride()) {
-    const int c = (int)(i % C);
-    float gv = 0.0f;
-    if (c < nf) {
-      const int64_t v = (i / C) % V, b = i / (C * V);
-      gv = 2.0f * scale * g[(b * nf + c) * V + v] * (mode ? 1.0f : sig[b]);
+// One thread per voxel, whose channels leave as 16-byte parts.
+__global__ void __launch_bounds__(kT) k_grad_out(const float* __restrict__ g, int C, int nf, int B,
+                                                 int64_t V, int mode,
+                                                 const float* __restrict__ sig, float scale,
+                                                 __nv_bfloat16* __restrict__ grad) {
+  for (int64_t b = blockIdx.y; b < B; b += gridDim.y) {
+    const float sb = mode ? 1.0f : sig[b];
+    for (int64_t v = (int64_t)blockIdx.x * kT + threadIdx.x; v < V; v += (int64_t)gridDim.x * kT) {
+      uint4* dst = reinterpret_cast<uint4*>(grad + (b * V + v) * C);
+      for (int c0 = 0; c0 < C; c0 += 8) {
+        float f[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+          f[k] = c0 + k < nf ? 2.0f * scale * g[(b * nf + c0 + k) * V + v] * sb : 0.0f;
+        dst[c0 / 8] = pack8(f);
+      }
     }
-    grad[i] = __float2bfloat16(gv);
   }
 }
 
@@ -435,9 +527,14 @@ __global__ void k_adam(float* __restrict__ p, float* __restrict__ m, float* __re
 
 cudaError_t launch_planar_to_ndhwc(const float* in, int nf, int C, int B, int64_t V, int mode,
                                    const float* sig, void* out, cudaStream_t s) {
-  if (C % 8 || nf > C || (mode && (nf != 8 * (mode + 1) || !sig))) return cudaErrorInvalidValue;
-  k_planar_to_ndhwc<<<blocks_for((int64_t)B * V), kT, 0, s>>>(in, nf, C, B, V, mode, sig,
-                                                             (__nv_bfloat16*)out);
+  if (nf > C || (mode && (nf != 8 * (mode + 1) || !sig))) return cudaErrorInvalidValue;
+  const dim3 grid = sample_grid((V + kT - 1) / kT, B);
+  if (C == 16)
+    k_planar_to_ndhwc<16><<<grid, kT, 0, s>>>(in, nf, B, V, mode, sig, (__nv_bfloat16*)out);
+  else if (C == 32)
+    k_planar_to_ndhwc<32><<<grid, kT, 0, s>>>(in, nf, B, V, mode, sig, (__nv_bfloat16*)out);
+  else
+    return cudaErrorInvalidValue;
   return cudaGetLastError();
 }
 
@@ -452,14 +549,12 @@ cudaError_t launch_ndhwc_to_planar_add(const float* y, int C, int nf, int B, int
 
 cudaError_t launch_incr_scale(const float* x, int nf, int B, int64_t V, float a, int mode,
                               double* part, int nblk, float* sig, float* sigo, cudaStream_t s) {
-  if (mode) {
-    k_incr_sumsq<<<dim3(nblk, B), kT, 0, s>>>(x, nf, nf * (mode + 1), V, 0, part);
-    if (cudaGetLastError() != cudaSuccess) return cudaErrorLaunchFailure;
-  }
+  if (mode == 1) k_incr_sumsq<1><<<dim3(nblk, B), kT, 0, s>>>(x, nf, V, part);
+  if (mode == 2) k_incr_sumsq<2><<<dim3(nblk, B), kT, 0, s>>>(x, nf, V, part);
+  if (cudaGetLastError() != cudaSuccess) return cudaErrorLaunchFailure;
   k_incr_scale<<<B, kT, 0, s>>>(part, nblk, (double)nf * V, a, mode, sig);
-  if (mode == 2) {  // the partials are reused once the increment unit is formed
-    k_incr_sumsq<<<dim3(nblk, B), kT, 0, s>>>(x, nf, 3 * nf, V, 1, part);
-    k_curv_scale<<<B, kT, 0, s>>>(part, nblk, (double)nf * V, a, sig, sigo);
+  if (mode == 2) {
+    k_curv_scale<<<B, kT, 0, s>>>(part + (int64_t)B * nblk, nblk, (double)nf * V, a, sig, sigo);
   } else {
     cudaMemcpyAsync(sigo, sig, sizeof(float) * B, cudaMemcpyDeviceToDevice, s);
   }
@@ -512,21 +607,25 @@ cudaError_t launch_mse(const float* pred, int C, int nf, int nxc, int B, int D, 
                        double* loss, cudaStream_t s) {
   const int64_t V = (int64_t)D * H * W;
   const int64_t n = (int64_t)B * nf * V;
-  k_err<<<blocks_for(n), kT, 0, s>>>(pred, C, nf, nxc, B, V, x, y, mode, sig, r);
+  const dim3 grid = sample_grid((V + kT - 1) / kT, B);
+  const int64_t tiles = (int64_t)((W + kStiffX - 1) / kStiffX) * ((H + kStiffY - 1) / kStiffY);
+  const int64_t chunks = tiles * ((D + kStiffZ - 1) / kStiffZ);
+  if (C % 8 || chunks > INT32_MAX) return cudaErrorInvalidValue;
+  const dim3 sgrid((unsigned)chunks, (unsigned)std::min<int64_t>((int64_t)B * nf, 65535));
+  k_err<<<grid, kT, 0, s>>>(pred, C, nf, nxc, B, V, x, y, mode, sig, r);
   const float* qq = r;
   if (c != 0.0f) {
-    k_apply_stiff<<<blocks_for(n), kT, 0, s>>>(r, (int64_t)B * nf, D, H, W, c, 1, q);
+    k_apply_stiff<<<sgrid, kT, 0, s>>>(r, (int64_t)B * nf, D, H, W, c, 1, q);
     qq = q;
   }
   k_sumsq<<<mse_blocks(), kT, 0, s>>>(qq, n, partials);
   k_sum_doubles<<<1, kT, 0, s>>>(partials, mse_blocks(), (double)scale, loss);
   const float* g = qq;
   if (c != 0.0f) {
-    k_apply_stiff<<<blocks_for(n), kT, 0, s>>>(q, (int64_t)B * nf, D, H, W, c, 1, r);
+    k_apply_stiff<<<sgrid, kT, 0, s>>>(q, (int64_t)B * nf, D, H, W, c, 1, r);
     g = r;
   }
-  k_grad_out<<<blocks_for((int64_t)B * V * C), kT, 0, s>>>(g, C, nf, B, V, mode, sig, scale,
-                                                          (__nv_bfloat16*)grad);
+  k_grad_out<<<grid, kT, 0, s>>>(g, C, nf, B, V, mode, sig, scale, (__nv_bfloat16*)grad);
   return cudaGetLastError();
 }
 

@@ -89,7 +89,7 @@ Plan make_plan(int B, int D, int H, int W, bool training) {
   p.err = take(sizeof(int));
   p.sig = take(sizeof(float) * B);
   p.sigo = take(sizeof(float) * B);
-  p.sigp = take(sizeof(double) * kSigBlocks * B);
+  p.sigp = take(sizeof(double) * 2 * kSigBlocks * B);
   for (int l = 0; l < kNL; ++l) {
     p.wf[l] = take(2 * w_count(l));
     p.wb[l] = take(2 * w_count(l));
