@@ -14,8 +14,8 @@ trajectories the L2 is flushed by writing a 512 MiB buffer.
   python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
 
 The line also carries "forms": each chosen execution form against its plain
-counterpart on the same inputs at the same accuracy -- the fused graph-replayed
-CH step vs one launch per step vs the plain two-pass step (2048^2); the
+counterpart on the same inputs at the same accuracy -- the CH steps in
+one launch vs one launch per step vs the plain two-pass step (2048^2); the
 256-instance AC ensemble in one persistent launch vs per-step vs per-instance
 launches; the coupled Allen-Cahn / Cahn-Hilliard step (2048^2); the checkpointed adjoint vs the forward trajectory (512^2, 2000
 steps); and Newton from the learned warm start vs the plain U^n start for 200
@@ -50,11 +50,12 @@ N_TSTEPS = 10_000
 PAR = dict(W=1.0, kappa=0.5, mobility=1.0, dt=1e-3)
 DOF_PER_NODE = 2
 ALG_BYTES_PER_NODE_STEP = 8  # read c, write c; mu never leaves the chip
-# FP32 flop per node of the fused CH step, counted from the kernel's sweep (one
-# lane = two nodes): 28 packed FMA (x 2 lanes x 2 flop) + 13 packed add/sub
-# (x 2) + 8 scalar add/sub = 146 per lane-row; the warm-up rows of each band
-# and the halo lanes of each strip are excluded (they repeat this work).
-FLOP_PER_NODE_STEP = 73
+# FP32 flop per node of the fused CH step, counted from the sweep's row (a pair
+# of nodes; square cells, symmetric well): 18 packed FMA (x 4 flop), 5 packed
+# multiplications and 8 packed additions (x 2), 4 scalar FMA (x 2) and 6 scalar
+# additions = 112; the warm-up rows of each band and the halo of each tile are
+# excluded (they repeat this work).
+FLOP_PER_NODE_STEP = 56
 NOMINAL_FP32_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12  # FP32 lanes x 2 flop x max SM clock
 _FP32_PEAK = {}
 
@@ -76,7 +77,7 @@ def fp32_peak(dev, stream):
         _FP32_PEAK[dev] = max(vals)
     return _FP32_PEAK[dev]
 WORKLOAD = "ch2d_2048x2048_10000steps"
-KERNEL_SRC = os.path.join(ROOT, "paper_2601_06079_gb300", "csrc", "k_explicit2d.cu")
+KERNEL_SRC = os.path.join(ROOT, "paper_2601_06079_gb300", "csrc", "k_onchip2d.cu")
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "ch2d_2048_dram_traffic.json")
 
 
@@ -124,7 +125,7 @@ def _peaks():
 
 
 def _traffic():
-    """DRAM bytes per launch of the step kernel from the committed ncu summary,
+    """DRAM bytes per launch of the trajectory kernel from a committed ncu summary,
     null when the kernel source changed since the capture."""
     try:
         with open(TRAFFIC_FILE) as f:
@@ -278,11 +279,12 @@ def run_ours(args):
                            "end_energy": E, "end_mass": M}),
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak, "traffic": _traffic(),
-                     "kernel": "k_explicit2d<CH> (fused mu + c update)",
+                     "kernel": "k_onchip2d<CH> (all steps in one launch, state on chip)",
                      "peak_source": f"{peak_kind} hbm_gbs",
+                     # per time step; one launch makes all of a trajectory's
                      "per_launch_s": step_launch_s,
                      "alg_bytes_per_launch": ALG_BYTES_PER_NODE_STEP * nodes},
-        # both planes stay in L2 over a trajectory: the FP32 pipe binds, so the
+        # the state stays on chip over a trajectory: the FP32 pipe binds, so the
         # same kernel against the measured FP32 FMA peak
         "roofline_alu": {"bound": "alu", "achieved": alu_achieved, "peak": alu_peak,
                          "unit": "TFLOP/s", "frac": alu_achieved / alu_peak,
@@ -291,7 +293,8 @@ def run_ours(args):
                          "nominal_peak": NOMINAL_FP32_TFLOPS},
         "e2e": {"value": e2e_value, "unit": "DOF-steps/s",
                 "h2d_bytes_per_step": nodes * 4, "d2h_bytes_per_step": nodes * 4 + 16},
-        "gpu_launches": args.steps * (N_TSTEPS + 4),
+        # one launch for all time steps, two for the energy and mass
+        "gpu_launches": args.steps * 3,
         "clocks": clk.summary(),
     }
     if not args.no_forms:
@@ -331,7 +334,7 @@ def _timed(stream, fn, flush=None):
 
 
 def forms_explicit(dev, stream, flush, c0_host, n_steps=2048):
-    """CH 2048^2: fused + graph (default) vs fused per launch vs plain two-pass."""
+    """CH 2048^2: the default form vs fused per launch vs plain two-pass."""
     import torch
 
     import paper_2601_06079_gb300 as pf

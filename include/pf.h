@@ -172,7 +172,9 @@ pf_status pf_set_form(pf_ctx* ctx, int form);
  * guess: device initial Newton iterate for the FIRST step (NULL = U^n); later
  * steps start from their U^n.  opts may be NULL (defaults); stats (host) may be
  * NULL.  Synchronises the stream.  PF_ERR_NOT_CONVERGED: state holds the last
- * iterate and stats the counts so far. */
+ * iterate and stats the counts so far.  2-D meshes of up to 2^20 nodes make all
+ * steps in one launch whose blocks wait for each other; PF_ERR_TIMEOUT if such a
+ * wait expired (about one second). */
 pf_status pf_step_implicit(pf_ctx* ctx, float* state, int64_t n_steps, const float* guess,
                            const pf_newton_opts* opts, pf_newton_stats* stats);
 
@@ -229,7 +231,8 @@ pf_status pf_adjoint_workspace(pf_ctx* ctx, int64_t n_steps, int ckpt_every, siz
  *   grad_mobility       device, N doubles: dLoss/dm_i for the mobility field (may be NULL)
  *   grad_state0         device, N floats: dLoss/dc^0 (may be NULL)
  * With no mobility field bound the field is taken as 1 everywhere.  State and
- * adjoint are FP32, all gradient sums FP64.  Synchronises the stream. */
+ * adjoint are FP32; gradient sums are compensated FP32 pairs (about 48 bits),
+ * finished in FP64.  Synchronises the stream. */
 pf_status pf_adjoint(pf_ctx* ctx, const float* state0, const float* target, int64_t n_steps,
                      int ckpt_every, int nodal_loss, void* adj_ws, size_t adj_bytes, double* loss,
                      double* grad_scalars, double* grad_mobility, float* grad_state0);
@@ -269,8 +272,9 @@ enum {
 
 /* Set the schedule of every instance: band height ty[i] (6, 12 or 24 rows per
  * warp task) and L2 policy l2[i] (PF_L2_*).  Either may be NULL (kept).  The
- * schedule changes no result.  Needs the workspace and parameters; uploads the
- * task list and synchronises the stream.  Out-of-range values: PF_ERR_ARG. */
+ * schedule changes no result, and applies to steps with the planes in memory
+ * (PF_ENS_PERSISTENT on chip has none).  Needs the workspace and parameters;
+ * uploads the task list and synchronises the stream.  Out-of-range values: PF_ERR_ARG. */
 pf_status pf_set_ensemble_schedule(pf_ctx* ctx, const int* ty, const int* l2);
 
 /* Autotuner of the schedule per size class (no counterpart in the paper).

@@ -348,7 +348,7 @@ __global__ void __launch_bounds__(kThreads) k_elastic_load(ElasticLoadArgs a, fl
 // x is moved along where p is read anyway, so an iteration passes over eight
 // vectors instead of nine.  Each block adds the partials of the launch before
 // it for itself, and block 0 leaves the sum in sc: as launches of their own
-// the two sums took 6 us each of a 90 us iteration on a 129^3 mesh, and
+// the two sums took 6 us each of a 74 us iteration on a 129^3 mesh, and
 // finished by the last block of the launch that makes them they cost its
 // blocks a fence each, as much again.  One block of 1024 threads per SM keeps
 // the sum to one per SM.  A solve on 129^3 nodes: 51.5 ms with two more launches
