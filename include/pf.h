@@ -231,8 +231,10 @@ pf_status pf_adjoint_workspace(pf_ctx* ctx, int64_t n_steps, int ckpt_every, siz
  *   grad_mobility       device, N doubles: dLoss/dm_i for the mobility field (may be NULL)
  *   grad_state0         device, N floats: dLoss/dc^0 (may be NULL)
  * With no mobility field bound the field is taken as 1 everywhere.  State and
- * adjoint are FP32; gradient sums are compensated FP32 pairs (about 48 bits),
- * finished in FP64.  Synchronises the stream. */
+ * adjoint are FP32.  The scalars' sums take the products of two nodes in FP32,
+ * then compensated FP32 pairs (about 48 bits) over nodes and steps, and finish in
+ * FP64; a node's mobility gradient is such a pair over the steps.  Synchronises
+ * the stream. */
 pf_status pf_adjoint(pf_ctx* ctx, const float* state0, const float* target, int64_t n_steps,
                      int ckpt_every, int nodal_loss, void* adj_ws, size_t adj_bytes, double* loss,
                      double* grad_scalars, double* grad_mobility, float* grad_state0);

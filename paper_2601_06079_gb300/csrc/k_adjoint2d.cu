@@ -26,6 +26,23 @@
 // 2 products per direction and element instead of 4 points' gradients; so does
 // the mobility's gradient (products of differences, projected along one axis).
 //
+// Constants.  dLoss/dM = (kappa dLoss/dkappa + W dLoss/dW) / M changes sign in
+// the course of a trajectory; near there it keeps 1e-8 only if the two parts do,
+// and a factor rounded once to FP32 (6e-8) costs each of them more.  So (see
+// pack_ch_mob):
+//   - g_hi is 1 / (1 + rho) for the rounded rho: interpolated constants stay exact;
+//   - the polynomials keep their coefficients, the stiffness stencil is divided by
+//     its corner weight (8 and -1 on square cells), and the factors in front of
+//     them meet at the node: r = kappa K : F, the fluxes' and the time step's, each
+//     an FP32 pair hi + lo in two FMAs;
+//   - dLoss/dM's sum is not taken: it follows from the other two.
+// dLoss/dM's error against FP64 over 60 meshes of 41 x 70 to 488 x 168 nodes and
+// 100 to 1,000 steps, as a share of (|kappa dLoss/dkappa| + |W dLoss/dW|) / M:
+// median 5.7e-9, largest 2.7e-8 (the rounding of the states); with g_hi of its own
+// and every factor rounded once 3.2e-8 and 1.2e-7; with node tiles, differences and
+// dt as the one rounded factor that mattered 1.1e-8 and 3.3e-8.  512^2 takes the
+// same time with the pairs and without (2,000 steps and their reverse: 25.8 ms).
+//
 // Measured at 512^2 (us per step, graph replay): forward 5.7 with 32 x 16 node
 // tiles in shared memory (element passes into corner arrays, four barriers), 2.9
 // so; reverse 13.6, 7.1 so.  Both are latency-bound there (8 warps per SM); the
@@ -97,7 +114,7 @@ struct Stencil {
   }
 };
 
-// m^-1 F(c) and m^-1 K c, row by row
+// F and K c, row by row, without their factors (ChMobArgs)
 struct Potential {
   u64 c1, c2, w1, w2, am, ap, tl, th;  // rows k-1, k-2 of c; their west + east sums
   u64 g[4];                            // Gauss values of the last element row
@@ -177,18 +194,20 @@ struct Mobility {
   }
 };
 
-// m^-1 K_M u: the shares of node row k-1 from the element rows above and below
+// m^-1 K_M u without its factors: the shares of node row k-1 from the fluxes
+// along x (ox) and y (oy) of the element rows above and below
 struct Flux {
   u64 X, Y;  // carried from the element row above
   template <bool kNode>
   __device__ __forceinline__ void take(const u64 (&dx)[2], const u64 (&dy)[2], const u64 (&mx)[2],
-                                       const u64 (&my)[2], u64 rho, u64 cX, u64 cY, u64& out) {
+                                       const u64 (&my)[2], u64 rho, u64& ox, u64& oy) {
     const u64 f0 = mul2(dx[0], mx[0]), f1 = mul2(dx[1], mx[1]);
     const u64 T = back_x(mul2(dy[0], my[0]), mul2(dy[1], my[1]), rho);
     if constexpr (kNode) {
       const u64 S = add2(fma2(rho, f1, f0), X);
       const u64 W = pk(from_left(phi(S)), plo(S));  // the element left of each column
-      out = fma2(cY, sub2(Y, T), mul2(cX, sub2(W, S)));
+      ox = sub2(W, S);
+      oy = sub2(Y, T);
     }
     X = fma2(rho, f0, f1);
     Y = T;
@@ -219,13 +238,21 @@ struct Lane {
   }
 };
 
+// a v + b u, the factors as pairs hi + lo
+__device__ __forceinline__ u64 scaled(const float (&a)[2], u64 v, const float (&b)[2], u64 u) {
+  return fma2(bc(b[0]), u, fma2(bc(a[0]), v, fma2(bc(b[1]), u, mul2(bc(a[1]), v))));
+}
+// v + r u
+__device__ __forceinline__ u64 with(u64 v, u64 u, const float (&r)[2]) {
+  return fma2(bc(r[0]), u, fma2(bc(r[1]), u, v));
+}
+
 __global__ void __launch_bounds__(kWarps * 32) k_ch_mob_step(const ChMobArgs a, float* out) {
   const int nx = a.nx, ny = a.ny;
   const int y0 = (block_row() * kWarps + (threadIdx.x >> 5)) * kTYFwd;
   if (y0 >= ny) return;
   const Lane L(nx);
-  const u64 rho = bc(kGLo / kGHi), kappa = bc(a.kappa);
-  const u64 cX = bc(-a.dt * a.cX), cY = bc(-a.dt * a.cY);
+  const u64 rho = bc(kGLo / kGHi);
   u64 nc[kAhead], nm[kAhead];
   const auto load = [&](int j, int k) {  // row y0 - 2 + k into slot j
     const int64_t row = (int64_t)reflect(y0 - 2 + k, ny) * nx;
@@ -249,33 +276,51 @@ __global__ void __launch_bounds__(kWarps * 32) k_ch_mob_step(const ChMobArgs a, 
     load(k % kAhead, k + kAhead);
     cc[k % 3] = c.v;
   };
-  u64 dx[2], dy[2], mx[2], my[2], kw;
+  u64 dx[2], dy[2], mx[2], my[2], ox, oy;
   next(0);
   pot.start(c, plo(rho));
   next(1);
   pot.take<false>(c, a, rho, F, Kc);
   next(2);
   pot.take<true>(c, a, rho, F, Kc);  // mu of row y0 - 1
-  dif.start(row_of(fma2(kappa, Kc, F)));
+  dif.start(row_of(with(F, Kc, a.r)));
   mob.start(m1);
 #pragma unroll
   for (int k = 3; k < kTYFwd + 4; ++k) {
     next(k);
     pot.take<true>(c, a, rho, F, Kc);  // mu of row y0 - 3 + k
-    dif.take(row_of(fma2(kappa, Kc, F)), rho, dx, dy);
+    dif.take(row_of(with(F, Kc, a.r)), rho, dx, dy);
     mob.take(m1, rho, mx, my);
     if (k == 3) {
-      flux.take<false>(dx, dy, mx, my, rho, cX, cY, kw);
+      flux.take<false>(dx, dy, mx, my, rho, ox, oy);
     } else {
-      flux.take<true>(dx, dy, mx, my, rho, cX, cY, kw);
+      flux.take<true>(dx, dy, mx, my, rho, ox, oy);
       const int y = y0 + k - 4;
-      if (L.writer && y < ny) L.store(out + (int64_t)y * nx, nx, add2(cc[(k - 2) % 3], kw));
+      if (L.writer && y < ny) L.store(out + (int64_t)y * nx, nx, add2(cc[(k - 2) % 3], scaled(a.fx, ox, a.fy, oy)));
     }
   }
 }
 
-// The reverse step.  acc: per warp three compensated FP32 pairs (hi, lo) of the
-// sums for kappa, W and M over all steps, the factors left to the end.
+// hi + lo, a sum with the rounding errors of its additions in lo
+struct Pair {
+  float hi, lo;
+  __device__ __forceinline__ void add(float x) {
+    const float t = hi + x, bp = t - hi;
+    lo += (hi - (t - bp)) + (x - bp);
+    hi = t;
+  }
+};
+__device__ __forceinline__ Pair runs(const u64 (&d)[2]) {
+  Pair p{plo(d[0]), 0.0f};
+  p.add(phi(d[0]));
+  p.add(plo(d[1]));
+  p.add(phi(d[1]));
+  return p;
+}
+
+// The reverse step.  acc: per warp two compensated FP32 pairs (hi, lo) of the
+// sums for kappa and W over all steps, the factors left to the end.  Two rows'
+// products of a column are one FP32 run; runs, lanes and steps add up as pairs.
 __global__ void __launch_bounds__(kWarps * 32)
     k_ch_adj_step(const ChMobArgs a, const float* yin, float* yout, float* grad_hi, float* grad_lo,
                   float2* acc) {
@@ -284,8 +329,7 @@ __global__ void __launch_bounds__(kWarps * 32)
   const int y0 = band * kTYRev;
   if (y0 >= ny) return;
   const Lane L(nx);
-  const u64 rho = bc(kGLo / kGHi), kappa = bc(a.kappa), ndt = bc(-a.dt);
-  const u64 cX = bc(a.cX), cY = bc(a.cY), gX = bc(a.gX), gY = bc(a.gY);
+  const u64 rho = bc(kGLo / kGHi), gX = bc(a.gX), gY = bc(a.gY);
   const u64 s0 = bc(a.h[0]), s1 = bc(a.h[1]), s2 = bc(a.h[2]);
   const Stencil K(a.k);
   u64 nc[kAhead], nm[kAhead], nyv[kAhead];
@@ -311,7 +355,7 @@ __global__ void __launch_bounds__(kWarps * 32)
   u64 wa = 0, wb = 0, hl = 0, hh = 0;  // x-interpolants of w; F' w's carry
   u64 gx = 0, gy = 0;                  // carries of the mobility gradient
   u64 px[2], py[2];                    // y's differences in element row (k-2, k-1)
-  u64 dK = 0, dW = 0, dM = 0;
+  u64 dK[2] = {0, 0}, dW[2] = {0, 0};  // rows 0 and 1, rows 2 and 3 of the band
   Row c, m, y;
   u64 yy[3], F, Kc, gq[4];
   const auto next = [&](int k) {
@@ -321,7 +365,7 @@ __global__ void __launch_bounds__(kWarps * 32)
     load(k % kAhead, k + kAhead);
     yy[k % 3] = y.v;
   };
-  u64 ex[2], ey[2], mx[2], my[2], w;
+  u64 ex[2], ey[2], mx[2], my[2], ox, oy;
   next(0);
   pot.start(c, plo(rho));
   dy_.start(y);
@@ -330,7 +374,7 @@ __global__ void __launch_bounds__(kWarps * 32)
   pot.take<false>(c, a, rho, F, Kc);
   dy_.take(y, rho, ex, ey);
   mob.take(m, rho, mx, my);
-  flux.take<false>(ex, ey, mx, my, rho, cX, cY, w);
+  flux.take<false>(ex, ey, mx, my, rho, ox, oy);
 #pragma unroll
   for (int k = 2; k < kTYRev + 4; ++k) {
     // row k is y0 - 2 + k: mu and w of the row before it
@@ -344,15 +388,16 @@ __global__ void __launch_bounds__(kWarps * 32)
     pot.take<true>(c, a, rho, F, Kc);
     dy_.take(y, rho, ex, ey);
     mob.take(m, rho, mx, my);
-    flux.take<true>(ex, ey, mx, my, rho, cX, cY, w);
+    flux.take<true>(ex, ey, mx, my, rho, ox, oy);
+    const u64 w = with(ox, oy, a.ay);  // without cW
     const Row wr = row_of(w);
-    const u64 mu = fma2(kappa, Kc, F), vw = beside(wr);
+    const u64 mu = with(F, Kc, a.r), vw = beside(wr);
     const int yr = y0 - 3 + k;  // the row of mu and w
     if (k >= 3 && k < kTYRev + 3 && yr < ny) {
       const u64 fw = mul2(mul2(fxp, bc(yr == 0 || yr == ny - 1 ? 0.5f : 1.0f)), w);
-      dK = fma2(fw, Kc, dK);
-      dW = fma2(fw, F, dW);
-      dM = fma2(fw, mu, dM);
+      const int run = (k - 3) / 2;
+      dK[run] = fma2(fw, Kc, dK[run]);
+      dW[run] = fma2(fw, F, dW[run]);
     }
     u64 na, nb;
     along_x(wr, plo(rho), na, nb);
@@ -371,13 +416,14 @@ __global__ void __launch_bounds__(kWarps * 32)
       if (k >= 4) {
         const int yo = y0 + k - 4;  // the finished row
         const u64 H = back_x(add2(fma2(rho, h[1], h[0]), hl), add2(fma2(rho, h[3], h[2]), hh), rho);
-        const u64 Hw = fma2(kappa, K(w2, w1, w, v2, v1, vw), H);
+        const u64 Hw = with(H, K(w2, w1, w, v2, v1, vw), a.r);
         const u64 S = add2(fma2(rho, q1, q0), gx);
         const u64 both = add2(S, pk(from_left(phi(S)), plo(S)));  // elements right and left
         const u64 G = fma2(gY, add2(gy, T), mul2(gX, both));
         if (L.writer && yo < ny) {
           const int64_t row = (int64_t)yo * nx;
-          L.store(yout + row, nx, fma2(ndt, Hw, yy[(k - 2) % 3]));
+          L.store(yout + row, nx,
+                  fma2(bc(a.n[0]), Hw, fma2(bc(a.n[1]), Hw, yy[(k - 2) % 3])));
           if (grad_hi) {
             const u64 v = mul2(mul2(fxp, bc(yo == 0 || yo == ny - 1 ? 0.5f : 1.0f)), G);
 #pragma unroll
@@ -406,43 +452,49 @@ __global__ void __launch_bounds__(kWarps * 32)
   }
   // the warp's sums, into its pairs (Knuth's two-sum; FP64 only at the end: an
   // FP64 instruction takes an SM 16 cycles per warp)
-  float v[3] = {plo(dK) + phi(dK), plo(dW) + phi(dW), plo(dM) + phi(dM)};
+  static_assert(kTYRev == 4, "two runs of two rows");
+  Pair v[2] = {runs(dK), runs(dW)};
 #pragma unroll
-  for (int j = 0; j < 3; ++j) {
+  for (int o = 16; o > 0; o >>= 1) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v[j] += __shfl_down_sync(kFull, v[j], o);
+    for (int j = 0; j < 2; ++j) {
+      const float h = __shfl_down_sync(kFull, v[j].hi, o);
+      v[j].lo += __shfl_down_sync(kFull, v[j].lo, o);
+      v[j].add(h);
+    }
   }
   if ((threadIdx.x & 31) == 0) {
-    float2* p = acc + 3 * ((int64_t)band * gridDim.x + blockIdx.x);
+    float2* p = acc + 2 * ((int64_t)band * gridDim.x + blockIdx.x);
 #pragma unroll
-    for (int j = 0; j < 3; ++j) {
+    for (int j = 0; j < 2; ++j) {
       const float2 q = p[j];
-      const float t = q.x + v[j], bp = t - q.x;
-      p[j] = make_float2(t, q.y + ((q.x - (t - bp)) + (v[j] - bp)));
+      v[j].lo += q.y;
+      v[j].add(q.x);
+      p[j] = make_float2(v[j].hi, v[j].lo);
     }
   }
 }
 
-// out[j] = scale[j] times the sum of the warps' pairs acc[3 i + j], one block
-__global__ void k_scalar_sums(const float2* __restrict__ acc, int n, double s0, double s1,
-                              double s2, double* __restrict__ out) {
-  __shared__ double red[3][kThreads / 32];
-  double v[3] = {0.0, 0.0, 0.0};
+// The gradients of kappa, W and M from the warps' pairs (kappa, W) in acc, one block
+__global__ void k_scalar_sums(const float2* __restrict__ acc, int n, ChMobScale sc,
+                              double* __restrict__ out) {
+  __shared__ double red[2][kThreads / 32];
+  double v[2] = {0.0, 0.0};
   for (int i = threadIdx.x; i < n; i += kThreads)
-    for (int j = 0; j < 3; ++j) v[j] += (double)acc[3 * (int64_t)i + j].x + (double)acc[3 * (int64_t)i + j].y;
-  for (int j = 0; j < 3; ++j) {
+    for (int j = 0; j < 2; ++j) v[j] += (double)acc[2 * (int64_t)i + j].x + (double)acc[2 * (int64_t)i + j].y;
+  for (int j = 0; j < 2; ++j) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v[j] += __shfl_down_sync(kFull, v[j], o);
     if ((threadIdx.x & 31) == 0) red[j][threadIdx.x >> 5] = v[j];
   }
   __syncthreads();
   if (threadIdx.x == 0) {
-    const double sc[3] = {s0, s1, s2};
-    for (int j = 0; j < 3; ++j) {
-      double s = 0.0;
-      for (int w = 0; w < kThreads / 32; ++w) s += red[j][w];
-      out[j] = sc[j] * s;
-    }
+    double s[2] = {0.0, 0.0};
+    for (int j = 0; j < 2; ++j)
+      for (int w = 0; w < kThreads / 32; ++w) s[j] += red[j][w];
+    out[0] = sc.kappa * s[0];
+    out[1] = sc.W * s[1];
+    out[2] = sc.M_kappa * s[0] + sc.M_W * s[1];
   }
 }
 
@@ -531,18 +583,41 @@ dim3 sweep_grid(const ChMobArgs& a, int ty) {
 
 int ch_mob_warps(int nx, int ny) { return strips(nx) * ((ny + kTYRev - 1) / kTYRev); }
 
-void pack_ch_mob(ChMobArgs& a) {
-  const double g = kGHi, g2 = g * g, wt = 0.25 * g2;
-  const double p[4] = {a.p0, a.p1, a.p2, a.p3}, h[3] = {a.s0, a.s1, a.s2};
-  double s = 1.0;
-  for (int i = 0; i < 4; ++i, s *= g2) a.q[i] = (float)(wt * s * p[i]);
-  s = 1.0;
-  for (int i = 0; i < 3; ++i, s *= g2) a.h[i] = (float)(wt * g2 * s * h[i]);
-  const double ix = a.ihx, iy = a.ihy, g3 = g * g2;
-  a.cX = (float)(0.25 * a.M * ix * ix * g3);
-  a.cY = (float)(0.25 * a.M * iy * iy * g3);
-  a.gX = (float)(0.25 * a.ngm * ix * ix * g3);
-  a.gY = (float)(0.25 * a.ngm * iy * iy * g3);
+void pack_ch_mob(const ChMobParams& p, ChMobArgs& a, ChMobScale& sc) {
+  // a value at a Gauss point is g2 times the one carried, and so is the weight
+  // back; the Gauss weight is |cell|/4 over the interior mass |cell|
+  const double g = 1.0 / (1.0 + (double)(kGLo / kGHi)), g2 = g * g, cF = 0.25 * g2 * g2;
+  double s = 1.0 / g2;
+  for (int i = 0; i < 4; ++i, s *= g2) {
+    a.q[i] = (float)(s * p.f1[i]);
+    if (i < 3) a.h[i] = (float)(s * g2 * p.f2[i]);
+  }
+  const double rx = p.hy / p.hx, ry = p.hx / p.hy, cell = p.hx * p.hy;
+  const double cK = (rx + ry) / (6.0 * cell);  // minus the corner weight of m^-1 K
+  a.k.c0 = 8.0f;
+  a.k.cx = (float)((-4.0 * rx + 2.0 * ry) / (rx + ry));
+  a.k.cy = (float)((2.0 * rx - 4.0 * ry) / (rx + ry));
+  a.k.cd = -1.0f;
+  const auto pair = [](double v, float (&o)[2]) {
+    o[0] = (float)v;
+    o[1] = (float)(v - (double)o[0]);
+  };
+  // fluxes: a difference takes g, the other direction's mobility sum and the
+  // weight back g each
+  const double w = 0.25 * g * g2, ix2 = 1.0 / (p.hx * p.hx), iy2 = 1.0 / (p.hy * p.hy);
+  const double cW = p.M * w * ix2;
+  pair(p.kappa * cK / cF, a.r);
+  pair(-p.dt * cF * cW, a.fx);
+  pair(-p.dt * cF * p.M * w * iy2, a.fy);
+  pair(iy2 / ix2, a.ay);
+  pair(-p.dt * cF * cW, a.n);
+  a.gX = (float)(-p.dt * cell * cF * p.M * w * ix2);
+  a.gY = (float)(-p.dt * cell * cF * p.M * w * iy2);
+  const double f = -p.dt * cell * cW;
+  sc.kappa = f * cK;
+  sc.W = f * cF / p.W;
+  sc.M_kappa = f * cK * p.kappa / p.M;
+  sc.M_W = f * cF / p.M;
 }
 
 cudaError_t launch_ch_mob_step(const ChMobArgs& a, float* out, cudaStream_t s) {
@@ -557,9 +632,9 @@ cudaError_t launch_ch_adj_step(const ChMobArgs& a, const float* yin, float* yout
   return cudaGetLastError();
 }
 
-cudaError_t launch_scalar_sums(const float2* acc, int n, const double scale[3], double* out,
+cudaError_t launch_scalar_sums(const float2* acc, int n, const ChMobScale& sc, double* out,
                                cudaStream_t s) {
-  k_scalar_sums<<<1, kThreads, 0, s>>>(acc, n, scale[0], scale[1], scale[2], out);
+  k_scalar_sums<<<1, kThreads, 0, s>>>(acc, n, sc, out);
   return cudaGetLastError();
 }
 

@@ -46,6 +46,7 @@ struct pf_ctx {
   pf::Explicit2DArgs ex{};
   pf::Implicit3DArgs im{};
   pf::ChMobArgs mob{};
+  pf::ChMobScale mob_scale{};
 
   // 3-D workspace segments (each n_fields * N floats)
   float* u = nullptr;   // current iterate / state
@@ -409,7 +410,7 @@ AdjLayout adj_layout(const pf_ctx* c, int64_t n_steps, int ckpt) {
   L.glo = off;
   off += field;
   L.acc = off;
-  off += align_up(sizeof(float2) * 3 * (size_t)pf::ch_mob_warps((int)c->n[0], (int)c->n[1]), 256);
+  off += align_up(sizeof(float2) * 2 * (size_t)pf::ch_mob_warps((int)c->n[0], (int)c->n[1]), 256);
   L.small = off;
   off += align_up(sizeof(double) * 512, 256);
   L.total = off;
@@ -914,23 +915,10 @@ pf_status pf_set_params(pf_ctx* c, const pf_params* p) {
     b.nx = a.nx;
     b.ny = a.ny;
     b.mfield = p->mobility_field;
-    b.p0 = (float)fp[0];
-    b.p1 = (float)fp[1];
-    b.p2 = (float)fp[2];
-    b.p3 = (float)fp[3];
-    // second derivative of f at s + d, expanded about s (exact quadratic in d)
-    b.s0 = (float)(W * (2 - 12 * s + 12 * s * s));
-    b.s1 = (float)(W * (-12 + 24 * s));
-    b.s2 = (float)(12 * W);
-    b.k = stiffness2d(hx, hy, 1.0 / m);
-    b.kappa = (float)p->kappa;
-    b.M = (float)p->mobility;
-    b.W = (float)W;
-    b.dt = (float)p->dt;
-    b.ihx = (float)(1.0 / hx);
-    b.ihy = (float)(1.0 / hy);
-    b.cell = m;
-    pf::pack_ch_mob(b);
+    pf::ChMobParams q{hx, hy, p->kappa, W, p->mobility, p->dt};
+    for (int i = 0; i < 4; ++i) q.f1[i] = fp[i];
+    for (int i = 0; i < 3; ++i) q.f2[i] = (i + 1) * fp[i + 1];  // f'' about s: the derivative of f'
+    pf::pack_ch_mob(q, b, c->mob_scale);
   }
   pf::pack_explicit2d(a);
   destroy_graph(c);
@@ -1638,8 +1626,6 @@ pf_status pf_adjoint(pf_ctx* c, const float* state0, const float* target, int64_
     c->mob.mfield = ones;
   }
   pf::ChMobArgs a = c->mob;
-  a.ngm = (float)(-(double)a.dt * a.M * a.cell);
-  pf::pack_ch_mob(a);
   // whole segments replay graphs captured here (while earlier work runs):
   // g[0] recomputes seg(1 .. ckpt-1) from seg(0), g[1 + p] reverses a segment
   // starting from y0 (p = 0) or y1 (p = 1); a shorter last segment launches
@@ -1699,7 +1685,7 @@ pf_status pf_adjoint(pf_ctx* c, const float* state0, const float* target, int64_
   if (st == PF_OK) {
     PF_CUDA(pf::launch_loss(ck(last), shift, target, nx, ny, cell, nodal_loss, y0, small + 8,
                             small, c->stream));
-    PF_CUDA(cudaMemsetAsync(acc, 0, sizeof(float2) * 3 * (size_t)nw, c->stream));
+    PF_CUDA(cudaMemsetAsync(acc, 0, sizeof(float2) * 2 * (size_t)nw, c->stream));
     if (grad_mobility) {
       PF_CUDA(cudaMemsetAsync(ghi, 0, sizeof(float) * N, c->stream));
       PF_CUDA(cudaMemsetAsync(glo, 0, sizeof(float) * N, c->stream));
@@ -1726,10 +1712,7 @@ pf_status pf_adjoint(pf_ctx* c, const float* state0, const float* target, int64_
       }
     }
     if (st == PF_OK) {
-      // -dt cell sums of w with m^-1 K c, m^-1 F and mu; F = W times its own
-      // polynomial, mu's mobility factor M
-      const double f = -(double)a.dt * a.cell, scale[3] = {f, f / a.W, f / a.M};
-      cudaError_t e = pf::launch_scalar_sums(acc, nw, scale, small + 1, c->stream);
+      cudaError_t e = pf::launch_scalar_sums(acc, nw, c->mob_scale, small + 1, c->stream);
       if (e == cudaSuccess && grad_mobility)
         e = pf::launch_grad_to_double(ghi, glo, grad_mobility, N, c->stream);
       if (e == cudaSuccess && grad_state0)

@@ -205,29 +205,39 @@ cudaError_t launch_energy2d(const Energy2DArgs& a, double* partials, double* res
 
 // 2-D Cahn-Hilliard with a per-node mobility field: explicit step and its
 // discrete adjoint (plain row-major planes, shifted state d = c - s).
+struct ChMobParams {
+  double hx, hy, kappa, W, M, dt;
+  double f1[4], f2[3];  // f' and f'' at s + d, increasing powers of d
+};
+// What the kernels carry: F without its factor cF, K c without the stencil's
+// corner weight cK, w without cW, mu in units of cF; pairs are hi + lo.
 struct ChMobArgs {
   const float* d;       // shifted state at which the operators are evaluated
   const float* mfield;  // mobility multiplier per node
   int nx, ny;
-  float p0, p1, p2, p3;  // f'(s + d) = p0 + d (p1 + d (p2 + d p3))
-  float s0, s1, s2;      // f''(s + d) = s0 + d (s1 + d s2)
-  Stencil2D k;           // Q1 stiffness stencil / cell
-  float kappa, M, W, dt, ihx, ihy;
-  double cell;
-  float ngm;  // -dt M cell, the factor of the mobility gradient (reverse step)
-  // filled by pack_ch_mob: the polynomials and the factors of the fluxes and of
-  // the mobility gradient, with the quadrature's weights
-  float q[4], h[3], cX, cY, gX, gY;
+  // filled by pack_ch_mob
+  float q[4], h[3];    // f' and f'' in interpolated values without the factor g_hi^2
+  Stencil2D k;         // Q1 stiffness stencil / cK
+  float r[2];          // kappa cK / cF
+  float fx[2], fy[2];  // forward: -dt cF times the fluxes' factors along x and y
+  float ay[2];         // flux factor along y over the one along x, which is cW
+  float n[2];          // reverse: -dt cF cW
+  float gX, gY;        // factors of the mobility gradient
 };
-void pack_ch_mob(ChMobArgs& a);
-int ch_mob_warps(int nx, int ny);  // triples of pairs in the reverse step's acc
+// factors of the reverse step's sums of w K c and w F: dLoss/dkappa, dLoss/dW,
+// dLoss/dM (both)
+struct ChMobScale {
+  double kappa, W, M_kappa, M_W;
+};
+void pack_ch_mob(const ChMobParams& p, ChMobArgs& a, ChMobScale& sc);
+int ch_mob_warps(int nx, int ny);  // twos of pairs in the reverse step's acc
 cudaError_t launch_ch_mob_step(const ChMobArgs& a, float* out, cudaStream_t s);
 // grad_hi / grad_lo: the running mobility gradient as a compensated FP32 pair
 // per node (both null: not accumulated); grad_to_double writes hi + lo in FP64.
 cudaError_t launch_ch_adj_step(const ChMobArgs& a, const float* yin, float* yout,
                                float* grad_hi, float* grad_lo, float2* acc, cudaStream_t s);
-// out[j] = scale[j] * (sum over i < n of the pair acc[3 i + j]), j < 3
-cudaError_t launch_scalar_sums(const float2* acc, int n, const double scale[3], double* out,
+// out = dLoss/dkappa, dLoss/dW, dLoss/dM from n warps' pairs
+cudaError_t launch_scalar_sums(const float2* acc, int n, const ChMobScale& sc, double* out,
                                cudaStream_t s);
 cudaError_t launch_grad_to_double(const float* hi, const float* lo, double* out, int64_t n,
                                   cudaStream_t s);
