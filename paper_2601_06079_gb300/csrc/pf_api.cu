@@ -819,13 +819,9 @@ void set_params_coupled(pf_ctx* c, const pf_params* p) {
 // The coupled step: framed working planes [c - shift; eta] in buf_a / buf_b
 // (ping-pong), one fused launch per step, replayed from graphs of kGraphSteps.
 pf_status step_coupled2d(pf_ctx* c, float* state, int64_t n_steps) {
-  const int64_t N = nodes2d(c), plane = c->cp.plane;
   const int nx = (int)c->n[0], ny = (int)c->n[1];
   const float shift = (float)c->par.shift;
-  for (float* buf : {c->buf_a, c->buf_b}) {
-    PF_CUDA(pf::launch_to_work(state, buf, nx, ny, shift, c->stream));
-    PF_CUDA(pf::launch_to_work(state + N, buf + plane, nx, ny, 0.0f, c->stream));
-  }
+  PF_CUDA(pf::launch_to_work(state, c->buf_a, c->buf_b, nx, ny, 2, shift, c->stream));
   int64_t left = n_steps;
   if (left >= kGraphSteps) {
     pf_status st = ensure_graph(c);
@@ -838,8 +834,7 @@ pf_status step_coupled2d(pf_ctx* c, float* state, int64_t n_steps) {
     PF_CUDA(launch_step(c, cur, oth, c->stream));
     std::swap(cur, oth);
   }
-  PF_CUDA(pf::launch_from_work(cur, state, nx, ny, shift, c->stream));
-  PF_CUDA(pf::launch_from_work(cur + plane, state + N, nx, ny, 0.0f, c->stream));
+  PF_CUDA(pf::launch_from_work(cur, state, nx, ny, 2, shift, c->stream));
   return PF_OK;
 }
 
@@ -981,8 +976,7 @@ pf_status pf_step_explicit(pf_ctx* c, float* state, int64_t n_steps) {
   const float shift = (float)c->par.shift;
   const int nx = (int)c->n[0], ny = (int)c->n[1];
   // working copies with the mirror frame: d = u - shift (both planes fully defined)
-  PF_CUDA(pf::launch_to_work(state, c->buf_a, nx, ny, shift, c->stream));
-  PF_CUDA(pf::launch_to_work(state, c->buf_b, nx, ny, shift, c->stream));
+  PF_CUDA(pf::launch_to_work(state, c->buf_a, c->buf_b, nx, ny, 1, shift, c->stream));
   int64_t left = n_steps;
   if (left >= kGraphSteps && c->form == PF_FORM_FUSED_GRAPH) {
     pf_status st = ensure_graph(c);
@@ -997,7 +991,7 @@ pf_status pf_step_explicit(pf_ctx* c, float* state, int64_t n_steps) {
     cur = oth;
     oth = t;
   }
-  PF_CUDA(pf::launch_from_work(cur, state, nx, ny, shift, c->stream));
+  PF_CUDA(pf::launch_from_work(cur, state, nx, ny, 1, shift, c->stream));
   return PF_OK;
 }
 

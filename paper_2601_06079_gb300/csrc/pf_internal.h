@@ -150,10 +150,12 @@ cudaError_t launch_ch2d(const Explicit2DArgs& a, cudaStream_t s);
 // Ghost-padded working planes: work_pitch(nx) x work_rows(ny) floats each.
 int work_pitch(int nx);
 int work_rows(int ny);
-cudaError_t launch_to_work(const float* in, float* work, int nx, int ny, float shift,
-                           cudaStream_t s);
-cudaError_t launch_from_work(const float* work, float* out, int nx, int ny, float shift,
-                             cudaStream_t s);
+// `fields` of them one after another, the shift applies to the first; to both
+// buffers a and b.
+cudaError_t launch_to_work(const float* in, float* a, float* b, int nx, int ny, int fields,
+                           float shift, cudaStream_t s);
+cudaError_t launch_from_work(const float* work, float* out, int nx, int ny, int fields,
+                             float shift, cudaStream_t s);
 
 // Explicit 2-D trajectories held on chip (k_onchip2d.cu): a job is one mesh, cut
 // into gx x gy tiles of one block each.
