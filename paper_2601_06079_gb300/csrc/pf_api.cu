@@ -823,7 +823,10 @@ pf_status step_coupled2d(pf_ctx* c, float* state, int64_t n_steps) {
   const float shift = (float)c->par.shift;
   PF_CUDA(pf::launch_to_work(state, c->buf_a, c->buf_b, nx, ny, 2, shift, c->stream));
   int64_t left = n_steps;
-  if (left >= kGraphSteps) {
+  // a graph cannot be launched into a capture: there, the steps themselves are
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  if (left >= kGraphSteps) PF_CUDA(cudaStreamIsCapturing(c->stream, &capture));
+  if (left >= kGraphSteps && capture == cudaStreamCaptureStatusNone) {
     pf_status st = ensure_graph(c);
     if (st != PF_OK) return st;
     for (; left >= kGraphSteps; left -= kGraphSteps) PF_CUDA(cudaGraphLaunch(c->graph, c->stream));

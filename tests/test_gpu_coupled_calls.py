@@ -31,3 +31,20 @@ def test_short_run_takes_two_launches_beside_its_steps():
     assert cuda.cuGraphGetNodes(graph, None, C.byref(n)) == 0
     cuda.cuGraphDestroy(graph)
     assert n.value == 22
+
+
+@pytest.mark.parametrize("steps", [20, 64, 150])
+def test_call_can_be_captured(steps):
+    stream = torch.cuda.Stream()
+    s = solver(stream)
+    u0 = torch.from_numpy(G.coupled_initial(3, (48, 70))).cuda()
+    a, b = u0.clone(), u0.clone()
+    torch.cuda.synchronize()
+    s.step_explicit(a, steps)
+    stream.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream):
+        s.step_explicit(b, steps)
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(a, b)
