@@ -171,6 +171,10 @@ __global__ void __launch_bounds__(kWarps * 32) k_coupled2d(const Coupled2DArgs a
   const int lane = threadIdx.x & 31;
   const int y0 = (block_row() * kWarps + (threadIdx.x >> 5)) * kTY;
   const int nx = a.nx, ny = a.ny;
+  // launched as dependent (launch_coupled2d): the next step may start to launch,
+  // and this one begins when the step before it is complete
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   if (y0 >= ny) return;
   const Coef K{a.pair};
   const int64_t pitch = a.pitch, plane = a.plane;
@@ -255,11 +259,19 @@ void pack_coupled2d(const CoupledPoly& f, double neg_dt_meta, Coupled2DArgs& a) 
 
 namespace {
 template <bool kIso, int kTY>
-cudaError_t launch(const Coupled2DArgs& a, cudaStream_t s) {
+cudaError_t launch(const Coupled2DArgs& a, bool dependent, cudaStream_t s) {
   const dim3 grid = row_grid((a.nx + kOutCols - 1) / kOutCols,
                              (a.ny + kWarps * kTY - 1) / (kWarps * kTY));
-  k_coupled2d<kIso, kTY><<<grid, kWarps * 32, 0, s>>>(a);
-  return cudaGetLastError();
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(kWarps * 32);
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = dependent ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, k_coupled2d<kIso, kTY>, a);
 }
 }  // namespace
 
@@ -267,13 +279,19 @@ cudaError_t launch(const Coupled2DArgs& a, cudaStream_t s) {
 // them fit), 7 beyond: us per step at 64^2 / 515 x 1031 / 1024^2 / 2048^2 with
 // 4 rows 3.8 / 6.9 / 10.4 / 30.6, with 7 rows 5.7 / 8.3 / 11.2 / 28.0, with 13
 // rows 9.0 / 11.1 / 12.7 / 28.6.
-cudaError_t launch_coupled2d(const Coupled2DArgs& a, cudaStream_t s) {
+//
+// dependent: for steps launched one by one, whose launch then overlaps the step
+// before.  20 steps, us: 64^2 140 without, 89 with (node tiles 127), 64 x 1500
+// 144 and 103 (149), 1024^2 272 and 224, 2048^2 643 and 607.  Not in a graph,
+// which launches close behind as it is: 200 steps 706 and 664 at 64^2, 728 and
+// 920 at 64 x 1500, 5,529 and 5,494 at 2048^2.
+cudaError_t launch_coupled2d(const Coupled2DArgs& a, bool dependent, cudaStream_t s) {
   const auto iso = [](const Stencil2D& k) { return k.cx == k.cd && k.cy == k.cd; };
   const bool both = iso(a.k1) && iso(a.k2);
   const int64_t warps = (int64_t)((a.nx + kOutCols - 1) / kOutCols) * ((a.ny + 6) / 7);
   if (warps < 40 * (int64_t)device_sm_count())
-    return both ? launch<true, 4>(a, s) : launch<false, 4>(a, s);
-  return both ? launch<true, 7>(a, s) : launch<false, 7>(a, s);
+    return both ? launch<true, 4>(a, dependent, s) : launch<false, 4>(a, dependent, s);
+  return both ? launch<true, 7>(a, dependent, s) : launch<false, 7>(a, dependent, s);
 }
 
 }  // namespace pf

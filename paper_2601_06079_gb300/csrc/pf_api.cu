@@ -269,12 +269,13 @@ struct CallGraphs {
   }
 };
 
-cudaError_t launch_step(pf_ctx* c, const float* in, float* out, cudaStream_t s) {
+// dependent: the launch may overlap the kernel before it in the stream (coupled step)
+cudaError_t launch_step(pf_ctx* c, const float* in, float* out, bool dependent, cudaStream_t s) {
   if (c->model == PF_MODEL_COUPLED) {
     pf::Coupled2DArgs a = c->cp;
     a.in = in;
     a.out = out;
-    return pf::launch_coupled2d(a, s);
+    return pf::launch_coupled2d(a, dependent, s);
   }
   pf::Explicit2DArgs a = c->ex;
   a.in = in;
@@ -289,8 +290,8 @@ pf_status ensure_graph(pf_ctx* c) {
   PF_CUDA(cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal));
   cudaError_t le = cudaSuccess;
   for (int i = 0; i < kGraphSteps && le == cudaSuccess; ++i)
-    le = (i % 2 == 0) ? launch_step(c, c->buf_a, c->buf_b, c->cap_stream)
-                      : launch_step(c, c->buf_b, c->buf_a, c->cap_stream);
+    le = (i % 2 == 0) ? launch_step(c, c->buf_a, c->buf_b, false, c->cap_stream)
+                      : launch_step(c, c->buf_b, c->buf_a, false, c->cap_stream);
   cudaGraph_t g = nullptr;
   cudaError_t ee = cudaStreamEndCapture(c->cap_stream, &g);
   if (le != cudaSuccess) {
@@ -824,9 +825,10 @@ pf_status step_coupled2d(pf_ctx* c, float* state, int64_t n_steps) {
   PF_CUDA(pf::launch_to_work(state, c->buf_a, c->buf_b, nx, ny, 2, shift, c->stream));
   int64_t left = n_steps;
   // a graph cannot be launched into a capture: there, the steps themselves are
-  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-  if (left >= kGraphSteps) PF_CUDA(cudaStreamIsCapturing(c->stream, &capture));
-  if (left >= kGraphSteps && capture == cudaStreamCaptureStatusNone) {
+  cudaStreamCaptureStatus capture;
+  PF_CUDA(cudaStreamIsCapturing(c->stream, &capture));
+  const bool captured = capture != cudaStreamCaptureStatusNone;
+  if (left >= kGraphSteps && !captured) {
     pf_status st = ensure_graph(c);
     if (st != PF_OK) return st;
     for (; left >= kGraphSteps; left -= kGraphSteps) PF_CUDA(cudaGraphLaunch(c->graph, c->stream));
@@ -834,7 +836,7 @@ pf_status step_coupled2d(pf_ctx* c, float* state, int64_t n_steps) {
   float* cur = c->buf_a;
   float* oth = c->buf_b;
   for (; left > 0; --left) {
-    PF_CUDA(launch_step(c, cur, oth, c->stream));
+    PF_CUDA(launch_step(c, cur, oth, !captured, c->stream));
     std::swap(cur, oth);
   }
   PF_CUDA(pf::launch_from_work(cur, state, nx, ny, 2, shift, c->stream));
@@ -989,7 +991,7 @@ pf_status pf_step_explicit(pf_ctx* c, float* state, int64_t n_steps) {
   float* cur = c->buf_a;
   float* oth = c->buf_b;
   for (; left > 0; --left) {
-    PF_CUDA(launch_step(c, cur, oth, c->stream));
+    PF_CUDA(launch_step(c, cur, oth, false, c->stream));
     float* t = cur;
     cur = oth;
     oth = t;

@@ -120,7 +120,7 @@ struct CoupledPoly {
   double fa[5], fb[3];
 };
 void pack_coupled2d(const CoupledPoly& f, double neg_dt_meta, Coupled2DArgs& a);
-cudaError_t launch_coupled2d(const Coupled2DArgs& a, cudaStream_t s);
+cudaError_t launch_coupled2d(const Coupled2DArgs& a, bool dependent, cudaStream_t s);
 // The plain two-pass comparison form (d, mu, out: nx x ny arrays without frame).
 cudaError_t launch_plain2d(bool ch, const Explicit2DArgs& a, const float* d, float* mu, float* out,
                            cudaStream_t s);

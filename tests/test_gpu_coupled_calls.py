@@ -9,9 +9,9 @@ import pf_inputs as G
 pytestmark = pytest.mark.gpu
 
 
-def solver(stream=None):
+def solver(stream=None, shape=(48, 70)):
     import paper_2601_06079_gb300 as pf
-    s = pf.Solver((48, 70), model="coupled", stream=stream)
+    s = pf.Solver(shape, model="coupled", stream=stream)
     s.set_params(kappa=0.3, mobility=1.0, mobility2=150.0, dt=1e-3)
     return s
 
@@ -33,11 +33,13 @@ def test_short_run_takes_two_launches_beside_its_steps():
     assert n.value == 22
 
 
-@pytest.mark.parametrize("steps", [20, 64, 150])
-def test_call_can_be_captured(steps):
+@pytest.mark.parametrize("shape,steps", [((48, 70), 20), ((48, 70), 64), ((48, 70), 150),
+                                         ((1400, 1501), 40)])
+def test_call_can_be_captured(shape, steps):
+    # also: steps that overlap the launch before them against steps that do not
     stream = torch.cuda.Stream()
-    s = solver(stream)
-    u0 = torch.from_numpy(G.coupled_initial(3, (48, 70))).cuda()
+    s = solver(stream, shape)
+    u0 = torch.from_numpy(G.coupled_initial(3, shape)).cuda()
     a, b = u0.clone(), u0.clone()
     torch.cuda.synchronize()
     s.step_explicit(a, steps)
