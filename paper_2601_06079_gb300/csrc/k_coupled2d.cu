@@ -171,9 +171,7 @@ __global__ void __launch_bounds__(kWarps * 32) k_coupled2d(const Coupled2DArgs a
   const int lane = threadIdx.x & 31;
   const int y0 = (block_row() * kWarps + (threadIdx.x >> 5)) * kTY;
   const int nx = a.nx, ny = a.ny;
-  // launched as dependent (launch_coupled2d): the next step may start to launch,
-  // and this one begins when the step before it is complete
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  // launched as dependent (launch_coupled2d): the step before this one is complete
   asm volatile("griddepcontrol.wait;" ::: "memory");
   if (y0 >= ny) return;
   const Coef K{a.pair};
@@ -218,6 +216,9 @@ __global__ void __launch_bounds__(kWarps * 32) k_coupled2d(const Coupled2DArgs a
       store(out0 + plane, y0 + i + j, oe);
     }
   }
+  // the next step may launch; were it let go at this one's start, its waiting
+  // blocks would pile up on a part of the SMs (512^2: 7.2 us a step, so 4.3)
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   consume(std::integral_constant<int, kOnlyC>{}, 1);
   store(out0, y0 + kTY - 1, oc);
 }
@@ -280,11 +281,10 @@ cudaError_t launch(const Coupled2DArgs& a, bool dependent, cudaStream_t s) {
 // 4 rows 3.8 / 6.9 / 10.4 / 30.6, with 7 rows 5.7 / 8.3 / 11.2 / 28.0, with 13
 // rows 9.0 / 11.1 / 12.7 / 28.6.
 //
-// dependent: for steps launched one by one, whose launch then overlaps the step
-// before.  20 steps, us: 64^2 140 without, 89 with (node tiles 127), 64 x 1500
-// 144 and 103 (149), 1024^2 272 and 224, 2048^2 643 and 607.  Not in a graph,
-// which launches close behind as it is: 200 steps 706 and 664 at 64^2, 728 and
-// 920 at 64 x 1500, 5,529 and 5,494 at 2048^2.
+// dependent: for steps launched one by one, whose launch then overlaps the end
+// of the step before.  20 steps, us, without / with (node tiles): 64^2 140 / 80
+// (125), 64 x 1500 144 / 85 (145), 512^2 140 / 102 (187), 1024^2 270 / 221 (352).
+// Steps in a graph, which launches them close behind one another, are not.
 cudaError_t launch_coupled2d(const Coupled2DArgs& a, bool dependent, cudaStream_t s) {
   const auto iso = [](const Stencil2D& k) { return k.cx == k.cd && k.cy == k.cd; };
   const bool both = iso(a.k1) && iso(a.k2);
