@@ -172,9 +172,9 @@ pf_status pf_set_form(pf_ctx* ctx, int form);
  * guess: device initial Newton iterate for the FIRST step (NULL = U^n); later
  * steps start from their U^n.  opts may be NULL (defaults); stats (host) may be
  * NULL.  Synchronises the stream.  PF_ERR_NOT_CONVERGED: state holds the last
- * iterate and stats the counts so far.  2-D meshes of up to 2^20 nodes make all
- * steps in one launch whose blocks wait for each other; PF_ERR_TIMEOUT if such a
- * wait expired (about one second). */
+ * iterate and stats the counts so far.  2-D meshes of up to 2^20 nodes (thin
+ * ones fewer) make all steps in one launch whose blocks wait for each other;
+ * PF_ERR_TIMEOUT if such a wait expired (about one second). */
 pf_status pf_step_implicit(pf_ctx* ctx, float* state, int64_t n_steps, const float* guess,
                            const pf_newton_opts* opts, pf_newton_stats* stats);
 

@@ -425,8 +425,12 @@ __global__ void __launch_bounds__(kThreads) k_newton2d(const Newton2DArgs a) {
 
 }  // namespace
 
+int64_t newton2d_tile_nodes(int nx, int ny) {
+  return (int64_t)((nx + TX - 1) / TX) * ((ny + TY - 1) / TY) * (TX * TY);
+}
+
 int newton2d_blocks(int nx, int ny) {
-  const int64_t tiles = (int64_t)((nx + TX - 1) / TX) * ((ny + TY - 1) / TY);
+  const int64_t tiles = newton2d_tile_nodes(nx, ny) / (TX * TY);
   const int64_t sms = device_sm_count();
   return (int)(tiles < sms ? tiles : sms);
 }

@@ -1033,13 +1033,25 @@ pf_status pf_energy(pf_ctx* c, const float* state, double* energy, double* mass)
   return PF_OK;
 }
 
-// Largest mesh whose implicit 2-D steps run as one launch.  Three steps of
+// Whether a mesh's implicit 2-D steps run as one launch.  Three steps of
 // dt = 0.5, us, one launch / launches per vector operation: Allen-Cahn 64^2
 // 840 / 2,870, 512^2 1,780 / 3,290, 1024^2 4,300 / 4,570, 1448^2 7,430 / 5,290;
 // Cahn-Hilliard 64^2 1,170 / 3,580, 512^2 2,590 / 4,460, 1024^2 6,380 / 6,550,
 // 1448^2 15,800 / 9,740 (a block's tiles outgrow its L1, and its 16 warps keep
-// fewer bytes on the way than the vector kernels).
+// fewer bytes on the way than the vector kernels).  What the one launch takes
+// grows with the tiles; the vector kernels take the nodes, and a least time for
+// their launches that a mesh of thin tiles does not get below.  So idle nodes of
+// tiles count, and a fifth more.  Two steps, us, launches / one launch, tiles,
+// share of their nodes in use: Allen-Cahn 32768 x 32 2,790 / 2,440 (2,048, 1.0);
+// 33 x 31775 2,860 / 3,300 (2,979, 0.69), 31775 x 33 3,050 / 4,460 (3,972, 0.52),
+// 116508 x 9 3,690 / 7,490 (7,282, 0.28), 2 x 200000 3,730 / 6,070 (6,250, 0.13),
+// 20000 x 17 2,500 / 1,840 (1,250, 0.53); Cahn-Hilliard 116508 x 9 7,590 / 16,390.
 constexpr int64_t kNewton2DNodes = 1 << 20;
+bool one_launch2d(const pf_ctx* c) {
+  const int64_t nodes = nnodes(c);
+  const int64_t all = pf::newton2d_tile_nodes((int)c->n[0], (int)c->n[1]);
+  return nodes <= kNewton2DNodes && all + (all - nodes) / 5 <= kNewton2DNodes + kNewton2DNodes / 50;
+}
 
 // n_steps steps by k_newton2d, in launches of at most 64 steps.
 pf_status step_newton2d(pf_ctx* c, float* state, int64_t n_steps, const float* guess,
@@ -1112,7 +1124,7 @@ pf_status pf_step_implicit(pf_ctx* c, float* state, int64_t n_steps, const float
   const int64_t n = vec_len(c);
   const double inv_dt = 1.0 / c->par.dt;
   const int64_t n_state = split_ch(c) ? nnodes(c) : n;  // CH: the state is c alone
-  if (c->dim == 2 && nnodes(c) <= kNewton2DNodes) {
+  if (c->dim == 2 && one_launch2d(c)) {
     st = step_newton2d(c, state, n_steps, guess, o,
                        kNoOversolve / std::sqrt(c->h[0] * c->h[1] * c->h[2]), &s);
     // as in the loop below, statistics are reported unless the solve broke off

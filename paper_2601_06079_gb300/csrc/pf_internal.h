@@ -300,6 +300,7 @@ struct Newton2DArgs {
   double newton_rtol, gmres_rtol, atol_factor, inv_dt;
 };
 int newton2d_blocks(int nx, int ny);
+int64_t newton2d_tile_nodes(int nx, int ny);  // nodes of the tiles that cover a mesh
 size_t newton2d_packet_bytes(int nx, int ny);
 cudaError_t launch_newton2d(const Newton2DArgs& a, cudaStream_t s);
 
