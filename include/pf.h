@@ -150,8 +150,10 @@ pf_status pf_step_explicit(pf_ctx* ctx, float* state, int64_t n_steps);
  *                         2,100^2 nodes) and the steps pay for it; otherwise one
  *                         fused kernel per step, replayed from a CUDA graph of
  *                         64 steps.  Bitwise the same results either way; should
- *                         a bounded wait between blocks expire, the state is
- *                         filled with NaN
+ *                         a bounded wait between blocks expire (about one
+ *                         second), some or all tiles of the state are filled
+ *                         with NaN, and pf_energy returns PF_ERR_TIMEOUT until
+ *                         the context steps again
  *   PF_FORM_FUSED_STREAM  the same kernel, one launch per step from the host
  *   PF_FORM_TWO_PASS      the plain form: node-centric quadrature with index
  *                         reflection, CH's mu written to and read back from
@@ -309,10 +311,21 @@ pf_status pf_step_ensemble(pf_ctx* ctx, float* packed_state, int64_t n_steps, in
 pf_status pf_barrier_selftest(unsigned* dev_scratch, long long limit_cycles, int phantom,
                               void* stream);
 
+/* Failure-detection self-test of the bounded waits between the blocks of one
+ * launch: n_steps (>= 8) steps of the context's mesh in the on-chip form of
+ * pf_step_explicit (implicit = 0) or the one-launch form of pf_step_implicit (1),
+ * with one block missing (explicit) or unheard (implicit), so that the waits for it
+ * run out after limit_cycles SM clocks each.  Returns PF_ERR_TIMEOUT, with the context still usable and the
+ * state undefined (explicit: NaN in some or all tiles); PF_ERR_ARG if the mesh
+ * does not take that form or takes one block.  Synchronises the stream. */
+pf_status pf_wait_selftest(pf_ctx* ctx, float* state, int64_t n_steps, long long limit_cycles,
+                           int implicit);
+
 /* Discrete free energy E_h = sum_e sum_q w_q |J| [f(U_q) + kappa/2 |grad U_q|^2]
  * (Eq. 5-6) and, per field, the mass integral sum_i m_i U_i, accumulated in FP64.
  * energy: host, 1 double; mass: host, n_fields doubles (either may be NULL).
- * 2-D meshes.  Synchronises the stream. */
+ * 2-D meshes.  PF_ERR_TIMEOUT if a wait of the last explicit run expired (see
+ * pf_set_form).  Synchronises the stream. */
 pf_status pf_energy(pf_ctx* ctx, const float* state, double* energy, double* mass);
 
 /* Energy and mass of a 2-D single-field double-well state (AC or CH) without a

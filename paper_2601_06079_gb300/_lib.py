@@ -118,6 +118,8 @@ def lib():
         L.pf_step_ensemble.argtypes = [ctx, C.c_void_p, C.c_int64, C.c_int]
         L.pf_barrier_selftest.restype = st
         L.pf_barrier_selftest.argtypes = [C.c_void_p, C.c_longlong, C.c_int, C.c_void_p]
+        L.pf_wait_selftest.restype = st
+        L.pf_wait_selftest.argtypes = [C.c_void_p, C.c_void_p, C.c_int64, C.c_longlong, C.c_int]
         L.pf_surrogate_param_count.restype = st
         L.pf_surrogate_param_count.argtypes = [C.POINTER(C.c_int64)]
         L.pf_surrogate_workspace.restype = st
@@ -193,7 +195,8 @@ def exported_symbols():
             "pf_adjoint", "pf_implicit_adjoint_workspace", "pf_implicit_adjoint",
             "pf_create_ensemble", "pf_set_ensemble_params", "pf_set_ensemble_schedule",
             "pf_tune_ensemble",
-            "pf_step_ensemble", "pf_barrier_selftest", "pf_surrogate_param_count",
+            "pf_step_ensemble", "pf_barrier_selftest", "pf_wait_selftest",
+            "pf_surrogate_param_count",
             "pf_surrogate_workspace", "pf_surrogate_predict", "pf_surrogate_train_step",
             "pf_surrogate_loss_grad",
             "pf_conv3d_check", "pf_energy", "pf_elastic_workspace", "pf_elastic_apply",
@@ -315,6 +318,11 @@ def pf_step_ensemble(ctx, state_ptr, n_steps, mode):
 def pf_barrier_selftest(scratch_ptr, limit_cycles, phantom, stream):
     return lib().pf_barrier_selftest(C.c_void_p(scratch_ptr), int(limit_cycles), int(phantom),
                                      C.c_void_p(stream))
+
+
+def pf_wait_selftest(ctx, state_ptr, n_steps, limit_cycles, implicit):
+    return lib().pf_wait_selftest(ctx, C.c_void_p(state_ptr), int(n_steps), int(limit_cycles),
+                                  int(implicit))
 
 
 def pf_surrogate_param_count():

@@ -55,6 +55,7 @@ struct Scalars {
   float coef[kMaxBasis];
   double hk[kMaxBasis], rel;
   int stop, failed;
+  unsigned mute;  // 0, or flips the tags of this block's packets (self-test)
 };
 
 // Ends a phase: k sums of sc.part over all blocks into sc.sums; a barrier for
@@ -83,10 +84,11 @@ __device__ __noinline__ bool end_phase(Scalars& sc, uint4* packets, unsigned tag
     }
     if (lane == 0) {
       const unsigned long long w = __double_as_longlong((double)v.hi + (double)v.lo);
+      const unsigned sent = tag ^ sc.mute;
       if (ordered) __threadfence();
       asm volatile("st.relaxed.gpu.global.v4.b32 [%0], {%1, %2, %3, %4};" ::"l"(
                        p + (size_t)j * gridDim.x + blockIdx.x),
-                   "r"((unsigned)w), "r"(tag), "r"((unsigned)(w >> 32)), "r"(tag)
+                   "r"((unsigned)w), "r"(sent), "r"((unsigned)(w >> 32)), "r"(sent)
                    : "memory");
     }
   }
@@ -146,6 +148,7 @@ __global__ void __launch_bounds__(kThreads) k_newton2d(const Newton2DArgs a) {
   float* const g = a.g;
   float* const d = a.d;
   unsigned phase = 0;
+  if (threadIdx.x == 0) sc.mute = (int)blockIdx.x < a.mute ? 0x80000000u : 0u;
 
   // f(node, x, y) for this thread's nodes, tile by tile; the first tile's node
   // (the only one on small meshes) is worked out once

@@ -34,8 +34,9 @@
 // so no fence and no separate flag lengthen the path.  Two slots alternate: a
 // block writes slot x+2 only after reading its neighbours' exchange x+1, which
 // they publish after reading x.  Tags start from a zeroed buffer in every
-// launch.  Every wait is bounded; when one runs out the error flag is set, all
-// blocks leave and write NaN over their tiles.
+// launch.  Every wait is bounded; when one runs out the error flag is set,
+// and the blocks that wait, or come to, leave and write NaN over their tiles (one
+// that has all its packets by then stores what it has: the flag is the report).
 #include <algorithm>
 #include <functional>
 #include <queue>
@@ -569,9 +570,10 @@ bool onchip_plan(bool ch, size_t bytes, OnchipJob* job) {
   return best >= 0;
 }
 
-cudaError_t launch_onchip(bool ch, const OnchipArgs& a, bool iso, bool odd, cudaStream_t s) {
+cudaError_t launch_onchip(bool ch, const OnchipArgs& a, bool iso, bool odd, int absent,
+                          cudaStream_t s) {
   const size_t smem = smem_of(ch, kMeshForm, a.job);
-  const int grid = a.job.gx * a.job.gy;
+  const int grid = a.job.gx * a.job.gy - absent;
   return ch ? launch<true, kMeshForm, false>(a, iso, odd, grid, smem, s)
             : launch<false, kMeshForm, false>(a, iso, odd, grid, smem, s);
 }

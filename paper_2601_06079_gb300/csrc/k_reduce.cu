@@ -79,7 +79,7 @@ __global__ void __launch_bounds__(kThreads) k_energy2d(const Energy2DArgs a, dou
 }
 
 __global__ void __launch_bounds__(kThreads) k_sum_partials(const double* partials, int nblocks,
-                                                           double* result) {
+                                                           const unsigned* err, double* result) {
   double e = 0.0, m = 0.0;
   for (int b = threadIdx.x; b < nblocks; b += kThreads) {
     e += partials[2 * b];
@@ -89,6 +89,7 @@ __global__ void __launch_bounds__(kThreads) k_sum_partials(const double* partial
   if (threadIdx.x == 0) {
     result[0] = e;
     result[1] = m;
+    if (err) result[2] = *err ? 1.0 : 0.0;
   }
 }
 
@@ -104,7 +105,7 @@ cudaError_t launch_energy2d(const Energy2DArgs& a, double* partials, double* res
                             cudaStream_t s) {
   const int nb = energy2d_blocks(a.nx, a.ny);
   k_energy2d<<<nb, kThreads, 0, s>>>(a, partials);
-  k_sum_partials<<<1, kThreads, 0, s>>>(partials, nb, result);
+  k_sum_partials<<<1, kThreads, 0, s>>>(partials, nb, a.err, result);
   return cudaGetLastError();
 }
 
@@ -242,7 +243,7 @@ extern "C" pf_status pf_sq_distance(const float* a, const float* b, int64_t n,
   const int nb = (int)(want < pf::kMaxBlocks ? want : pf::kMaxBlocks);
   double* result = dev_scratch + 2 * pf::kMaxBlocks;
   pf::k_sq_distance<<<nb, pf::kThreads, 0, s>>>(a, b, n, dev_scratch);
-  pf::k_sum_partials<<<1, pf::kThreads, 0, s>>>(dev_scratch, nb, result);
+  pf::k_sum_partials<<<1, pf::kThreads, 0, s>>>(dev_scratch, nb, nullptr, result);
   double host = 0.0;
   if (cudaGetLastError() != cudaSuccess ||
       cudaMemcpyAsync(&host, result, sizeof(double), cudaMemcpyDeviceToHost, s) != cudaSuccess ||

@@ -41,6 +41,7 @@ struct pf_ctx {
   // explicit trajectories held on chip
   pf::OnchipJob oc{};
   bool oc_fits = false;
+  bool oc_flag = false;  // buf_a holds the error flag of the last trajectory
 
   // derived coefficients
   pf::Explicit2DArgs ex{};
@@ -770,6 +771,7 @@ pf_status pf_bind_workspace(pf_ctx* c, void* dev_ptr, size_t bytes) {
     c->buf_a = (float*)(c->ws + L.a);
     c->buf_b = (float*)(c->ws + L.b);
   }
+  c->oc_flag = false;
   c->u = c->un = c->g = c->d = c->basis = nullptr;
   if (has_implicit(c)) {
     char* v = c->ws + L.vecs;
@@ -943,8 +945,9 @@ pf_status step_plain2d(pf_ctx* c, float* state, int64_t n_steps) {
 }
 
 // The whole trajectory in one launch, the state on chip; the working planes'
-// memory holds the exchange buffer.
-pf_status step_onchip(pf_ctx* c, float* state, int n_steps) {
+// memory holds the exchange buffer and the error flag, which pf_energy reports
+// (not of a captured call, whose launch is yet to come).
+pf_status step_onchip(pf_ctx* c, float* state, int n_steps, long long limit, int absent) {
   const bool ch = c->model == PF_MODEL_CH;
   pf::OnchipArgs a{};
   a.state = state;
@@ -954,13 +957,16 @@ pf_status step_onchip(pf_ctx* c, float* state, int n_steps) {
   char* buf = (char*)c->buf_a;
   a.err = (unsigned*)buf;
   a.xchg = buf + kOnchipErr;
-  a.limit = kWaitCycles;
+  a.limit = limit;
   a.n_steps = n_steps;
   const size_t bytes = pf::onchip_exchange_bytes(ch, c->oc);
   if (bytes) PF_CUDA(cudaMemsetAsync(buf, 0, kOnchipErr + bytes, c->stream));
   const auto iso = [](const pf::Stencil2D& k) { return k.cx == k.cd && k.cy == k.cd; };
   PF_CUDA(pf::launch_onchip(ch, a, iso(c->ex.k1) && (!ch || iso(c->ex.k2)),
-                            c->ex.odd != 0, c->stream));
+                            c->ex.odd != 0, absent, c->stream));
+  cudaStreamCaptureStatus capture;
+  PF_CUDA(cudaStreamIsCapturing(c->stream, &capture));
+  c->oc_flag = bytes && capture == cudaStreamCaptureStatusNone;
   return PF_OK;
 }
 
@@ -972,12 +978,13 @@ pf_status pf_step_explicit(pf_ctx* c, float* state, int64_t n_steps) {
   if (n_steps < 0) return fail(c, PF_ERR_ARG, "n_steps < 0");
   if (n_steps == 0) return PF_OK;
   if (c->dim == 3) return step_explicit3d(c, state, n_steps);
+  c->oc_flag = false;
   if (c->model == PF_MODEL_COUPLED) return step_coupled2d(c, state, n_steps);
   if (c->par.mobility_field) return step_explicit_mob(c, state, n_steps);
   if (c->form == PF_FORM_TWO_PASS) return step_plain2d(c, state, n_steps);
   if (c->form == PF_FORM_FUSED_GRAPH && c->oc_fits && n_steps >= onchip_steps(nodes2d(c)) &&
       n_steps <= INT32_MAX)
-    return step_onchip(c, state, (int)n_steps);
+    return step_onchip(c, state, (int)n_steps, kWaitCycles, 0);
   const float shift = (float)c->par.shift;
   const int nx = (int)c->n[0], ny = (int)c->n[1];
   // working copies with the mirror frame: d = u - shift (both planes fully defined)
@@ -1022,12 +1029,15 @@ pf_status pf_energy(pf_ctx* c, const float* state, double* energy, double* mass)
   a.q3 = (float)(-2 * W);
   a.q4 = (float)W;
   a.kappa = (float)c->par.kappa;
+  a.err = c->oc_flag ? (const unsigned*)c->buf_a : nullptr;
   PF_CUDA(pf::launch_energy2d(a, c->partials, c->result, c->stream));
-  double host[2];
+  double host[3];
   PF_CUDA(cudaMemcpyAsync(host, c->result, sizeof(host), cudaMemcpyDeviceToHost, c->stream));
   PF_CUDA(cudaStreamSynchronize(c->stream));
   if (energy) *energy = host[0];
   if (mass) *mass = host[1];
+  if (a.err && host[2] != 0.0)
+    return fail(c, PF_ERR_TIMEOUT, "a tile's wait expired in the last explicit run");
   if (!isfinite(host[0]) || !isfinite(host[1]))
     return fail(c, PF_ERR_NONFINITE, "non-finite energy or mass (unstable time step?)");
   return PF_OK;
@@ -1055,7 +1065,8 @@ bool one_launch2d(const pf_ctx* c) {
 
 // n_steps steps by k_newton2d, in launches of at most 64 steps.
 pf_status step_newton2d(pf_ctx* c, float* state, int64_t n_steps, const float* guess,
-                        const pf_newton_opts& o, double atol_factor, pf_newton_stats* s) {
+                        const pf_newton_opts& o, double atol_factor, long long limit, int mute,
+                        pf_newton_stats* s) {
   pf::Newton2DArgs a{};
   a.op = c->im2;
   a.state = state;
@@ -1068,7 +1079,8 @@ pf_status step_newton2d(pf_ctx* c, float* state, int64_t n_steps, const float* g
   a.packets = (uint4*)c->partials;
   const size_t packet_bytes = pf::newton2d_packet_bytes(a.op.nx, a.op.ny);
   a.result = c->small;
-  a.limit = kWaitCycles;
+  a.limit = limit;
+  a.mute = mute;
   a.max_newton = o.max_newton;
   a.restart = o.gmres_restart;
   a.maxit = o.gmres_max_iters;
@@ -1126,7 +1138,7 @@ pf_status pf_step_implicit(pf_ctx* c, float* state, int64_t n_steps, const float
   const int64_t n_state = split_ch(c) ? nnodes(c) : n;  // CH: the state is c alone
   if (c->dim == 2 && one_launch2d(c)) {
     st = step_newton2d(c, state, n_steps, guess, o,
-                       kNoOversolve / std::sqrt(c->h[0] * c->h[1] * c->h[2]), &s);
+                       kNoOversolve / std::sqrt(c->h[0] * c->h[1] * c->h[2]), kWaitCycles, 0, &s);
     // as in the loop below, statistics are reported unless the solve broke off
     if (stats && (st == PF_OK || st == PF_ERR_NOT_CONVERGED)) *stats = s;
     return st;
@@ -1188,6 +1200,32 @@ pf_status pf_step_implicit(pf_ctx* c, float* state, int64_t n_steps, const float
   PF_CUDA(cudaStreamSynchronize(c->stream));
   if (stats) *stats = s;
   return PF_OK;
+}
+
+pf_status pf_wait_selftest(pf_ctx* c, float* state, int64_t n_steps, long long limit_cycles,
+                           int implicit) {
+  if (!c) return PF_ERR_ARG;
+  pf_status st = check_ready(c);
+  if (st != PF_OK) return st;
+  if (!state || n_steps < 8 || n_steps > INT32_MAX || limit_cycles < 1)
+    return fail(c, PF_ERR_ARG, "need a state, n_steps >= 8 and limit_cycles >= 1");
+  if (c->ens_count > 0 || c->dim != 2 || c->model == PF_MODEL_COUPLED || c->par.mobility_field)
+    return fail(c, PF_ERR_ARG, "needs a 2-D AC / CH mesh without a mobility field");
+  if (implicit) {
+    if ((st = need_implicit_ws(c)) != PF_OK) return st;
+    if (!one_launch2d(c) || pf::newton2d_blocks((int)c->n[0], (int)c->n[1]) < 2)
+      return fail(c, PF_ERR_ARG, "the mesh has no implicit form with blocks that wait");
+    pf_newton_stats s{};
+    return step_newton2d(c, state, n_steps, nullptr, pf_newton_opts{20, 30, 300, 1e-5, 1e-3}, 0.0,
+                         limit_cycles, 1, &s);
+  }
+  if (!c->oc_fits || c->oc.gx * c->oc.gy < 2)
+    return fail(c, PF_ERR_ARG, "the mesh has no on-chip form with blocks that wait");
+  if ((st = step_onchip(c, state, (int)n_steps, limit_cycles, 1)) != PF_OK) return st;
+  unsigned flag = 0;
+  PF_CUDA(cudaMemcpyAsync(&flag, c->buf_a, sizeof(flag), cudaMemcpyDeviceToHost, c->stream));
+  PF_CUDA(cudaStreamSynchronize(c->stream));
+  return flag ? fail(c, PF_ERR_TIMEOUT, "a tile's wait expired") : PF_OK;
 }
 
 pf_status pf_create_ensemble(pf_ctx** out, int count, const int64_t* nx, const int64_t* ny,
@@ -1610,6 +1648,7 @@ pf_status pf_adjoint(pf_ctx* c, const float* state0, const float* target, int64_
     return fail(c, PF_ERR_ARG, "the adjoint needs a 2-D Cahn-Hilliard mesh");
   if (!state0 || !target || !adj_ws) return fail(c, PF_ERR_ARG, "null array");
   if (n_steps < 1 || ckpt_every < 1) return fail(c, PF_ERR_ARG, "n_steps and ckpt_every must be >= 1");
+  c->oc_flag = false;  // the forward pass runs through buf_a
   const AdjLayout L = adj_layout(c, n_steps, ckpt_every);
   if (adj_bytes < L.total || (uintptr_t)adj_ws % 256)
     return fail(c, PF_ERR_ARG, "adjoint workspace too small or misaligned (%zu < %zu)", adj_bytes,

@@ -184,7 +184,9 @@ struct OnchipArgs {
 // mesh does not fit.
 bool onchip_plan(bool ch, size_t bytes, OnchipJob* job);
 size_t onchip_exchange_bytes(bool ch, const OnchipJob& b);
-cudaError_t launch_onchip(bool ch, const OnchipArgs& a, bool iso, bool odd, cudaStream_t s);
+// absent: blocks left out, for whose tiles the others wait in vain (self-test)
+cudaError_t launch_onchip(bool ch, const OnchipArgs& a, bool iso, bool odd, int absent,
+                          cudaStream_t s);
 // Tile grids, per-block lists, exchange bytes and shared memory for Allen-Cahn
 // instances (sizes set in jobs); false if one does not fit.
 bool onchip_plan_ensemble(std::vector<OnchipJob>& jobs, std::vector<int>* first,
@@ -200,6 +202,7 @@ struct Energy2DArgs {
   float shift;
   float q0, q1, q2, q3, q4;  // f(shift + d) = q0 + d (q1 + d (q2 + d (q3 + d q4)))
   float kappa;
+  const unsigned* err;  // null, or an error flag: 1.0 in result[2] if it is set
 };
 int energy2d_blocks(int nx, int ny);
 cudaError_t launch_energy2d(const Energy2DArgs& a, double* partials, double* result,
@@ -296,6 +299,7 @@ struct Newton2DArgs {
   double* result;       // status, Newton and GMRES iterations, initial and final residual,
                         // last tolerance, steps done
   long long limit;      // SM cycles of a wait
+  int mute;             // the first blocks, whose packets nobody accepts (self-test)
   int n_steps, max_newton, restart, maxit;
   double newton_rtol, gmres_rtol, atol_factor, inv_dt;
 };
