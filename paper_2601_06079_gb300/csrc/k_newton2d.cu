@@ -9,8 +9,8 @@
 // phases that end in a reduction:
 //   w = J v on the own tiles, products with the basis;
 //   first update and second products;  second update and norm.
-// A partial sum travels as two words with the phase's number beside each
-// (16 bytes); every block polls all blocks' packets, so a reduction is one
+// A partial sum travels as a packet of two words under the phase's number
+// (packet.h); every block polls all blocks' packets, so a reduction is one
 // store and one load through L2, and a barrier where the writer fences first
 // and the reader after (needed only before the operator reads a halo).  Every
 // block sums the partials in the same order, so all take the same decisions, and thread 0 of each runs the (FP64) Givens
@@ -24,6 +24,7 @@
 #include <type_traits>
 
 #include "implicit2d_op.h"
+#include "packet.h"
 #include "pf_internal.h"
 
 namespace pf {
@@ -62,10 +63,10 @@ struct Scalars {
 // memory too if `ordered`.  Packets alternate between two buffers: a block
 // writes phase p + 2 only after it has all of phase p + 1, which the others
 // wrote after reading phase p.
-__device__ __noinline__ bool end_phase(Scalars& sc, uint4* packets, unsigned tag, int k,
+__device__ __noinline__ bool end_phase(Scalars& sc, Packet* packets, unsigned tag, int k,
                                        bool ordered, long long limit) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  uint4* const p = packets + (size_t)(tag & 1) * kMaxBasis * gridDim.x;
+  Packet* const p = packets + (size_t)(tag & 1) * kMaxBasis * gridDim.x;
   const int kk = k > 0 ? k : 1;  // without sums: an empty packet
   if (threadIdx.x == 0) sc.failed = 0;
   __syncthreads();
@@ -84,32 +85,25 @@ __device__ __noinline__ bool end_phase(Scalars& sc, uint4* packets, unsigned tag
     }
     if (lane == 0) {
       const unsigned long long w = __double_as_longlong((double)v.hi + (double)v.lo);
-      const unsigned sent = tag ^ sc.mute;
       if (ordered) __threadfence();
-      asm volatile("st.relaxed.gpu.global.v4.b32 [%0], {%1, %2, %3, %4};" ::"l"(
-                       p + (size_t)j * gridDim.x + blockIdx.x),
-                   "r"((unsigned)w), "r"(sent), "r"((unsigned)(w >> 32)), "r"(sent)
-                   : "memory");
+      publish(p + (size_t)j * gridDim.x + blockIdx.x, (unsigned)w, (unsigned)(w >> 32),
+              tag ^ sc.mute);
     }
   }
   for (int j = warp; j < kk; j += kWarps) {
     double v = 0.0;
     // kPoll packets of a lane on the way together
     for (int b0 = lane; b0 < (int)gridDim.x; b0 += 32 * kPoll) {
-      uint4 q[kPoll];
+      Packet q[kPoll];
       long long began = 0;
       for (int spin = 1;; ++spin) {
         bool all = true;
 #pragma unroll
         for (int i = 0; i < kPoll; ++i)
-          if (b0 + 32 * i < (int)gridDim.x)
-            asm volatile("ld.relaxed.gpu.global.v4.b32 {%0, %1, %2, %3}, [%4];"
-                         : "=r"(q[i].x), "=r"(q[i].y), "=r"(q[i].z), "=r"(q[i].w)
-                         : "l"(p + (size_t)j * gridDim.x + b0 + 32 * i)
-                         : "memory");
+          if (b0 + 32 * i < (int)gridDim.x) q[i] = look(p + (size_t)j * gridDim.x + b0 + 32 * i);
 #pragma unroll
         for (int i = 0; i < kPoll; ++i)
-          if (b0 + 32 * i < (int)gridDim.x) all = all && q[i].y == tag && q[i].w == tag;
+          if (b0 + 32 * i < (int)gridDim.x) all = all && arrived(q[i], tag);
         if (all) break;
         if (spin % 256 == 0) {
           const long long now = clock64();
@@ -123,7 +117,8 @@ __device__ __noinline__ bool end_phase(Scalars& sc, uint4* packets, unsigned tag
 #pragma unroll
       for (int i = 0; i < kPoll; ++i)
         if (b0 + 32 * i < (int)gridDim.x)
-          v += __longlong_as_double((long long)(((unsigned long long)q[i].z << 32) | q[i].x));
+          v += __longlong_as_double(
+              (long long)((unsigned long long)value_of(q[i].b) << 32 | value_of(q[i].a)));
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
@@ -185,7 +180,7 @@ __global__ void __launch_bounds__(kThreads) k_newton2d(const Newton2DArgs a) {
     }
   };
   const auto reduce = [&](int k, bool ordered) {
-    return end_phase(sc, a.packets, ++phase, k, ordered, a.limit);
+    return end_phase(sc, static_cast<Packet*>(a.packets), ++phase, k, ordered, a.limit);
   };
   const auto apply = [&](auto jvp, const float* U, const float* W, auto&& put) {
     Implicit2DArgs op = a.op;
@@ -439,7 +434,7 @@ int newton2d_blocks(int nx, int ny) {
 }
 
 size_t newton2d_packet_bytes(int nx, int ny) {
-  return sizeof(uint4) * 2 * kMaxBasis * (size_t)newton2d_blocks(nx, ny);
+  return sizeof(Packet) * 2 * kMaxBasis * (size_t)newton2d_blocks(nx, ny);
 }
 
 cudaError_t launch_newton2d(const Newton2DArgs& a, cudaStream_t s) {

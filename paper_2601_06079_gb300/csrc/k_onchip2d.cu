@@ -29,9 +29,8 @@
 // column is refreshed after every step; it takes the share that lane 0 needs of
 // the elements left of the strip from a column pass before the sweep.
 //
-// An edge travels as 16-byte packets {value, tag, value, tag}, the tag being
-// the exchange's number: a reader polls the packet itself until both tags match,
-// so no fence and no separate flag lengthen the path.  Two slots alternate: a
+// An edge travels as packets of two values (packet.h), the tag being the
+// exchange's number: a reader polls the packet itself until both tags match.  Two slots alternate: a
 // block writes slot x+2 only after reading its neighbours' exchange x+1, which
 // they publish after reading x.  Tags start from a zeroed buffer in every
 // launch.  Every wait is bounded; when one runs out the error flag is set,
@@ -42,6 +41,7 @@
 #include <queue>
 #include <type_traits>
 
+#include "packet.h"
 #include "pf_internal.h"
 #include "sweep2d.h"
 
@@ -89,19 +89,6 @@ __host__ __device__ inline int tallest(const OnchipJob& b) { return (b.ny + b.gy
 template <class G>
 __host__ __device__ inline int slot_packets(int hmax) {
   return 2 * G::kRows * G::kPairs + G::kEdge * hmax;
-}
-
-struct alignas(16) Packet {
-  float a;
-  unsigned ta;
-  float b;
-  unsigned tb;
-};
-
-__device__ __forceinline__ void publish(Packet* p, float a, float b, unsigned tag) {
-  asm volatile("st.relaxed.gpu.global.v4.b32 [%0], {%1, %2, %3, %4};" ::"l"(p),
-               "r"(__float_as_uint(a)), "r"(tag), "r"(__float_as_uint(b)), "r"(tag)
-               : "memory");
 }
 
 __device__ __forceinline__ int reflect(int k, int n) {
@@ -370,7 +357,7 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocks)
       for (int i = threadIdx.x; i < nsend; i += kThreads) {
         const Send q = send[i];
         const u64 v = *reinterpret_cast<const u64*>(store + q.cell);
-        publish(out + q.packet, plo(v), phi(v), tag);
+        publish(out + q.packet, __float_as_uint(plo(v)), __float_as_uint(phi(v)), tag);
       }
       const Packet* const in = region + (tag & 1) * slot;
       // kBatch polls of a thread are in flight together
@@ -392,19 +379,15 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocks)
         }
         long long began = 0;
         for (int spin = 1;; ++spin) {
-          uint4 v[kBatch];
+          Packet v[kBatch];
           bool more = false;
 #pragma unroll
           for (int k = 0; k < kBatch; ++k)
-            if (wait[k])
-              asm volatile("ld.relaxed.gpu.global.v4.b32 {%0, %1, %2, %3}, [%4];"
-                           : "=r"(v[k].x), "=r"(v[k].y), "=r"(v[k].z), "=r"(v[k].w)
-                           : "l"(in + f[k].src)
-                           : "memory");
+            if (wait[k]) v[k] = look(in + f[k].src);
 #pragma unroll
           for (int k = 0; k < kBatch; ++k) {
             if (!wait[k]) continue;
-            if (v[k].y != tag || v[k].w != tag) {
+            if (!arrived(v[k], tag)) {
               more = true;
               continue;
             }
@@ -412,9 +395,10 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocks)
             float* d = store + (f[k].dst & 0xffffu);
             const unsigned kind = f[k].dst >> 16;
             if (kind == kPair)
-              *reinterpret_cast<u64*>(d) = pk(__uint_as_float(v[k].x), __uint_as_float(v[k].z));
+              *reinterpret_cast<u64*>(d) =
+                  pk(__uint_as_float(value_of(v[k].a)), __uint_as_float(value_of(v[k].b)));
             else
-              d[0] = __uint_as_float(kind == kFirst ? v[k].x : v[k].z);
+              d[0] = __uint_as_float(value_of(kind == kFirst ? v[k].a : v[k].b));
           }
           if (!more) break;
           if (spin % 256 == 0) {

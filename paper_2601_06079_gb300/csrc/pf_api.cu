@@ -1076,7 +1076,7 @@ pf_status step_newton2d(pf_ctx* c, float* state, int64_t n_steps, const float* g
   a.d = c->d;
   a.V = c->basis;
   a.ldv = c->ldv;
-  a.packets = (uint4*)c->partials;
+  a.packets = c->partials;
   const size_t packet_bytes = pf::newton2d_packet_bytes(a.op.nx, a.op.ny);
   a.result = c->small;
   a.limit = limit;

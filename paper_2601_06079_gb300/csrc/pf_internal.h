@@ -295,7 +295,7 @@ struct Newton2DArgs {
   const float* guess;   // first iterate of the first step, or null
   float *u, *un, *g, *d, *V;  // vectors of nx ny values per plane, V: restart + 1 of them
   int64_t ldv;
-  uint4* packets;       // newton2d_packet_bytes(), zeroed
+  void* packets;        // newton2d_packet_bytes(), zeroed
   double* result;       // status, Newton and GMRES iterations, initial and final residual,
                         // last tolerance, steps done
   long long limit;      // SM cycles of a wait
