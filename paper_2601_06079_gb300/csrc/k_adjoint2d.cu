@@ -252,7 +252,7 @@ __global__ void __launch_bounds__(kWarps * 32) k_ch_mob_step(const ChMobArgs a, 
   const int y0 = (block_row() * kWarps + (threadIdx.x >> 5)) * kTYFwd;
   if (y0 >= ny) return;
   const Lane L(nx);
-  const u64 rho = bc(kGLo / kGHi);
+  const u64 rho = bc(kRho);
   u64 nc[kAhead], nm[kAhead];
   const auto load = [&](int j, int k) {  // row y0 - 2 + k into slot j
     const int64_t row = (int64_t)reflect(y0 - 2 + k, ny) * nx;
@@ -329,7 +329,7 @@ __global__ void __launch_bounds__(kWarps * 32)
   const int y0 = band * kTYRev;
   if (y0 >= ny) return;
   const Lane L(nx);
-  const u64 rho = bc(kGLo / kGHi), gX = bc(a.gX), gY = bc(a.gY);
+  const u64 rho = bc(kRho), gX = bc(a.gX), gY = bc(a.gY);
   const u64 s0 = bc(a.h[0]), s1 = bc(a.h[1]), s2 = bc(a.h[2]);
   const Stencil K(a.k);
   u64 nc[kAhead], nm[kAhead], nyv[kAhead];
@@ -586,7 +586,7 @@ int ch_mob_warps(int nx, int ny) { return strips(nx) * ((ny + kTYRev - 1) / kTYR
 void pack_ch_mob(const ChMobParams& p, ChMobArgs& a, ChMobScale& sc) {
   // a value at a Gauss point is g2 times the one carried, and so is the weight
   // back; the Gauss weight is |cell|/4 over the interior mass |cell|
-  const double g = 1.0 / (1.0 + (double)(kGLo / kGHi)), g2 = g * g, cF = 0.25 * g2 * g2;
+  const double g = kGRho, g2 = g * g, cF = 0.25 * g2 * g2;
   double s = 1.0 / g2;
   for (int i = 0; i < 4; ++i, s *= g2) {
     a.q[i] = (float)(s * p.f1[i]);

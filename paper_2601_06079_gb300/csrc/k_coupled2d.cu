@@ -234,9 +234,9 @@ void pack_coupled2d(const CoupledPoly& f, double neg_dt_meta, Coupled2DArgs& a) 
   };
   // a value at a Gauss point is g2 times the one carried, and so is the weight
   // back; the Gauss weight is |cell|/4 over the interior mass |cell|
-  const double g2 = (double)kGHi * kGHi, wt = 0.25 * g2;
+  const double g2 = kGRho * kGRho, wt = 0.25 * g2;
   double s = 1.0;
-  a.pair[0] = two((double)kGLo / kGHi);
+  a.pair[0] = two(kRho);
   a.pair[1] = two(-g2);
   for (int i = 0; i < 5; ++i, s *= g2) {
     const double dfa = i < 4 ? (i + 1) * f.fa[i + 1] : 0.0;

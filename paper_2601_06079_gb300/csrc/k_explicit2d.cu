@@ -409,30 +409,38 @@ cudaError_t launch_ch2d(const Explicit2DArgs& a, cudaStream_t s) {
   }
 }
 
-void pack_explicit2d(Explicit2DArgs& a) {
+void pack_explicit2d(const double (&f)[4], Explicit2DArgs& a) {
   auto pk_host = [](float v) {
     unsigned int b;
     memcpy(&b, &v, 4);
     return (unsigned long long)b | ((unsigned long long)b << 32);
   };
+  a.p0 = (float)f[0];
+  a.p1 = (float)f[1];
+  a.p2 = (float)f[2];
+  a.p3 = (float)f[3];
   // interpolated values lack a factor g_hi^2 and so do the weights back, so
   // p_i carries g_hi^(2 i + 2); the polynomial is odd about the double well's
-  // centre (p0 = p2 = 0), and its form p3 (v^2 + p1/p3) v needs p3 != 0
-  const double g2 = (double)kGHi * kGHi;
-  const double p[4] = {a.p0 * g2, a.p1 * g2 * g2, a.p2 * g2 * g2 * g2, a.p3 * g2 * g2 * g2 * g2};
-  a.odd = a.p0 == 0.0f && a.p2 == 0.0f && a.p3 != 0.0f && std::isfinite(p[1] / p[3]);
-  a.pair[0] = pk_host((float)((double)kGLo / kGHi));
-  a.pair[1] = pk_host(a.odd ? (float)(p[1] / p[3]) : 0.0f);
+  // centre (p0 = p2 = 0), and its form p3 (v^2 + p1/p3) v needs p3 != 0.  Every
+  // coefficient is rounded once, p1/p3 so that its product with the rounded p3,
+  // the slope at the centre, is
+  const double g2 = kGRho * kGRho;
+  double p[4], s = g2;
+  for (int i = 0; i < 4; ++i, s *= g2) p[i] = f[i] * s;
+  const float ratio = (float)(p[1] / (double)(float)p[3]);
+  a.odd = a.p0 == 0.0f && a.p2 == 0.0f && a.p3 != 0.0f && std::isfinite(ratio);
+  a.pair[0] = pk_host(kRho);
+  a.pair[1] = pk_host(a.odd ? ratio : 0.0f);
   a.pair[2] = pk_host((float)p[3]);
   for (int i = 0; i < 4; ++i) a.pair[3 + i] = pk_host((float)p[i]);
   const Stencil2D* st[2] = {&a.k1, &a.k2};
-  for (int s = 0; s < 2; ++s) {
-    a.pair[7 + 6 * s + 0] = pk_host(st[s]->c0 - st[s]->cd);
-    a.pair[7 + 6 * s + 1] = pk_host(st[s]->cd);
-    a.pair[7 + 6 * s + 2] = pk_host(st[s]->c0);
-    a.pair[7 + 6 * s + 3] = pk_host(st[s]->cx);
-    a.pair[7 + 6 * s + 4] = pk_host(st[s]->cy);
-    a.pair[7 + 6 * s + 5] = pk_host(st[s]->cd);
+  for (int k = 0; k < 2; ++k) {
+    a.pair[7 + 6 * k + 0] = pk_host(st[k]->c0 - st[k]->cd);
+    a.pair[7 + 6 * k + 1] = pk_host(st[k]->cd);
+    a.pair[7 + 6 * k + 2] = pk_host(st[k]->c0);
+    a.pair[7 + 6 * k + 3] = pk_host(st[k]->cx);
+    a.pair[7 + 6 * k + 4] = pk_host(st[k]->cy);
+    a.pair[7 + 6 * k + 5] = pk_host(st[k]->cd);
   }
 }
 

@@ -898,19 +898,13 @@ pf_status pf_set_params(pf_ctx* c, const pf_params* p) {
   pf::Explicit2DArgs& a = c->ex;
   a.nx = (int)c->n[0];
   a.ny = (int)c->n[1];
+  double poly = 0.25;  // factor of f' in the kernel's polynomial
   if (c->model == PF_MODEL_AC) {
     const double f = -p->dt * p->mobility;
-    a.p0 = (float)(f * fp[0] / 4);
-    a.p1 = (float)(f * fp[1] / 4);
-    a.p2 = (float)(f * fp[2] / 4);
-    a.p3 = (float)(f * fp[3] / 4);
+    poly = f / 4;
     a.k1 = stiffness2d(hx, hy, f * p->kappa / m);
     a.k2 = stiffness2d(hx, hy, 0.0);
   } else {
-    a.p0 = (float)(fp[0] / 4);
-    a.p1 = (float)(fp[1] / 4);
-    a.p2 = (float)(fp[2] / 4);
-    a.p3 = (float)(fp[3] / 4);
     a.k1 = stiffness2d(hx, hy, p->kappa / m);
     a.k2 = stiffness2d(hx, hy, -p->dt * p->mobility / m);
     pf::ChMobArgs& b = c->mob;
@@ -922,7 +916,7 @@ pf_status pf_set_params(pf_ctx* c, const pf_params* p) {
     for (int i = 0; i < 3; ++i) q.f2[i] = (i + 1) * fp[i + 1];  // f'' about s: the derivative of f'
     pf::pack_ch_mob(q, b, c->mob_scale);
   }
-  pf::pack_explicit2d(a);
+  pf::pack_explicit2d({poly * fp[0], poly * fp[1], poly * fp[2], poly * fp[3]}, a);
   destroy_graph(c);
   return PF_OK;
 }
@@ -1303,14 +1297,10 @@ pf_status pf_set_ensemble_params(pf_ctx* c, const pf_params* p) {
     const double s = q.shift, W = q.W, hx = c->ens_hx[i], hy = c->ens_hy[i], m = hx * hy;
     const double fp[4] = {W * (2 * s - 6 * s * s + 4 * s * s * s), W * (2 - 12 * s + 12 * s * s),
                           W * (-12 + 24 * s) / 2, 4 * W};
-    const double f = -q.dt * q.mobility;
-    a.p0 = (float)(f * fp[0] / 4);
-    a.p1 = (float)(f * fp[1] / 4);
-    a.p2 = (float)(f * fp[2] / 4);
-    a.p3 = (float)(f * fp[3] / 4);
+    const double f = -q.dt * q.mobility, g = f / 4;
     a.k1 = stiffness2d(hx, hy, f * q.kappa / m);
     a.k2 = stiffness2d(hx, hy, 0.0);
-    pf::pack_explicit2d(a);
+    pf::pack_explicit2d({g * fp[0], g * fp[1], g * fp[2], g * fp[3]}, a);
     if (!(a.k1.cx == a.k1.cd && a.k1.cy == a.k1.cd)) c->ens_iso = false;
     if (!a.odd) c->ens_odd = false;
   }

@@ -16,6 +16,11 @@ namespace pf {
 // g_lo = N_0 at the upper point = N_1 at the lower point, and vice versa.
 constexpr float kGHi = 0.78867513459481288225f;
 constexpr float kGLo = 0.21132486540518711775f;
+// Sweeps that carry values at Gauss points without their factor weigh with 1 and
+// kRho; the factor that belongs to the rounded kRho makes the weights sum to one,
+// so that an interpolated constant is exact (kGHi itself is 5.6e-9 off).
+constexpr float kRho = kGLo / kGHi;
+constexpr double kGRho = 1.0 / (1.0 + (double)kRho);
 
 // 2-D launches put rows of blocks on grid.y, which holds at most 65,535; a
 // taller mesh (up to 2^20 node rows) continues on grid.z.  block_row() is the
@@ -97,7 +102,8 @@ struct Explicit2DArgs {
   // ignore it
   int l2;
 };
-void pack_explicit2d(Explicit2DArgs& a);
+// p0..p3 and pair, from f (p0..p3 in FP64) and the stencils
+void pack_explicit2d(const double (&f)[4], Explicit2DArgs& a);
 constexpr int kL2Normal = 0;      // evict_normal
 constexpr int kL2Stream = 1;      // evict_first: the lines go first when L2 needs room
 constexpr int kL2StreamHalf = 2;  // evict_first for half of the lines, the rest unchanged
