@@ -367,7 +367,9 @@ __global__ void __launch_bounds__(kCgThreads) k_cg_r(float* __restrict__ r,
   }
   __syncthreads();
   const float alpha = sh;
-  // four runs of at most a few dozen squares per thread; blocks sum in FP64
+  // four FP32 runs per thread, of n / (4,096 SMs) squares each (11 at 129^3, 6,500
+  // at the largest mesh allowed, half of a run with x beside r); the warps' sums
+  // add up in FP64
   float4 q = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
   const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, nth = (int64_t)gridDim.x * blockDim.x;
   constexpr int kU = 4;

@@ -431,13 +431,21 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocks)
 // one pair, 16 warps, halo 4: 9.0 / 2.6 / 0.95; two pairs, halo 4: 9.2 / 3.7 /
 // 1.4, halo 8: 9.4 / 3.7 / 1.9; an exchange every step: 9.8 / 3.4 / 1.6; 24 or
 // 32 warps spill (10.2 and 13 at 2048^2).  The step kernel replayed from a
-// graph takes 10.0 / 3.7 / 2.7 (12.4 / 4.0 / 5.5 before this arithmetic).  At
-// 2048^2 a step is 14,300 cycles of sweeps, 500 before them and 2,800 of
-// exchange; the sweeps keep the FMA pipe 70 % busy.
+// graph takes 10.0 / 3.7 / 2.7 (12.4 / 4.0 / 5.5 before this arithmetic).
+// Cycles of a step (clock64 at the barriers, 1,000 steps): 2048^2 14,400 of
+// sweeps, 630 before them and 2,800 of exchange; 515 x 1031 2,770, 630 and 1,500;
+// Allen-Cahn 64^2 540, 260 and 770.
 // Ensembles: two blocks per SM work on different instances, so one's exchange
 // runs under the other's sweeps, and exact strips lose no column at the widths
 // of 128: 51 us per step of 256 instances (31.7 M nodes), against 60 to 70 for
-// forms with halo lanes, 97 for one launch per step and 109 before.
+// forms with halo lanes, 97 for one launch per step and 109 before.  At other
+// widths strips of 128 columns leave lanes idle, and still: 256 square instances,
+// us for 200 steps on chip / one launch per step, tuned (the band sweep in one
+// launch is within 9 % of that): side 128 1,330 / 4,560, 130 2,840 / 4,560, 150 3,170 /
+// 4,980, 190 4,560 / 7,790, 200 4,810 / 8,290, 300 10,820 / 14,540, 350 12,350 /
+// 19,910, 500 37,350 / 38,140.  The sweep is level on many tiny instances (5,000
+// of 16^2, 120 steps: 3,740 / 3,020, before 3,820) and strips of 8 columns (20 of
+// 3000 x 8: 1,870 / 1,800, before 2,140).
 struct Form {
   int kp, warps, blocks, halo;
 };
