@@ -46,7 +46,7 @@
 // Measured at 512^2 (us per step, graph replay): forward 5.7 with 32 x 16 node
 // tiles in shared memory (element passes into corner arrays, four barriers), 2.9
 // so; reverse 13.6, 7.1 so.  Both are latency-bound there (8 warps per SM); the
-// reverse sweep holds 164 registers.
+// reverse sweep holds 162 registers.
 #include "pf_internal.h"
 #include "sweep2d.h"
 
