@@ -562,6 +562,29 @@ bool onchip_plan(bool ch, size_t bytes, OnchipJob* job) {
   return best >= 0;
 }
 
+// us: a step of the band sweep replayed from a graph (fixed, per million nodes) and
+// of the on-chip form (fixed, per 100 rows of a tile), by sweep_variant.  A step on
+// chip takes what its tile's height does, however many SMs have a tile: 600 x 4300
+// makes 77 tiles of 600 rows and takes 10.3 us (Cahn-Hilliard, square cells) where
+// the sweep takes 7.1 (8.2 before this form), 1000 x 3000 108 tiles, 8.6 and 7.9,
+// 2048^2 148 tiles, 8.9 and 10.4, 300 x 8000 143 tiles, 5.7 and 6.9.  Fitted to 26
+// meshes of 64^2 to 3000^2 nodes, each within 0.3 us.
+struct Rate {
+  double band0, band1, chip0, chip1;
+};
+constexpr Rate kRates[2][3] = {
+    {{2.25, 1.33, 0.75, 1.14}, {2.3, 1.34, 0.75, 1.2}, {2.35, 1.53, 0.8, 1.38}},  // Allen-Cahn
+    {{2.45, 1.87, 1.5, 1.45}, {2.4, 1.93, 1.5, 1.56}, {2.5, 2.14, 1.6, 1.74}}};
+
+bool onchip_pays(bool ch, bool iso, bool odd, const OnchipJob& b, int64_t steps, bool graph) {
+  const Rate& r = kRates[ch][sweep_variant(iso, odd)];
+  const double nodes = 1e-6 * b.nx * b.ny, h = 0.01 * tallest(b);
+  // a sweep launched by itself takes up to 2 us more; a call's tiles, tables and
+  // conversions
+  const double band = r.band0 + r.band1 * nodes + (graph ? 0.0 : 2.0), chip = r.chip0 + r.chip1 * h;
+  return 13.0 + 18.0 * h + chip * steps <= 13.5 + 4.0 * nodes + band * steps;
+}
+
 cudaError_t launch_onchip(bool ch, const OnchipArgs& a, bool iso, bool odd, int absent,
                           cudaStream_t s) {
   const size_t smem = smem_of(ch, kMeshForm, a.job);

@@ -103,7 +103,7 @@ constexpr int kGraphSteps = 64;  // even, so a replay returns to buf_a
 // and 100 us at 2048^2 (the tiles are 16 times as tall), which the steps have to
 // win back against one launch each: 8 steps take 21 against 67 us (Allen-Cahn,
 // 64^2), 47 against 67 (Cahn-Hilliard, 515 x 1031), 173 against 135 (2048^2;
-// 32 steps: 383 against 431).
+// 32 steps: 383 against 431).  For a single mesh, onchip_pays weighs the steps too.
 int64_t onchip_steps(int64_t nodes) { return 8 + (nodes >> 18); }
 constexpr size_t kOnchipErr = 256;  // error flag in front of the exchange buffer
 constexpr long long kWaitCycles = 2000000000LL;  // about one second
@@ -283,6 +283,15 @@ cudaError_t launch_step(pf_ctx* c, const float* in, float* out, bool dependent, 
   a.out = out;
   a.pitch = pf::work_pitch((int)c->n[0]);
   return c->model == PF_MODEL_CH ? pf::launch_ch2d(a, s) : pf::launch_ac2d(a, s);
+}
+
+// Whether the context's stream is being captured: a graph cannot be launched into
+// a capture, so there the steps themselves are.
+pf_status in_capture(pf_ctx* c, bool* yes) {
+  cudaStreamCaptureStatus s;
+  PF_CUDA(cudaStreamIsCapturing(c->stream, &s));
+  *yes = s != cudaStreamCaptureStatusNone;
+  return PF_OK;
 }
 
 pf_status ensure_graph(pf_ctx* c) {
@@ -826,10 +835,8 @@ pf_status step_coupled2d(pf_ctx* c, float* state, int64_t n_steps) {
   const float shift = (float)c->par.shift;
   PF_CUDA(pf::launch_to_work(state, c->buf_a, c->buf_b, nx, ny, 2, shift, c->stream));
   int64_t left = n_steps;
-  // a graph cannot be launched into a capture: there, the steps themselves are
-  cudaStreamCaptureStatus capture;
-  PF_CUDA(cudaStreamIsCapturing(c->stream, &capture));
-  const bool captured = capture != cudaStreamCaptureStatusNone;
+  bool captured = false;
+  if (pf_status st = in_capture(c, &captured)) return st;
   if (left >= kGraphSteps && !captured) {
     pf_status st = ensure_graph(c);
     if (st != PF_OK) return st;
@@ -938,6 +945,12 @@ pf_status step_plain2d(pf_ctx* c, float* state, int64_t n_steps) {
   return PF_OK;
 }
 
+// the explicit step's stencils are those of square cells
+bool square_cells(const pf_ctx* c) {
+  const auto iso = [](const pf::Stencil2D& k) { return k.cx == k.cd && k.cy == k.cd; };
+  return iso(c->ex.k1) && (c->model != PF_MODEL_CH || iso(c->ex.k2));
+}
+
 // The whole trajectory in one launch, the state on chip; the working planes'
 // memory holds the exchange buffer and the error flag, which pf_energy reports
 // (not of a captured call, whose launch is yet to come).
@@ -955,12 +968,10 @@ pf_status step_onchip(pf_ctx* c, float* state, int n_steps, long long limit, int
   a.n_steps = n_steps;
   const size_t bytes = pf::onchip_exchange_bytes(ch, c->oc);
   if (bytes) PF_CUDA(cudaMemsetAsync(buf, 0, kOnchipErr + bytes, c->stream));
-  const auto iso = [](const pf::Stencil2D& k) { return k.cx == k.cd && k.cy == k.cd; };
-  PF_CUDA(pf::launch_onchip(ch, a, iso(c->ex.k1) && (!ch || iso(c->ex.k2)),
-                            c->ex.odd != 0, absent, c->stream));
-  cudaStreamCaptureStatus capture;
-  PF_CUDA(cudaStreamIsCapturing(c->stream, &capture));
-  c->oc_flag = bytes && capture == cudaStreamCaptureStatusNone;
+  PF_CUDA(pf::launch_onchip(ch, a, square_cells(c), c->ex.odd != 0, absent, c->stream));
+  bool captured = false;
+  if (pf_status st = in_capture(c, &captured)) return st;
+  c->oc_flag = bytes && !captured;
   return PF_OK;
 }
 
@@ -977,14 +988,18 @@ pf_status pf_step_explicit(pf_ctx* c, float* state, int64_t n_steps) {
   if (c->par.mobility_field) return step_explicit_mob(c, state, n_steps);
   if (c->form == PF_FORM_TWO_PASS) return step_plain2d(c, state, n_steps);
   if (c->form == PF_FORM_FUSED_GRAPH && c->oc_fits && n_steps >= onchip_steps(nodes2d(c)) &&
-      n_steps <= INT32_MAX)
+      n_steps <= INT32_MAX &&
+      pf::onchip_pays(c->model == PF_MODEL_CH, square_cells(c), c->ex.odd != 0, c->oc, n_steps,
+                      n_steps >= kGraphSteps))
     return step_onchip(c, state, (int)n_steps, kWaitCycles, 0);
   const float shift = (float)c->par.shift;
   const int nx = (int)c->n[0], ny = (int)c->n[1];
   // working copies with the mirror frame: d = u - shift (both planes fully defined)
   PF_CUDA(pf::launch_to_work(state, c->buf_a, c->buf_b, nx, ny, 1, shift, c->stream));
   int64_t left = n_steps;
-  if (left >= kGraphSteps && c->form == PF_FORM_FUSED_GRAPH) {
+  bool captured = false;
+  if (pf_status st = in_capture(c, &captured)) return st;
+  if (left >= kGraphSteps && c->form == PF_FORM_FUSED_GRAPH && !captured) {
     pf_status st = ensure_graph(c);
     if (st != PF_OK) return st;
     for (; left >= kGraphSteps; left -= kGraphSteps) PF_CUDA(cudaGraphLaunch(c->graph, c->stream));

@@ -190,6 +190,9 @@ struct OnchipArgs {
 // mesh does not fit.
 bool onchip_plan(bool ch, size_t bytes, OnchipJob* job);
 size_t onchip_exchange_bytes(bool ch, const OnchipJob& b);
+// Whether a call of `steps` steps takes less time on chip than as band sweeps
+// (graph: replayed from a graph).
+bool onchip_pays(bool ch, bool iso, bool odd, const OnchipJob& b, int64_t steps, bool graph);
 // absent: blocks left out, for whose tiles the others wait in vain (self-test)
 cudaError_t launch_onchip(bool ch, const OnchipArgs& a, bool iso, bool odd, int absent,
                           cudaStream_t s);

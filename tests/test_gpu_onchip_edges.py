@@ -56,3 +56,21 @@ def test_tile_edges(model, shape):
         stream.synchronize()
         steps_form.step_explicit(b, steps)
         assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("model", ["ac", "ch"])
+@pytest.mark.parametrize("shape,on_chip", [((600, 4300), False), ((1000, 3000), False),
+                                           ((300, 8000), True), ((3000, 1000), True)])
+def test_wide_meshes(model, shape, on_chip):
+    # tiles of 56 columns and few of them down the mesh: 77 and 108 tall tiles take
+    # longer than the band sweep, 143 and 144 low ones do not
+    u0 = torch.from_numpy(G.ch_initial(12, shape)).cuda()
+    stream = torch.cuda.Stream()
+    s = solver(model, shape, "fused_graph", stream)
+    assert (enqueued(s, stream, u0.clone(), 100) <= 2) == on_chip
+    a, b = u0.clone(), u0.clone()
+    torch.cuda.synchronize()
+    s.step_explicit(a, 100)
+    stream.synchronize()
+    solver(model, shape, "fused_stream").step_explicit(b, 100)
+    assert torch.equal(a, b)
