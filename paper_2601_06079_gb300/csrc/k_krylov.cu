@@ -39,12 +39,14 @@ __device__ __forceinline__ double warp_sum(double v) {
 // The reductions' last stages.  warp_value: the warp's sum of accumulator j
 // into shared memory (no block barrier per vector); then finish_sums: the
 // block's sums into partials[j * blocks + b], and the last block to finish adds
-// all blocks' partials into out[j], a warp per vector, in a fixed order (blocks
-// in steps of 32 per lane, then a tree), so one launch gives the final,
-// repeatable values.  count: device counter, 0 before the launch and reset to
-// 0 by the last block.  (With two barriers per vector and block, and the last
-// block taking the vectors one after another, 8 products of 4,096 values took
-// 16.5 us, nearly all of it here; now 4.)
+// all blocks' partials into out[j], its 8 warps shared out among up to 4 vectors
+// (more have a warp each, in turn), in a fixed order (blocks in steps of
+// 32 lanes times the vector's warps, a tree, then the warps), so one launch gives
+// the final, repeatable values.  count: device counter, 0 before the launch and
+// reset to 0 by the last block.  (With two barriers per vector and block, and the
+// last block taking the vectors one after another, 8 products of 4,096 values took
+// 16.5 us, nearly all of it here; now 4.  A single sum of 456 partials by one warp cost
+// 0.9 us more: k_update of 10^6 values 10.3 us, so 9.4.)
 constexpr int kWarpsPerBlock = kThreads / 32;
 
 __device__ __forceinline__ void warp_value(Acc2 a, int j, double (*sums)[kWarpsPerBlock]) {
@@ -56,6 +58,14 @@ __device__ __forceinline__ void warp_value(Acc2 a, int j, double (*sums)[kWarpsP
     a.lo += l;
   }
   if ((threadIdx.x & 31) == 0) sums[j][threadIdx.x >> 5] = a.value();
+}
+
+// a warp's share (part of kShare) of the blocks' partials, in its lane 0
+template <int kShare>
+__device__ __forceinline__ double partial_sum(const double* p, int blocks, int part, int lane) {
+  double v = 0.0;
+  for (int b = 32 * part + lane; b < blocks; b += 32 * kShare) v += __ldcg(p + b);
+  return warp_sum(v);
 }
 
 __device__ void finish_sums(double (*sums)[kWarpsPerBlock], double* partials, int k,
@@ -79,11 +89,26 @@ __device__ void finish_sums(double (*sums)[kWarpsPerBlock], double* partials, in
   __syncthreads();
   if (!last) return;
   __threadfence();
-  for (int j = w; j < k; j += kWarpsPerBlock) {
-    double v = 0.0;
-    for (int b = l; b < blocks; b += 32) v += __ldcg(partials + (int64_t)j * blocks + b);
-    v = warp_sum(v);
-    if (l == 0) out[j] = v;
+  if (k > 4) {  // a warp per vector
+    for (int j = w; j < k; j += kWarpsPerBlock) {
+      const double v = partial_sum<1>(partials + (int64_t)j * blocks, blocks, 0, l);
+      if (l == 0) out[j] = v;
+    }
+  } else {
+    const int share = k == 1 ? 8 : (k == 2 ? 4 : 2), j = w / share;
+    if (j < k) {
+      const double* p = partials + (int64_t)j * blocks;
+      const double v = share == 8   ? partial_sum<8>(p, blocks, w % 8, l)
+                       : share == 4 ? partial_sum<4>(p, blocks, w % 4, l)
+                                    : partial_sum<2>(p, blocks, w % 2, l);
+      if (l == 0) sums[j][w % share] = v;
+    }
+    __syncthreads();
+    if (threadIdx.x < k) {
+      double v = sums[threadIdx.x][0];
+      for (int i = 1; i < share; ++i) v += sums[threadIdx.x][i];
+      out[threadIdx.x] = v;
+    }
   }
   if (threadIdx.x == 0) *count = 0;
 }
@@ -287,19 +312,29 @@ __global__ void k_axpby(float a, const float* __restrict__ x, float b, float* __
 }
 
 // x <- x / sqrt(*norm2) unless it is 0: a vector is normalised by the sum its
-// reduction left on the device, before the host has read it
+// reduction left on the device, before the host has read it.  One thread of a
+// block takes the FP64 root and reciprocal while the first values are on their
+// way; in every thread they took most of the launch (10^6 values: 10.5 us, so
+// 4.4).
 template <bool kVec>
 __global__ void k_normalise(float* x, const double* __restrict__ norm2, int64_t n) {
-  const double s = *norm2;
-  if (!(s > 0.0)) return;
-  const float a = (float)(1.0 / sqrt(s));
-  for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; 4 * c < n;
-       c += (int64_t)gridDim.x * blockDim.x) {
-    float v[4];
-    load4<kVec>(x, 4 * c, n, v);
+  __shared__ float scale;
+  int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  float v[4];
+  load4<kVec>(x, 4 * c, n, v);  // past the end: zeros
+  if (threadIdx.x == 0) {
+    const double s = *norm2;
+    scale = s > 0.0 ? (float)(1.0 / sqrt(s)) : -1.0f;
+  }
+  __syncthreads();
+  const float a = scale;
+  if (a < 0.0f) return;
+  while (4 * c < n) {
 #pragma unroll
     for (int t = 0; t < 4; ++t) v[t] *= a;
     store4<kVec>(x, 4 * c, n, v);
+    c += (int64_t)gridDim.x * blockDim.x;
+    load4<kVec>(x, 4 * c, n, v);
   }
 }
 
