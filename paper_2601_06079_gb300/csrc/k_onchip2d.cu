@@ -519,15 +519,16 @@ cudaError_t launch(const OnchipArgs& a, bool iso, bool odd, int grid, size_t sme
   return cudaLaunchKernelEx(&cfg, k, a);
 }
 
-// the tile grid of a mesh for tiles at most hcap rows tall; false if it has none
-bool tile_grid(bool ch, int form, int hcap, OnchipJob* b) {
+// the tile grid of a mesh for tiles at most hcap rows tall on `blocks` blocks; false
+// if it has none
+bool tile_grid(bool ch, int form, int blocks, int hcap, OnchipJob* b) {
   const Form& f = kForms[form];
   const int np = (b->nx + 1) / 2, half = cols_of(ch, form) / 2;
   b->gx = (np + half - 1) / half;
   b->gy = (b->ny + hcap - 1) / hcap;
   if (b->gy > 1 && b->ny / b->gy < f.halo + 1) return false;  // rows that a neighbour needs
   if (b->gx > 1 && np / b->gx < 3) return false;
-  return (int64_t)b->gx * b->gy <= blocks_of(form) &&
+  return (int64_t)b->gx * b->gy <= blocks &&
          (f.halo > 1 || (tallest(*b) + f.warps - 1) / f.warps <= kMaxBand) &&
          smem_of(ch, form, *b) <= smem_cap(form);
 }
@@ -549,8 +550,9 @@ bool onchip_plan(bool ch, size_t bytes, OnchipJob* job) {
   double best = -1.0;
   OnchipJob pick = *job, b = *job;
   const int half = cols_of(ch, kMeshForm) / 2, gx = ((b.nx + 1) / 2 + half - 1) / half;
-  for (int gy = 1; gx * gy <= blocks_of(kMeshForm) && gy <= b.ny; ++gy) {
-    if (!tile_grid(ch, kMeshForm, (b.ny + gy - 1) / gy, &b) || b.gy != gy) continue;
+  const int blocks = blocks_of(kMeshForm);
+  for (int gy = 1; gx * gy <= blocks && gy <= b.ny; ++gy) {
+    if (!tile_grid(ch, kMeshForm, blocks, (b.ny + gy - 1) / gy, &b) || b.gy != gy) continue;
     if (onchip_exchange_bytes(ch, b) > bytes) continue;
     const double c = tile_cycles(ch, kMeshForm, tallest(b), gx * gy == 1);
     if (best < 0 || c < best) {
@@ -603,16 +605,23 @@ bool onchip_plan_ensemble(std::vector<OnchipJob>& jobs, std::vector<int>* first,
   const int blocks = blocks_of(kEnsForm);
   double best = -1.0;
   std::vector<OnchipJob> best_jobs;
-  std::vector<std::vector<OnchipItem>> best_lists;
+  std::vector<std::pair<int, OnchipItem>> placed, best_placed;  // (block, item) in order
   std::vector<int> heights = {384, 320, 256, 192, 128, 96, 64, 32, 16};
   if (jobs.size() > 4096) heights = {192};  // as many jobs as blocks many times over
+  std::vector<OnchipJob> js = jobs;
+  std::vector<int> scheduled;
+  std::vector<double> cost(js.size());
+  std::vector<int> order(js.size());
   for (int hcap : heights) {
-    std::vector<OnchipJob> js = jobs;
+    // the next lower cap often gives the grids that were scheduled last
+    std::vector<int> rows(js.size());
     bool ok = true;
-    for (size_t i = 0; i < js.size() && ok; ++i) ok = tile_grid(false, kEnsForm, hcap, &js[i]);
-    if (!ok) continue;
-    std::vector<double> cost(js.size());
-    std::vector<int> order(js.size());
+    for (size_t i = 0; i < js.size() && ok; ++i) {
+      ok = tile_grid(false, kEnsForm, blocks, hcap, &js[i]);
+      rows[i] = js[i].gy;
+    }
+    if (!ok || rows == scheduled) continue;
+    scheduled.swap(rows);
     for (size_t i = 0; i < js.size(); ++i) {
       cost[i] = tile_cycles(false, kEnsForm, tallest(js[i]), js[i].gx * js[i].gy == 1);
       order[i] = (int)i;
@@ -622,9 +631,11 @@ bool onchip_plan_ensemble(std::vector<OnchipJob>& jobs, std::vector<int>* first,
       return gx != gy ? gx > gy : cost[x] > cost[y];
     });
     typedef std::pair<double, int> Free;  // (time a block is free, block)
-    std::priority_queue<Free, std::vector<Free>, std::greater<Free>> q;
-    for (int b = 0; b < blocks; ++b) q.push(Free(0.0, b));
-    std::vector<std::vector<OnchipItem>> lists(blocks);
+    std::vector<Free> idle(blocks);
+    for (int b = 0; b < blocks; ++b) idle[b] = Free(0.0, b);
+    std::priority_queue<Free, std::vector<Free>, std::greater<Free>> q(std::greater<Free>(),
+                                                                       std::move(idle));
+    placed.clear();
     double end = 0.0;
     std::vector<int> gang;
     for (int j : order) {
@@ -637,7 +648,7 @@ bool onchip_plan_ensemble(std::vector<OnchipJob>& jobs, std::vector<int>* first,
         q.pop();
       }
       for (int t = 0; t < g; ++t) {
-        lists[gang[t]].push_back(OnchipItem{j, t});
+        placed.emplace_back(gang[t], OnchipItem{j, t});
         q.push(Free(start + cost[j], gang[t]));
       }
       end = std::max(end, start + cost[j]);
@@ -645,18 +656,18 @@ bool onchip_plan_ensemble(std::vector<OnchipJob>& jobs, std::vector<int>* first,
     if (best < 0 || end < best) {
       best = end;
       best_jobs = js;
-      best_lists = lists;
+      best_placed.swap(placed);
     }
   }
   if (best < 0) return false;
   jobs = best_jobs;
-  first->clear();
-  list->clear();
-  for (const auto& l : best_lists) {
-    first->push_back((int)list->size());
-    list->insert(list->end(), l.begin(), l.end());
-  }
-  first->push_back((int)list->size());
+  // the blocks' lists one after another, each in the order of placing
+  first->assign(blocks + 1, 0);
+  for (const auto& p : best_placed) ++(*first)[p.first + 1];
+  for (int b = 0; b < blocks; ++b) (*first)[b + 1] += (*first)[b];
+  std::vector<int> next(first->begin(), first->end() - 1);
+  list->resize(best_placed.size());
+  for (const auto& p : best_placed) (*list)[next[p.first]++] = p.second;
   *exchange = 0;
   *smem = 0;
   for (OnchipJob& b : jobs) {

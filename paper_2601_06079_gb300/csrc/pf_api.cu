@@ -1447,15 +1447,18 @@ pf_status pf_tune_ensemble(pf_ctx* c, int reps, int* ty_out, int* l2_out, double
       for (int j = 0; j < kEnsCands; ++j) us_out[kEnsCands * ci + j] = j == bj ? best : -1.0;
   // 2. coordinate descent over the classes, most nodes first (the classes
   // that fill L2 the most are the first to try streaming): a class keeps
-  // another candidate only if the whole step gets at least 1 % faster
+  // another candidate only if the whole step gets at least 1 % faster.  It ends
+  // when every class in turn has kept its own since the last change.
   std::vector<int> order(nc);
   for (int ci = 0; ci < nc; ++ci) order[ci] = ci;
   std::stable_sort(order.begin(), order.end(), [&](int x, int y) {
     return classes[x].first * classes[x].second > classes[y].first * classes[y].second;
   });
-  for (int pass = 0; pass < 3 && st == PF_OK; ++pass) {
-    bool changed = false;
+  int kept = 0;
+  for (int pass = 0; pass < 3 && st == PF_OK && kept < nc; ++pass) {
     for (int ci : order) {
+      if (kept == nc) break;
+      bool changed = false;
       for (int j = 0; j < kEnsCands && st == PF_OK; ++j) {
         if (j == assign[ci]) continue;
         std::vector<int> trial = assign;
@@ -1471,8 +1474,8 @@ pf_status pf_tune_ensemble(pf_ctx* c, int reps, int* ty_out, int* l2_out, double
         }
       }
       if (st != PF_OK) break;
+      kept = changed ? 0 : kept + 1;
     }
-    if (!changed) break;
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
