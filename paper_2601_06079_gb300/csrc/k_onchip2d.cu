@@ -552,7 +552,10 @@ bool onchip_plan(bool ch, size_t bytes, OnchipJob* job) {
   const int half = cols_of(ch, kMeshForm) / 2, gx = ((b.nx + 1) / 2 + half - 1) / half;
   const int blocks = blocks_of(kMeshForm);
   for (int gy = 1; gx * gy <= blocks && gy <= b.ny; ++gy) {
-    if (!tile_grid(ch, kMeshForm, blocks, (b.ny + gy - 1) / gy, &b) || b.gy != gy) continue;
+    const int h = (b.ny + gy - 1) / gy;
+    if (gy > 1 && b.ny / gy < kForms[kMeshForm].halo + 1) break;  // nor do more
+    if ((b.ny + h - 1) / h != gy) continue;  // as fewer tiles of this height
+    if (!tile_grid(ch, kMeshForm, blocks, h, &b)) continue;
     if (onchip_exchange_bytes(ch, b) > bytes) continue;
     const double c = tile_cycles(ch, kMeshForm, tallest(b), gx * gy == 1);
     if (best < 0 || c < best) {
