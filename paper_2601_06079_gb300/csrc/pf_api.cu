@@ -1103,8 +1103,11 @@ pf_status step_newton2d(pf_ctx* c, float* state, int64_t n_steps, const float* g
     PF_CUDA(cudaMemsetAsync(a.packets, 0, packet_bytes, c->stream));
     PF_CUDA(cudaMemsetAsync(a.result, 0xff, sizeof(double), c->stream));  // NaN: no result
     PF_CUDA(pf::launch_newton2d(a, c->stream));
-    if (pf_status st = fetch_scalars(c, a.result, 7)) return st;
-    const double* r = c->host_sc;
+    // one read-back a launch: pinned memory would cost a new context more than the
+    // staged copy does (50 us to allocate, 40 to free)
+    double r[7];
+    PF_CUDA(cudaMemcpyAsync(r, a.result, sizeof(r), cudaMemcpyDeviceToHost, c->stream));
+    PF_CUDA(cudaStreamSynchronize(c->stream));
     if (std::isnan(r[0]))
       return fail(c, PF_ERR_TIMEOUT, "a wait between blocks expired in the implicit solver");
     s->newton_iters += (int)r[1];
