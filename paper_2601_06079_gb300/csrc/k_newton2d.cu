@@ -129,8 +129,10 @@ __device__ __noinline__ bool end_phase(Scalars& sc, Packet* packets, unsigned ta
   return !sc.failed;
 }
 
+// One block per SM: without that bound the Allen-Cahn form was held to 64 registers
+// and spilled (six steps at 64^2 1,610 us, so 1,538; two at 1024^2 2,400 and 2,260).
 template <bool kCH>
-__global__ void __launch_bounds__(kThreads) k_newton2d(const Newton2DArgs a) {
+__global__ void __launch_bounds__(kThreads, 1) k_newton2d(const Newton2DArgs a) {
   __shared__ TileMem<kCH> mem;
   __shared__ Scalars sc;
   const int64_t N = (int64_t)a.op.nx * a.op.ny;
