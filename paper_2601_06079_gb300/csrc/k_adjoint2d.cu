@@ -34,19 +34,22 @@
 //   - the polynomials keep their coefficients, the stiffness stencil is divided by
 //     its corner weight (8 and -1 on square cells), and the factors in front of
 //     them meet at the node: r = kappa K : F, the fluxes' and the time step's, each
-//     an FP32 pair hi + lo in two FMAs;
+//     an FP32 pair hi + lo that meets an unrounded product;
 //   - dLoss/dM's sum is not taken: it follows from the other two.
 // dLoss/dM's error against FP64 over 60 meshes of 41 x 70 to 488 x 168 nodes and
 // 100 to 1,000 steps, as a share of (|kappa dLoss/dkappa| + |W dLoss/dW|) / M:
-// median 5.7e-9, largest 2.7e-8 (the rounding of the states); with g_hi of its own
+// median 5.0e-9, largest 2.7e-8 (the rounding of the states); with g_hi of its own
 // and every factor rounded once 3.2e-8 and 1.2e-7; with node tiles, differences and
-// dt as the one rounded factor that mattered 1.1e-8 and 3.3e-8.  512^2 takes the
-// same time with the pairs and without (2,000 steps and their reverse: 25.8 ms).
+// dt as the one rounded factor that mattered 1.1e-8 and 3.3e-8.  The pairs cost the
+// forward step 1 to 2 % (1,024 steps of 512^2 2,994 and 3,061 us); with the warp's
+// running sums asked for at the start and added before the last row, 1,000 steps
+// and their reverse take 12.1 ms without them and 12.4 with, on 300 x 400 10.5 and
+// 10.1.
 //
 // Measured at 512^2 (us per step, graph replay): forward 5.7 with 32 x 16 node
 // tiles in shared memory (element passes into corner arrays, four barriers), 2.9
 // so; reverse 13.6, 7.1 so.  Both are latency-bound there (8 warps per SM); the
-// reverse sweep holds 162 registers.
+// reverse sweep holds 166 registers.
 #include "pf_internal.h"
 #include "sweep2d.h"
 
@@ -238,13 +241,15 @@ struct Lane {
   }
 };
 
-// a v + b u, the factors as pairs hi + lo
-__device__ __forceinline__ u64 scaled(const float (&a)[2], u64 v, const float (&b)[2], u64 u) {
-  return fma2(bc(b[0]), u, fma2(bc(a[0]), v, fma2(bc(b[1]), u, mul2(bc(a[1]), v))));
+// u times a factor hi + lo: the low part meets the unrounded product (added to a
+// rounded sum it would be lost)
+__device__ __forceinline__ u64 times(const float (&f)[2], u64 u) {
+  return fma2(bc(f[0]), u, mul2(bc(f[1]), u));
 }
-// v + r u
-__device__ __forceinline__ u64 with(u64 v, u64 u, const float (&r)[2]) {
-  return fma2(bc(r[0]), u, fma2(bc(r[1]), u, v));
+
+// the sum of two such products, the low parts first
+__device__ __forceinline__ u64 times(const float (&f)[2], u64 u, const float (&g)[2], u64 v) {
+  return fma2(bc(g[0]), v, fma2(bc(f[0]), u, fma2(bc(g[1]), v, mul2(bc(f[1]), u))));
 }
 
 __global__ void __launch_bounds__(kWarps * 32) k_ch_mob_step(const ChMobArgs a, float* out) {
@@ -283,25 +288,25 @@ __global__ void __launch_bounds__(kWarps * 32) k_ch_mob_step(const ChMobArgs a, 
   pot.take<false>(c, a, rho, F, Kc);
   next(2);
   pot.take<true>(c, a, rho, F, Kc);  // mu of row y0 - 1
-  dif.start(row_of(with(F, Kc, a.r)));
+  dif.start(row_of(add2(F, times(a.r, Kc))));
   mob.start(m1);
 #pragma unroll
   for (int k = 3; k < kTYFwd + 4; ++k) {
     next(k);
     pot.take<true>(c, a, rho, F, Kc);  // mu of row y0 - 3 + k
-    dif.take(row_of(with(F, Kc, a.r)), rho, dx, dy);
+    dif.take(row_of(add2(F, times(a.r, Kc))), rho, dx, dy);
     mob.take(m1, rho, mx, my);
     if (k == 3) {
       flux.take<false>(dx, dy, mx, my, rho, ox, oy);
     } else {
       flux.take<true>(dx, dy, mx, my, rho, ox, oy);
       const int y = y0 + k - 4;
-      if (L.writer && y < ny) L.store(out + (int64_t)y * nx, nx, add2(cc[(k - 2) % 3], scaled(a.fx, ox, a.fy, oy)));
+      if (L.writer && y < ny) L.store(out + (int64_t)y * nx, nx, add2(cc[(k - 2) % 3], times(a.fx, ox, a.fy, oy)));
     }
   }
 }
 
-// hi + lo, a sum with the rounding errors of its additions in lo
+// hi + lo, a sum with the rounding errors of its additions in lo (Knuth's two-sum)
 struct Pair {
   float hi, lo;
   __device__ __forceinline__ void add(float x) {
@@ -331,6 +336,9 @@ __global__ void __launch_bounds__(kWarps * 32)
   const Lane L(nx);
   const u64 rho = bc(kRho), gX = bc(a.gX), gY = bc(a.gY);
   const u64 s0 = bc(a.h[0]), s1 = bc(a.h[1]), s2 = bc(a.h[2]);
+  // the warp's two pairs so far, asked for before they are needed
+  float4* const pairs = reinterpret_cast<float4*>(acc) + ((int64_t)band * gridDim.x + blockIdx.x);
+  const float4 kept = (threadIdx.x & 31) == 0 ? *pairs : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
   const Stencil K(a.k);
   u64 nc[kAhead], nm[kAhead], nyv[kAhead];
   const auto load = [&](int j, int k) {
@@ -389,9 +397,9 @@ __global__ void __launch_bounds__(kWarps * 32)
     dy_.take(y, rho, ex, ey);
     mob.take(m, rho, mx, my);
     flux.take<true>(ex, ey, mx, my, rho, ox, oy);
-    const u64 w = with(ox, oy, a.ay);  // without cW
+    const u64 w = add2(ox, times(a.ay, oy));  // without cW
     const Row wr = row_of(w);
-    const u64 mu = with(F, Kc, a.r), vw = beside(wr);
+    const u64 mu = add2(F, times(a.r, Kc)), vw = beside(wr);
     const int yr = y0 - 3 + k;  // the row of mu and w
     if (k >= 3 && k < kTYRev + 3 && yr < ny) {
       const u64 fw = mul2(mul2(fxp, bc(yr == 0 || yr == ny - 1 ? 0.5f : 1.0f)), w);
@@ -416,14 +424,13 @@ __global__ void __launch_bounds__(kWarps * 32)
       if (k >= 4) {
         const int yo = y0 + k - 4;  // the finished row
         const u64 H = back_x(add2(fma2(rho, h[1], h[0]), hl), add2(fma2(rho, h[3], h[2]), hh), rho);
-        const u64 Hw = with(H, K(w2, w1, w, v2, v1, vw), a.r);
+        const u64 Hw = add2(H, times(a.r, K(w2, w1, w, v2, v1, vw)));
         const u64 S = add2(fma2(rho, q1, q0), gx);
         const u64 both = add2(S, pk(from_left(phi(S)), plo(S)));  // elements right and left
         const u64 G = fma2(gY, add2(gy, T), mul2(gX, both));
         if (L.writer && yo < ny) {
           const int64_t row = (int64_t)yo * nx;
-          L.store(yout + row, nx,
-                  fma2(bc(a.n[0]), Hw, fma2(bc(a.n[1]), Hw, yy[(k - 2) % 3])));
+          L.store(yout + row, nx, add2(yy[(k - 2) % 3], times(a.n, Hw)));
           if (grad_hi) {
             const u64 v = mul2(mul2(fxp, bc(yo == 0 || yo == ny - 1 ? 0.5f : 1.0f)), G);
 #pragma unroll
@@ -449,28 +456,25 @@ __global__ void __launch_bounds__(kWarps * 32)
     v1 = vw;
     wa = na;
     wb = nb;
-  }
-  // the warp's sums, into its pairs (Knuth's two-sum; FP64 only at the end: an
-  // FP64 instruction takes an SM 16 cycles per warp)
-  static_assert(kTYRev == 4, "two runs of two rows");
-  Pair v[2] = {runs(dK), runs(dW)};
+    if (k == kTYRev + 2) {
+      // the warp's sums, into its pairs (FP64 only at the end: an FP64 instruction
+      // takes an SM 16 cycles per warp), while the last row is still to do
+      static_assert(kTYRev == 4, "two runs of two rows");
+      Pair v[2] = {runs(dK), runs(dW)};
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
+      for (int o = 16; o > 0; o >>= 1) {
 #pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      const float h = __shfl_down_sync(kFull, v[j].hi, o);
-      v[j].lo += __shfl_down_sync(kFull, v[j].lo, o);
-      v[j].add(h);
-    }
-  }
-  if ((threadIdx.x & 31) == 0) {
-    float2* p = acc + 2 * ((int64_t)band * gridDim.x + blockIdx.x);
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      const float2 q = p[j];
-      v[j].lo += q.y;
-      v[j].add(q.x);
-      p[j] = make_float2(v[j].hi, v[j].lo);
+        for (int j = 0; j < 2; ++j) {
+          const float h = __shfl_down_sync(kFull, v[j].hi, o);
+          v[j].lo += __shfl_down_sync(kFull, v[j].lo, o);
+          v[j].add(h);
+        }
+      }
+      v[0].lo += kept.y;
+      v[0].add(kept.x);
+      v[1].lo += kept.w;
+      v[1].add(kept.z);
+      if ((threadIdx.x & 31) == 0) *pairs = make_float4(v[0].hi, v[0].lo, v[1].hi, v[1].lo);
     }
   }
 }
