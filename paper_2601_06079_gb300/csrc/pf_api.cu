@@ -14,6 +14,8 @@
 
 #include "pf_internal.h"
 
+constexpr int kHostScalars = 2 * pf::kMaxBasis + 1;  // a GMRES column: h1, h2, the norm
+
 struct pf_ctx {
   int dim = 2;
   int64_t n[3] = {1, 1, 1};
@@ -58,6 +60,9 @@ struct pf_ctx {
   int64_t ldv = 0;         // floats between consecutive Krylov vectors
   double* small = nullptr; // h1[32], h2[32], scalars
   double* host_sc = nullptr;  // pinned: reduction results on their way to the host
+  double staged_sc[kHostScalars];        // pageable: the first ones
+  const double* scalars = staged_sc;     // where the last ones are
+  int fetches = 0;
   unsigned* count = nullptr;  // block counter of the single-launch reductions (0 between calls)
   bool count_zeroed = false;  // set once the counter has been cleared after a bind
 
@@ -566,13 +571,18 @@ pf_status clear_count(pf_ctx* c) {
   return PF_OK;
 }
 
-// The first n doubles at p (device) on the host, through pinned memory: a copy
-// to pageable memory is staged and costs several us more per GMRES iteration.
-constexpr int kHostScalars = 2 * pf::kMaxBasis + 1;
+// The first n doubles at p (device) on the host, in c->scalars.  A copy to pageable
+// memory is staged and costs several us more per GMRES iteration than one to
+// pinned memory, which costs a context 30 us to allocate and 200 to free: taken
+// once a context has read back more often than a few steps do.
+constexpr int kStagedFetches = 64;
 pf_status fetch_scalars(pf_ctx* c, const double* p, int n) {
-  if (!c->host_sc) PF_CUDA(cudaHostAlloc((void**)&c->host_sc, sizeof(double) * kHostScalars, 0));
-  PF_CUDA(cudaMemcpyAsync(c->host_sc, p, sizeof(double) * n, cudaMemcpyDeviceToHost, c->stream));
+  if (!c->host_sc && ++c->fetches > kStagedFetches)
+    PF_CUDA(cudaHostAlloc((void**)&c->host_sc, sizeof(double) * kHostScalars, 0));
+  double* const to = c->host_sc ? c->host_sc : c->staged_sc;
+  PF_CUDA(cudaMemcpyAsync(to, p, sizeof(double) * n, cudaMemcpyDeviceToHost, c->stream));
   PF_CUDA(cudaStreamSynchronize(c->stream));
+  c->scalars = to;
   return PF_OK;
 }
 
@@ -582,7 +592,7 @@ pf_status mass_norm(pf_ctx* c, const float* g, double* out) {
                                c->h[0] * c->h[1] * c->h[2], c->partials, c->result, c->count,
                                c->stream));
   if (pf_status st = fetch_scalars(c, c->result, 1)) return st;
-  *out = std::sqrt(c->host_sc[0]);
+  *out = std::sqrt(c->scalars[0]);
   return PF_OK;
 }
 
@@ -615,7 +625,7 @@ pf_status gmres3d(pf_ctx* c, int m, int maxit, double rtol, double atol, int* it
     PF_CUDA(pf::launch_dots(V, ldv, 1, nullptr, n, c->partials, dnrm, c->count, c->stream));
     PF_CUDA(pf::launch_normalise(V, dnrm, n, c->stream));
     if (pf_status st = fetch_scalars(c, dnrm, 1)) return st;
-    const double* host = c->host_sc;
+    const double* host = c->scalars;
     const double beta = std::sqrt(host[0]);
     if (beta0 < 0) beta0 = beta;
     if (beta0 == 0.0) {
@@ -638,6 +648,7 @@ pf_status gmres3d(pf_ctx* c, int m, int maxit, double rtol, double atol, int* it
       PF_CUDA(pf::launch_update(V, ldv, k + 1, dh2, vk1, n, c->partials, dnrm, c->count, c->stream));
       PF_CUDA(pf::launch_normalise(vk1, dnrm, n, c->stream));
       if (pf_status st = fetch_scalars(c, c->small, kHostScalars)) return st;
+      host = c->scalars;
       ++total;
       for (int j = 0; j <= k; ++j) H[(size_t)j * m + k] = host[j] + host[pf::kMaxBasis + j];
       const double hk1 = std::sqrt(std::max(host[2 * pf::kMaxBasis], 0.0));
